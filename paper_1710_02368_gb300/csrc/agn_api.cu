@@ -156,8 +156,9 @@ Status bounds_collect(cudaStream_t st) {
 #endif
 
 struct agn_handle {
-  // problem
-  std::vector<int> dims;
+  // problem: the caller's layer dims and the device's (d_0 .. d_{L-1} padded to
+  // multiples of 8 on the tensor-core path, see create)
+  std::vector<int> udims, dims;
   int L = 0, n = 0, lam = 0;
   double eta = 0.0;
   uint64_t seed = 0;
@@ -189,8 +190,8 @@ struct agn_handle {
   int64_t N = 0, S = 0;
   std::vector<int> tdims;
   int64_t P = 0, P_pad = 0;
+  int C = 0;                  // classes d_L
   std::vector<int64_t> woff, boff, woff_flat, boff_flat;   // per layer (index l-1)
-  int maxd = 0;
   // CUDA
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -217,6 +218,7 @@ struct agn_handle {
                               // 5 output layer as its own kernel
   struct LayerMaps {
     CUtensorMap w_k, w_mn, h_k, h_mn, dz_k, dz_mn;
+    CUtensorMap w_k256;          // split mode: w_k without swizzle, for column tiles of 256
     CUtensorMap theta, acc;      // fp32 W_l of every replica / accumulator, box {128, 32}
     CUtensorMap h_mn32, dz_mn32; // split mode: 32-sample boxes for the dW kernel
   };
@@ -236,6 +238,9 @@ struct agn_handle {
   std::vector<bf16*> dZp;         // pieces of dZ_l, l = 1..L-1: [3][n][m][d_l]
   // output layer fused into one kernel (forward + softmax-CE + dX) when narrow
   bool use_head = false;
+  // a wide output layer (!use_head) on the tensor cores: dims[L] is then its
+  // classes padded to a multiple of 8
+  bool out_tc = false;
   // the output layer's dW runs as tiles of the persistent tensor-core dW
   // launch: dZ_L padded to ldz_out columns (zero beyond d_L) with its pieces,
   // and H_{L-1}'s pieces kept
@@ -250,8 +255,8 @@ struct agn_handle {
   int* fh_counter = nullptr;      // [2][n][ceil(m / 32)]
   int fh_parity = 0;
   // loss_parts holds loss_q values per local step of a commit: the fused
-  // output layer writes one per 32-sample chunk, the other paths the step's
-  // loss in the first and zeros after it
+  // output layer and the softmax kernel write one per 32-sample chunk, the
+  // output head the step's loss in the first and zeros after it
   int loss_q = 1;
   // the gather copies a local step's minibatch before waiting for the
   // preceding kernel: the layer-1 operand the tensor-core kernels read
@@ -410,8 +415,9 @@ void collect_profile(agn_handle* h) {
   h->ev_used = 0;
 }
 
-// Layer l (1-based) runs on the tensor cores: bf16 mode, a hidden layer.
-bool tc_layer(const agn_handle* h, int l) { return h->use_tc && l < h->L; }
+// Layer l (1-based) runs on the tensor cores: a hidden layer, or an output
+// layer too wide for the output-layer kernels.
+bool tc_layer(const agn_handle* h, int l) { return h->use_tc && (l < h->L || h->out_tc); }
 
 agn::TcArgs tc_args(agn_handle* h, const int* sw, const long long* st0, int step) {
   agn::TcArgs t{};
@@ -448,7 +454,7 @@ void next_counters(agn_handle* h, agn::TcArgs* t) {
 // Tensor maps of the tcgen05 path (addresses are fixed for the handle's life).
 Status build_tc_maps(agn_handle* h) {
   const int n = h->n, m = h->m, L = h->L;
-  const uint32_t bn = (uint32_t)agn::tc_bn(m);
+  constexpr uint32_t bn = agn::kTcBoxN;
   h->tmaps.assign(L - 1, {});
   for (int l = 1; l < L; ++l) {
     const uint64_t fi = h->dims[l - 1], fo = h->dims[l];
@@ -466,7 +472,8 @@ Status build_tc_maps(agn_handle* h) {
       const float* W = h->rep + h->woff[l - 1];
       // (with column tiles up to 128 the forward's converters read the tile
       // row by row into tensor memory: 128-byte swizzle, conflict-free)
-      AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, bk, 128, bn <= 128));
+      AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, bk, 128, true));
+      AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k256, W, fi, fo, n, fi, h->P_pad, bk, 128));
       AGN_TRY(agn::make_tmap_f32_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 128, bk));
       const bf16* Hp = h->Hs[l - 1];
       const uint64_t hp = (uint64_t)n * m * fi;
@@ -530,6 +537,25 @@ Status build_tc_maps(agn_handle* h) {
                                   128, 32));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.acc, h->acc + h->woff[L - 1], fi, fo, n, fi, h->P_pad,
                                   128, 32));
+    if (h->out_tc) {   // and its forward and dX
+      if (h->split) {
+        constexpr uint32_t bk = agn::kTcSplitBK;
+        const float* W = h->rep + h->woff[L - 1];
+        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, bk, 128, true));
+        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k256, W, fi, fo, n, fi, h->P_pad, bk, 128));
+        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 128, bk));
+        AGN_TRY(agn::make_tmap_bf16_4d(&mp.h_k, h->Hs[L - 1], fi, m, n, fi, (uint64_t)m * fi,
+                                       (uint64_t)n * m * fi, bk, bn));
+        AGN_TRY(agn::make_tmap_bf16_4d(&mp.dz_k, h->dZp[L], lz, m, n, lz, (uint64_t)m * lz,
+                                       (uint64_t)n * m * lz, bk, bn));
+      } else {
+        const bf16* W = h->rep_b + h->woff[L - 1];
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, 64, 128));
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 64, 64));
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, h->H[L - 1], fi, m, n, fi, (uint64_t)m * fi, 64, bn));
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, h->dZ[L], lz, m, n, lz, (uint64_t)m * lz, 64, bn));
+      }
+    }
     if (h->split) {
       const bf16* Hp = h->Hs[L - 1];
       AGN_TRY(agn::make_tmap_bf16_4d(&mp.h_mn32, Hp, fi, m, n, fi, (uint64_t)m * fi,
@@ -544,13 +570,28 @@ Status build_tc_maps(agn_handle* h) {
   return Status::Ok();
 }
 
-// Split K of a forward or dX GEMM with M rows, N = m columns and K inner
-// over s slots: one CTA per output tile, unless the tiles leave SMs idle
+// Column tile of a forward or dX GEMM with M rows and N = m columns over s
+// slots.  fp32 mode, m > 128: 256 only where the tiles nearly fill the SMs.  A
+// tile of 128 takes A's pieces from tensor memory and gives small waves twice
+// the CTAs; one of 256 converts every weight tile half as often.  Measured, us
+// per local step of 784-1000-1000-10 at m = 256: 1 worker 56.5 (128) / 60.9
+// (256), 4 workers 110.7 / 112.0, 16 workers 394 / 357; 784-4096-4096-10, 4
+// workers, 822 / 721; 64-48-10 at m = 200, 41.1 / 60.5.
+int tc_bn(const agn_handle* h, int M, int s) {
+  const int m = h->m;
+  if (m <= 64) return 64;
+  if (m <= 128) return 128;
+  if (!h->split) return 256;
+  return 4 * ceil_div(M, 128) * ceil_div(m, 256) * (int64_t)s >= 3 * (int64_t)h->num_sms ? 256 : 128;
+}
+
+// Split K of a forward or dX GEMM with M rows, N = m columns in tiles of bn and
+// K inner over s slots: one CTA per output tile, unless the tiles leave SMs idle
 // (small waves); then ks CTAs share each tile, with ks <= SMs / tiles and
 // every CTA's range of 64-deep k steps non-empty.
-int pick_ksplit(const agn_handle* h, int M, int K, int s) {
+int pick_ksplit(const agn_handle* h, int M, int K, int s, int bn) {
   if (h->tc_mask & 16) return 1;
-  const int64_t tiles = ceil_div(M, 128) * ceil_div(h->m, agn::tc_bn(h->m)) * (int64_t)s;
+  const int64_t tiles = ceil_div(M, 128) * ceil_div(h->m, bn) * (int64_t)s;
   if (tiles >= h->num_sms) return 1;
   const int kt = (int)ceil_div(K, 64);
   int ks = (int)std::min<int64_t>(kt, h->num_sms / tiles);
@@ -599,7 +640,9 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // this local step's buffer of layer 1's tensor-core operand
     const bool alt = h->early_gather && h->gparity;
     const agn_handle::LayerMaps& l1 = alt ? h->l1_alt : h->tmaps.empty() ? h->l1_alt : h->tmaps[0];
-    auto maps_of = [&](int l) -> const agn_handle::LayerMaps& { return l == 1 ? l1 : h->tmaps[l - 1]; };
+    auto maps_of = [&](int l) -> const agn_handle::LayerMaps& {
+      return l == 1 ? l1 : l == L ? h->out_maps : h->tmaps[l - 1];
+    };
     if (!h->direct_x) {
       // fp32 mode with the early gather: the fp32 rows are not read by the
       // tensor-core kernels, only their pieces
@@ -620,7 +663,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // launch's CTAs fit the SMs at once
     const bool fuse_head_now =
         h->fuse_head && tc_layer(h, L - 1) &&
-        ceil_div(h->dims[L - 1], 128) * (int64_t)s <= (int64_t)h->num_sms;
+        ceil_div(h->dims[L - 1], 128) * ceil_div(m, tc_bn(h, h->dims[L - 1], s)) * (int64_t)s <=
+            (int64_t)h->num_sms;
     bool head_done = false;
     // forward, l = 1..L
     for (int l = 1; l <= L; ++l) {
@@ -705,11 +749,12 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
           t.no_a_prefetch = l == 1 && (h->tc_mask & 512) ? 1 : 0;
-          t.ksplit = pick_ksplit(h, fo, fi, s);
+          const int bn = tc_bn(h, fo, s);
+          t.ksplit = pick_ksplit(h, fo, fi, s, bn);
           next_counters(h, &t);
           bool launched = false;
-          AGN_TRY(agn::tc_forward_head(mp.w_k, mp.h_k, t, s, h->stream, h->split,
-                                       agn::tc_bn(m), h->num_sms, &launched));
+          AGN_TRY(agn::tc_forward_head(h->split && bn == 256 ? mp.w_k256 : mp.w_k, mp.h_k, t, s,
+                                       h->stream, h->split, bn, h->num_sms, &launched));
           if (!launched) return Status::Err(AGN_E_CUDA, "internal: fused output layer not resident");
           pieces_done = true;
           head_done = true;
@@ -718,15 +763,19 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           agn::TcArgs t = tc_args(h, sw, st0, i);
           t.M = fo; t.N = m; t.K = fi;
           t.a_by_worker = 1;
-          t.out = h->H[l]; t.ldo = fo; t.out_bstride = (int64_t)m * fo;
-          t.relu = 1; t.boff = h->boff[l - 1];
+          t.out = l == L ? static_cast<void*>(h->Z) : h->H[l];
+          t.out_f32 = l == L;
+          t.ldo = fo; t.out_bstride = (int64_t)m * fo;
+          t.relu = l < L; t.boff = h->boff[l - 1];
           t.out_pieces = h_pieces; t.out_plane = (int64_t)n * m * fo;
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
           t.no_a_prefetch = l == 1 && (h->tc_mask & 512) ? 1 : 0;
-          t.ksplit = pick_ksplit(h, fo, fi, s);
+          const int bn = tc_bn(h, fo, s);
+          t.ksplit = pick_ksplit(h, fo, fi, s, bn);
           next_counters(h, &t);
-          AGN_TRY(agn::tc_forward(mp.w_k, mp.h_k, t, s, h->stream, h->split, agn::tc_bn(m)));
+          AGN_TRY(agn::tc_forward(h->split && bn == 256 ? mp.w_k256 : mp.w_k, mp.h_k, t, s,
+                                  h->stream, h->split, bn));
           pieces_done = true;
         } else {
           AGN_TRY(agn::simt_forward<T>(g, l == L, s, h->stream));
@@ -735,14 +784,22 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       if (h_pieces && !pieces_done) AGN_TRY(split_act(h, h->H[l], h_pieces, fo, s, launches));
     }
     if (!h->use_head) {
-      Launch k(h, AGN_K_SOFTMAX, 0.0, (double)s * m * (h->dims[L] * (4.0 + es) + 4.0), launches);
-      AGN_TRY(agn::softmax_xent<T>(h->Z, h->yb, static_cast<T*>(h->dZ[L]), m, h->dims[L],
-                                   h->loss_parts, sc, h->lam, i, h->flag, s, h->stream));
+      agn::SoftmaxArgs a{};
+      a.Z = h->Z; a.m = m; a.C = h->C; a.ld = h->dims[L];
+      a.yb = h->yb; a.slot_worker = sw; a.slot_t0 = st0; a.x_shard = h->direct_x ? h->S : 0;
+      a.dZ = h->dZ[L];
+      a.dZ_pieces = dz_pieces(L); a.dZ_plane = dz_plane(L);
+      a.loss_parts = h->loss_parts; a.slot_commit = sc; a.lam = h->lam; a.step = i;
+      a.flag = h->flag;
+      Launch k(h, AGN_K_SOFTMAX, 0.0,
+               (double)s * m * (h->C * (4.0 + es + (a.dZ_pieces ? 6.0 : 0.0)) + 4.0), launches);
+      AGN_TRY(agn::softmax_xent<T>(a, s, h->stream));
     }
     // backward: dX for l = L..2 (each reads W_l before its update), then the
     // weight and bias gradients with the local step of every layer
     std::vector<char> have_pieces(L + 1, 0);   // pieces of dZ_l written by its producer
     if (L > 1) have_pieces[L - 1] = dz_ready;
+    have_pieces[L] = dz_pieces(L) != nullptr;   // by the softmax kernel
     auto ensure_pieces = [&](int l) -> Status {
       if (dz_pieces(l) && !have_pieces[l]) {
         AGN_TRY(split_act(h, h->dZ[l], dz_pieces(l), h->dims[l], s, launches, dz_plane(l)));
@@ -767,11 +824,11 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         t.out = h->dZ[l - 1]; t.ldo = fi; t.out_bstride = (int64_t)m * fi;
         t.mask = Hprev; t.mask_bstride = (int64_t)m * fi;
         t.out_pieces = next_pieces; t.out_plane = dz_plane(l - 1);
-        const auto& mp = h->tmaps[l - 1];
-        t.ksplit = pick_ksplit(h, fi, fo, s);
+        const auto& mp = maps_of(l);
+        const int bn = tc_bn(h, fi, s);
+        t.ksplit = pick_ksplit(h, fi, fo, s, bn);
         next_counters(h, &t);
-        AGN_TRY(agn::tc_backward_dx(mp.w_mn, mp.dz_k, t, s, h->stream, h->split,
-                                    agn::tc_bn(m)));
+        AGN_TRY(agn::tc_backward_dx(mp.w_mn, mp.dz_k, t, s, h->stream, h->split, bn));
         have_pieces[l - 1] = next_pieces != nullptr;
       } else {
         agn::GemmArgs g{};
@@ -1098,10 +1155,11 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
     AGN_TRY(agn::reduce_losses(h->loss_parts, h->lam, h->loss_q, k, h->loss + V0, h->stream));
   }
   AGN_TRY_CUDA(cudaEventRecord(h->ev1, h->stream));
-  int flags[2] = {0, 0};
-  AGN_TRY_CUDA(cudaMemcpyAsync(flags, h->flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   const double host_ms =
       std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_host0).count();
+  // (this copy to pageable memory waits for the queued work)
+  int flags[2] = {0, 0};
+  AGN_TRY_CUDA(cudaMemcpyAsync(flags, h->flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
   const Status bounds = agn::bounds_collect(h->stream);   // bounds-checked build only
   float ms = 0.f;
@@ -1133,6 +1191,18 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
     return Status::Err(AGN_E_NONFINITE, "a loss or a commit was not finite");
   }
   return bounds;
+}
+
+// Host rows of `width` elements into device rows of `ld` >= width, zero beyond.
+Status upload_rows(void* dst, const void* src, int64_t rows, int64_t width, int64_t ld, size_t es) {
+  if (width == ld) {
+    AGN_TRY_CUDA(cudaMemcpy(dst, src, (size_t)(rows * ld) * es, cudaMemcpyHostToDevice));
+    return Status::Ok();
+  }
+  AGN_TRY_CUDA(cudaMemset(dst, 0, (size_t)(rows * ld) * es));
+  AGN_TRY_CUDA(cudaMemcpy2D(dst, (size_t)ld * es, src, (size_t)width * es, (size_t)width * es,
+                            (size_t)rows, cudaMemcpyHostToDevice));
+  return Status::Ok();
 }
 
 Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_workers, int32_t lambda,
@@ -1172,8 +1242,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   if (o.elide_accumulator && (o.tc_mask & 8))
     return Status::Err(AGN_E_UNSUPPORTED,
                        "the one-tile-per-CTA dW kernel (tc_mask bit 3) keeps the accumulator");
-  h->dims.assign(dims, dims + n_dims);
+  h->udims.assign(dims, dims + n_dims);
   h->L = n_dims - 1;
+  h->C = dims[h->L];
   h->n = n_workers;
   h->lam = lambda;
   h->eta = eta;
@@ -1202,9 +1273,37 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   } else {
     h->tdims = {dims[0], 64, dims[n_dims - 1]};
   }
-  // parameter layouts: flat (the ABI's order) and padded (device, 64-element aligned tensors)
+  // tcgen05 path: a hidden layer and every TMA row 16-byte aligned.  bf16 mode
+  // feeds bf16 operands; fp32 mode feeds each fp32 operand as three exact bf16
+  // pieces (split mode).
+  bool tc_ok = h->m <= 256 && h->L >= 2;
+  for (int l = 0; l < h->L; ++l) tc_ok = tc_ok && dims[l] % 8 == 0;
+  if (o.gemm == AGN_GEMM_TCGEN05 && !tc_ok)
+    return Status::Err(AGN_E_UNSUPPORTED,
+                       "tcgen05 GEMMs need batch <= 256, at least one hidden layer "
+                       "and d_0 .. d_{L-1} multiples of 8");
+  h->use_tc = h->L >= 2 && o.gemm != AGN_GEMM_SIMT;
+  h->split = h->use_tc && h->prec == AGN_PREC_FP32;
+  h->tc_mask = (o.tc_mask & 7) == 0 ? (o.tc_mask | 7) : o.tc_mask;
+  // Device dims.  The tensor-core path pads d_0 .. d_{L-1} to multiples of 8
+  // with inputs, features and weights that are zero and stay zero: a padded
+  // feature's pre-activation and gradient are zero, and so are the gradients
+  // of the weights into and out of it (SGD, Adam and the commits leave a zero
+  // with a zero gradient unchanged).  Every size gains over the CUDA-core
+  // kernels, us per local step of either: 3-5-2 17.0 / 18.4, 37-65-13-7 at 5
+  // workers 30 / 38, 613-301-150-26 (m = 100, 8 workers) 64 / 170,
+  // 784-1000-1000-10 (m = 512, 4 workers) 178 / 888.
+  h->dims = h->udims;
+  if (h->use_tc)
+    for (int l = 0; l < h->L; ++l) h->dims[l] = (int)round_up(dims[l], 8);
+  const int dl1 = h->dims[h->L - 1];
+  h->use_head = h->prec == AGN_PREC_BF16 ? agn::head_fits<bf16>(dl1, h->C)
+                                         : agn::head_fits<float>(dl1, h->C);
+  h->out_tc = h->use_tc && !h->use_head && (h->tc_mask & 7) == 7 && !(h->tc_mask & 8);
+  if (h->out_tc) h->dims[h->L] = (int)round_up(h->C, 8);
+  // parameter layouts: flat (the ABI's order, the caller's dims) and the
+  // device's (the device dims, 64-element aligned tensors)
   int64_t off = 0, offp = 0;
-  h->maxd = 0;
   for (int l = 1; l <= h->L; ++l) {
     const int64_t fi = dims[l - 1], fo = dims[l];
     h->woff_flat.push_back(off);
@@ -1212,25 +1311,12 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     off += fo * fi + fo;
     offp = round_up(offp, 64);
     h->woff.push_back(offp);
-    offp = round_up(offp + fo * fi, 64);
+    offp = round_up(offp + (int64_t)h->dims[l] * h->dims[l - 1], 64);
     h->boff.push_back(offp);
-    offp += fo;
-    h->maxd = std::max<int>(h->maxd, (int)fo);
+    offp += h->dims[l];
   }
   h->P = off;
   h->P_pad = round_up(offp, 64);
-  // tcgen05 path: m <= 256, a hidden layer, every TMA row 16-byte aligned.
-  // bf16 mode feeds bf16 operands; fp32 mode feeds each fp32 operand as three
-  // exact bf16 pieces (split mode).
-  bool tc_ok = h->m <= 256 && h->L >= 2;
-  for (int l = 0; l < h->L; ++l) tc_ok = tc_ok && dims[l] % 8 == 0;
-  if (o.gemm == AGN_GEMM_TCGEN05 && !tc_ok)
-    return Status::Err(AGN_E_UNSUPPORTED,
-                       "tcgen05 GEMMs need batch <= 256, at least one hidden layer "
-                       "and d_0 .. d_{L-1} multiples of 8");
-  h->use_tc = tc_ok && o.gemm != AGN_GEMM_SIMT;
-  h->split = h->use_tc && h->prec == AGN_PREC_FP32;
-  h->tc_mask = (o.tc_mask & 7) == 0 ? (o.tc_mask | 7) : o.tc_mask;
   h->prev.assign(h->n, -1);
   h->pulled_v.assign(h->n, 0);
   h->steps.assign(h->n, 0);
@@ -1247,34 +1333,36 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   AGN_TRY_CUDA(cudaEventCreate(&h->ev1));
 
   // host inputs
-  const int d0 = dims[0];
-  h->hX.resize((size_t)h->N * d0);
+  const int u0 = dims[0];
+  h->hX.resize((size_t)h->N * u0);
   h->hy.resize((size_t)h->N);
   h->htheta0.resize((size_t)h->P);
   if (o.x_init) std::memcpy(h->hX.data(), o.x_init, h->hX.size() * sizeof(float));
-  else agn::gen_dataset(seed, d0, h->N, h->dist, h->hX.data());
+  else agn::gen_dataset(seed, u0, h->N, h->dist, h->hX.data());
   if (o.y_init) {
     std::memcpy(h->hy.data(), o.y_init, h->hy.size() * sizeof(int32_t));
     for (int32_t v : h->hy)
       if (v < 0 || v >= dims[n_dims - 1]) return Status::Err(AGN_E_INVALID, "label out of range");
   } else {
     auto Ws = agn::gen_teacher(seed, h->tdims);
-    agn::gen_teacher_labels(h->hX.data(), h->N, d0, h->dist, h->tdims, Ws, h->hy.data());
+    agn::gen_teacher_labels(h->hX.data(), h->N, u0, h->dist, h->tdims, Ws, h->hy.data());
   }
   if (o.theta_init) std::memcpy(h->htheta0.data(), o.theta_init, h->htheta0.size() * sizeof(float));
-  else agn::gen_init(seed, h->dims, h->htheta0.data());
+  else agn::gen_init(seed, h->udims, h->htheta0.data());
   std::vector<float> hXe;
   std::vector<int32_t> hye;
   if (o.n_eval > 0) {   // held-out rows of the same generator, labelled by the same teacher
     h->n_eval = o.n_eval;
-    hXe.resize((size_t)(o.n_eval * d0));
+    hXe.resize((size_t)(o.n_eval * u0));
     hye.resize((size_t)o.n_eval);
-    agn::gen_dataset_rows(seed, d0, h->N, o.n_eval, h->dist, hXe.data());
+    agn::gen_dataset_rows(seed, u0, h->N, o.n_eval, h->dist, hXe.data());
     auto Ws = agn::gen_teacher(seed, h->tdims);
-    agn::gen_teacher_labels(hXe.data(), o.n_eval, d0, h->dist, h->tdims, Ws, hye.data());
+    agn::gen_teacher_labels(hXe.data(), o.n_eval, u0, h->dist, h->tdims, Ws, hye.data());
   }
 
-  // device buffers
+  // device buffers (the device dims from here on)
+  dims = h->dims.data();
+  const int d0 = dims[0];
   const size_t es = elem_size(h);
   const int64_t n = h->n, m = h->m;
   AGN_TRY(dalloc_t(h, &h->theta_c, (size_t)h->P_pad));
@@ -1288,11 +1376,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     for (float* p : {h->grad, h->mom1, h->mom2})
       AGN_TRY_CUDA(cudaMemset(p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
   }
-  h->use_head = h->prec == AGN_PREC_BF16 ? agn::head_fits<bf16>(dims[h->L - 1], dims[h->L])
-                                         : agn::head_fits<float>(dims[h->L - 1], dims[h->L]);
-  h->fuse_out_dw = h->use_tc && h->use_head && h->L >= 2 && (h->tc_mask & 4) && !(h->tc_mask & 8);
+  h->fuse_out_dw = h->use_tc && (h->use_head || h->out_tc) && (h->tc_mask & 4) && !(h->tc_mask & 8);
   h->ldz_out = h->fuse_out_dw ? (int)round_up(dims[h->L], 8) : dims[h->L];
-  h->fuse_head = h->use_tc && h->use_head && h->L >= 2 && (h->tc_mask & 1) &&
+  h->fuse_head = h->use_tc && h->use_head && (h->tc_mask & 1) &&
                  !(h->tc_mask & 32) && dims[h->L] <= agn::kHeadMaxClasses;
   if (h->split) {   // three piece planes of the activations (the weights stay fp32)
     h->Hs.assign(h->L, nullptr);
@@ -1312,9 +1398,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   // layer 1's operand is a tensor-core kernel (forward and dW)
   h->early_gather = h->use_tc && (h->tc_mask & 1) && (h->tc_mask & 4) && !(h->tc_mask & 8) &&
                     h->L >= 2 && d0 % 4 == 0;
-  // no gather at all when, besides, every reader of the labels is one of the
-  // output-layer kernels (the padded shards replace the alternate buffers)
-  h->direct_x = h->early_gather && h->use_head && !(h->tc_mask & 64);
+  // no gather at all then: the output-layer kernels and the softmax kernel read
+  // the labels in place too (the padded shards replace the alternate buffers)
+  h->direct_x = h->early_gather && !(h->tc_mask & 64);
   if (h->direct_x) {
     h->early_gather = false;
     const size_t rows = (size_t)(n * (h->S + m));
@@ -1353,7 +1439,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY(dalloc_t(h, &h->e_pred, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->e_out, 2));
     AGN_TRY(dalloc_t(h, &h->e_sw, 1));
-    AGN_TRY_CUDA(cudaMemcpy(h->Xe, hXe.data(), hXe.size() * sizeof(float), cudaMemcpyHostToDevice));
+    AGN_TRY(upload_rows(h->Xe, hXe.data(), E, h->udims[0], d0, sizeof(float)));
     AGN_TRY_CUDA(cudaMemcpy(h->ye, hye.data(), hye.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemset(h->e_sw, 0, sizeof(int)));
   }
@@ -1364,8 +1450,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY(dalloc_t(h, &h->fh_counter, (size_t)(2 * n * nchk)));
     AGN_TRY_CUDA(cudaMemsetAsync(h->fh_counter, 0, (size_t)(2 * n * nchk) * sizeof(int),
                                  h->stream));
-    h->loss_q = (int)nchk;
   }
+  if (h->fuse_head || !h->use_head) h->loss_q = (int)ceil_div(m, 32);
   h->grid = agn::commit_grid(h->P_pad);
   AGN_TRY(dalloc_t(h, &h->partials, (size_t)agn::kMaxCommitsPerLaunch * h->grid));
   AGN_TRY(dalloc_t(h, &h->pull_list, (size_t)n));
@@ -1376,8 +1462,10 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   // uploads
   std::vector<float> tpad((size_t)h->P_pad, 0.f);
   for (int l = 0; l < h->L; ++l) {
-    const int64_t fi = dims[l], fo = dims[l + 1];
-    std::memcpy(&tpad[h->woff[l]], &h->htheta0[h->woff_flat[l]], (size_t)(fo * fi) * sizeof(float));
+    const int64_t fi = h->udims[l], fo = h->udims[l + 1], ld = dims[l];
+    for (int64_t f = 0; f < fo; ++f)
+      std::memcpy(&tpad[h->woff[l] + f * ld], &h->htheta0[h->woff_flat[l] + f * fi],
+                  (size_t)fi * sizeof(float));
     std::memcpy(&tpad[h->boff[l]], &h->htheta0[h->boff_flat[l]], (size_t)fo * sizeof(float));
   }
   AGN_TRY_CUDA(cudaMemcpy(h->theta_c, tpad.data(), tpad.size() * sizeof(float),
@@ -1385,10 +1473,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   if (h->prec == AGN_PREC_BF16) {
     std::vector<bf16> xb(h->hX.size());
     for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16_rn(h->hX[i]);
-    AGN_TRY_CUDA(cudaMemcpy(h->X, xb.data(), xb.size() * sizeof(bf16), cudaMemcpyHostToDevice));
+    AGN_TRY(upload_rows(h->X, xb.data(), h->N, h->udims[0], d0, es));
   } else {
-    AGN_TRY_CUDA(cudaMemcpy(h->X, h->hX.data(), h->hX.size() * sizeof(float),
-                            cudaMemcpyHostToDevice));
+    AGN_TRY(upload_rows(h->X, h->hX.data(), h->N, h->udims[0], d0, es));
   }
   AGN_TRY_CUDA(cudaMemcpy(h->y, h->hy.data(), h->hy.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice));
@@ -1436,7 +1523,7 @@ Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int6
   if (h->n_eval <= 0)
     return Status::Err(AGN_E_INVALID, "the handle has no evaluation set (agn_options.n_eval)");
   if (pred && cap < h->n_eval) return Status::Err(AGN_E_INVALID, "pred shorter than n_eval");
-  const int L = h->L, C = h->dims[L];
+  const int L = h->L;
   AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build only
   for (int64_t r0 = 0; r0 < h->n_eval; r0 += h->eval_chunk) {
     const int rows = (int)std::min<int64_t>(h->eval_chunk, h->n_eval - r0);
@@ -1455,8 +1542,8 @@ Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int6
       AGN_TRY(agn::simt_forward<float>(g, l == L, 1, h->stream));
       in = out;
     }
-    AGN_TRY(agn::eval_logits(h->Ze, h->ye + r0, rows, C, h->e_loss + r0, h->e_correct + r0,
-                             h->e_pred + r0, h->stream));
+    AGN_TRY(agn::eval_logits(h->Ze, h->ye + r0, rows, h->C, h->dims[L], h->e_loss + r0,
+                             h->e_correct + r0, h->e_pred + r0, h->stream));
   }
   AGN_TRY(agn::eval_reduce(h->e_loss, h->e_correct, h->n_eval, h->e_out, h->stream));
   float o2[2];
@@ -1477,8 +1564,10 @@ Status read_params(agn_handle* h, const float* dev, float* out, int64_t cap) {
   AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
   AGN_TRY_CUDA(cudaMemcpy(tpad.data(), dev, tpad.size() * sizeof(float), cudaMemcpyDeviceToHost));
   for (int l = 0; l < h->L; ++l) {
-    const int64_t fi = h->dims[l], fo = h->dims[l + 1];
-    std::memcpy(out + h->woff_flat[l], &tpad[h->woff[l]], (size_t)(fo * fi) * sizeof(float));
+    const int64_t fi = h->udims[l], fo = h->udims[l + 1], ld = h->dims[l];
+    for (int64_t f = 0; f < fo; ++f)
+      std::memcpy(out + h->woff_flat[l] + f * fi, &tpad[h->woff[l] + f * ld],
+                  (size_t)fi * sizeof(float));
     std::memcpy(out + h->boff_flat[l], &tpad[h->boff[l]], (size_t)fo * sizeof(float));
   }
   return Status::Ok();

@@ -51,11 +51,26 @@ template <typename T>
 Status simt_backward_dx(const GemmArgs& g, int slots, cudaStream_t st);
 template <typename T>
 Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st);
-// Loss of slot z at local step `step` goes to loss_parts[slot_commit[z] * lam + step].
+// Softmax cross-entropy of a wave's logits: dZ = (softmax(Z) - onehot(y)) / m
+// and the loss of every 32-sample chunk of a slot, its cross-entropy sum / m,
+// at loss_parts[(slot_commit[z] * lam + step) * ceil(m / 32) + chunk].
+struct SoftmaxArgs {
+  const float* Z;          // [slots][m][ld] logits
+  int m, C, ld;            // columns C .. ld - 1 of dZ are left alone
+  const int* yb;           // labels [slots][m], or padded ones (x_shard > 0, batch_row0)
+  const int* slot_worker;
+  const long long* slot_t0;
+  int64_t x_shard;
+  void* dZ;                // out [slots][m][ld] (T)
+  bf16* dZ_pieces;         // fp32 T only: also its three exact bf16 pieces, planes
+  int64_t dZ_plane;        // dZ_plane apart; null = no
+  float* loss_parts;
+  const int* slot_commit;
+  int lam, step;
+  int* flag;
+};
 template <typename T>
-Status softmax_xent(const float* Z, const int* yb, T* dZ, int m, int C, float* loss_parts,
-                    const int* slot_commit, int lam, int step, int* flag, int slots,
-                    cudaStream_t st);
+Status softmax_xent(const SoftmaxArgs& a, int slots, cudaStream_t st);
 template <typename T>
 Status gather_batch(const T* X, const int* y, T* Xb, int* yb, int d0, int m, int64_t S,
                     const int* slot_worker, const long long* slot_t0, int step, int slots,
@@ -137,9 +152,9 @@ struct AdamArgs {
 Status adam_step(const AdamArgs& a, int slots, int num_sms, cudaStream_t st);
 
 // Evaluation (mlp_eval.cu): per-sample loss / correctness / prediction of
-// fp32 logits Z [rows][C] against labels y, and their fixed-order means
+// fp32 logits Z [rows][ld] (C classes) against labels y, and their fixed-order means
 // (out[0] loss, out[1] accuracy).
-Status eval_logits(const float* Z, const int* y, int rows, int C, float* loss, int* correct,
+Status eval_logits(const float* Z, const int* y, int rows, int C, int ld, float* loss, int* correct,
                    int* pred, cudaStream_t st);
 Status eval_reduce(const float* loss, const int* correct, int64_t E, float* out,
                    cudaStream_t st);

@@ -1,6 +1,8 @@
-// Kernels (a) and (b) on CUDA cores: the batched-over-workers MLP forward,
-// softmax cross-entropy, and backward with the fused local SGD step and
-// gradient accumulation of Algorithm 1 (g = grad L; theta_k -= eta g; a_k += g).
+// Kernels (a) and (b) on CUDA cores: the batched-over-workers MLP forward and
+// backward with the fused local SGD step and gradient accumulation of
+// Algorithm 1 (g = grad L; theta_k -= eta g; a_k += g) for AGN_GEMM_SIMT and
+// nets without a hidden layer; and, for either GEMM path, the softmax
+// cross-entropy of output layers the output-layer kernels do not take.
 //
 // One launch covers every worker of a wave: grid.z indexes the wave's slots,
 // and slot z reads and updates the replica of worker slot_worker[z].  All
@@ -204,48 +206,100 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
   }
 }
 
-// Softmax cross-entropy on Z [m][C] (fp32) per slot: dZ = (softmax - onehot)/m,
-// loss = mean_j (logsumexp(z_j) - z_j[y_j]), summed over the block in a fixed
-// order.  One block per slot.
-template <typename T>
-__global__ void __launch_bounds__(128) softmax_xent_kernel(const float* __restrict__ Z,
-                                                           const int* __restrict__ yb, T* dZ,
-                                                           int m, int C, float* loss_parts,
-                                                           const int* slot_commit, int lam,
-                                                           int step, int* flag) {
+// Softmax cross-entropy (SoftmaxArgs).  A block takes a 32-sample chunk of a
+// slot, a warp four of its samples with the classes across the lanes, so that
+// a launch of few slots still fills the GPU and every load is coalesced: one
+// block per slot with a sample per thread took 38 us a launch at 4 slots x 512
+// samples x 10 classes.  kPer > 0: up to 32 kPer
+// classes held in registers; 0: any number, read three times.  Sums are fixed
+// shuffle trees, the chunk's loss a fixed tree over its samples.
+constexpr int kXentThreads = 256;
+template <typename T, int kPer>
+__global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const SoftmaxArgs a) {
   pdl_begin();
-  const int z = blockIdx.x;
-  const float* Zs = Z + (int64_t)z * m * C;
-  T* dZs = dZ + (int64_t)z * m * C;
-  const int* ys = yb + (int64_t)z * m;
+  __shared__ float ces[32];
+  const int z = blockIdx.y, chunk = blockIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = a.m, C = a.C;
   const float inv_m = 1.0f / (float)m;
-  float part = 0.f;
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    const float* zr = Zs + (int64_t)j * C;
-    float mx = AGN_LD(zr);
-    for (int c = 1; c < C; ++c) mx = fmaxf(mx, AGN_LD(zr + c));
-    float s = 0.f;
-    for (int c = 0; c < C; ++c) s += expf(AGN_LD(zr + c) - mx);
-    const int y = AGN_LD(ys + j);
-    part += (logf(s) + mx) - AGN_LD(zr + y);
-    const float inv_s = 1.0f / s;
-    for (int c = 0; c < C; ++c) {
-      float p = expf(AGN_LD(zr + c) - mx) * inv_s;
-      if (c == y) p -= 1.0f;
-      AGN_ST(dZs + (int64_t)j * C + c, from_f<T>(p * inv_m));
+  constexpr int kSamples = 32 / (kXentThreads / 32);   // per warp
+  const int* yrow =
+      a.x_shard > 0
+          ? a.yb + (int64_t)AGN_LD(a.slot_worker + z) * (a.x_shard + m) +
+                batch_row0(a.slot_t0, z, a.step, m, a.x_shard)
+          : a.yb + (int64_t)z * m;
+  float v[kSamples][kPer > 0 ? kPer : 1];
+  if (kPer > 0) {   // every sample's loads in flight together
+#pragma unroll
+    for (int u = 0; u < kSamples; ++u) {
+      const int j = 32 * chunk + kSamples * warp + u;
+#pragma unroll
+      for (int e = 0; e < kPer; ++e)
+        v[u][e] = j < m && lane + 32 * e < C
+                      ? AGN_LD(a.Z + ((int64_t)z * m + j) * a.ld + lane + 32 * e)
+                      : -INFINITY;
     }
   }
-  __shared__ float red[128];
-  red[threadIdx.x] = part;
-  __syncthreads();
-  for (int s = 64; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kSamples; ++u) {
+    const int jl = kSamples * warp + u, j = 32 * chunk + jl;
+    if (j >= m) {   // warp-uniform
+      if (lane == 0) ces[jl] = 0.f;
+      continue;
+    }
+    const int64_t row = ((int64_t)z * m + j) * a.ld;
+    const float* zr = a.Z + row;
+    const int n = kPer > 0 ? kPer : (C + 31) / 32;
+    auto at = [&](int e) {
+      return kPer > 0 ? v[u][kPer > 0 ? e : 0] : lane + 32 * e < C ? AGN_LD(zr + lane + 32 * e) : -INFINITY;
+    };
+    float mx = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < n; ++e) mx = fmaxf(mx, at(e));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    const int y = AGN_LD(yrow + j);
+    float s = 0.f, zy = 0.f;
+#pragma unroll
+    for (int e = 0; e < n; ++e) {
+      const int c = lane + 32 * e;
+      if (c < C) s += expf(at(e) - mx);
+      if (c == y) zy = at(e);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    zy = __shfl_sync(0xffffffffu, zy, y & 31);
+    const float inv_s = 1.0f / s;
+#pragma unroll
+    for (int e = 0; e < n; ++e) {
+      const int c = lane + 32 * e;
+      if (c >= C) continue;
+      float p = expf(at(e) - mx) * inv_s;
+      if (c == y) p -= 1.0f;
+      const T g = from_f<T>(p * inv_m);
+      AGN_ST(static_cast<T*>(a.dZ) + row + c, g);
+      if (a.dZ_pieces) {
+        bf16 q0, q1, q2;
+        split3(to_f(g), q0, q1, q2);
+        AGN_ST(a.dZ_pieces + row + c, q0);
+        AGN_ST(a.dZ_pieces + a.dZ_plane + row + c, q1);
+        AGN_ST(a.dZ_pieces + 2 * a.dZ_plane + row + c, q2);
+      }
+    }
+    if (lane == 0) ces[jl] = (logf(s) + mx) - zy;
   }
-  if (threadIdx.x == 0) {
-    const float loss = red[0] * inv_m;
-    AGN_ST(loss_parts + (int64_t)AGN_LD(slot_commit + z) * lam + step, loss);
-    if (!isfinite(loss)) atomicExch(flag, 1);
+  __syncthreads();
+  if (warp == 0) {
+    float ce = ces[lane];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, off);
+    if (lane == 0) {
+      const float part = ce * inv_m;
+      AGN_ST(a.loss_parts +
+                 ((int64_t)AGN_LD(a.slot_commit + z) * a.lam + a.step) * gridDim.x + chunk,
+             part);
+      if (!isfinite(part)) atomicExch(a.flag, 1);
+    }
   }
 }
 
@@ -350,14 +404,12 @@ Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st) {
   return launch_gemm<T, T, false, false, kEpiDW>(g, slots, st);
 }
 template <typename T>
-Status softmax_xent(const float* Z, const int* yb, T* dZ, int m, int C, float* loss_parts,
-                    const int* slot_commit, int lam, int step, int* flag, int slots,
-                    cudaStream_t st) {
-  {
-    auto kf = softmax_xent_kernel<T>;
-    AGN_TRY_CUDA(launch_pdl(kf, slots, 128, 0, st, Z,
-                            yb, dZ, m, C, loss_parts, slot_commit, lam, step, flag));
-  }
+Status softmax_xent(const SoftmaxArgs& a, int slots, cudaStream_t st) {
+  const dim3 grid((unsigned)ceil_div(a.m, 32), (unsigned)slots);
+  auto kf = a.C <= 32    ? softmax_xent_kernel<T, 1>
+            : a.C <= 128 ? softmax_xent_kernel<T, 4>
+                         : softmax_xent_kernel<T, 0>;
+  AGN_TRY_CUDA(launch_pdl(kf, grid, kXentThreads, 0, st, a));
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();
 }
@@ -394,8 +446,7 @@ Status gather_batch(const T* X, const int* y, T* Xb, int* yb, int d0, int m, int
   template Status simt_forward<T>(const GemmArgs&, bool, int, cudaStream_t);                 \
   template Status simt_backward_dx<T>(const GemmArgs&, int, cudaStream_t);                   \
   template Status simt_backward_dw<T>(const GemmArgs&, int, cudaStream_t);                   \
-  template Status softmax_xent<T>(const float*, const int*, T*, int, int, float*, const int*, \
-                                  int, int, int*, int, cudaStream_t);                        \
+  template Status softmax_xent<T>(const SoftmaxArgs&, int, cudaStream_t);                    \
   template Status gather_batch<T>(const T*, const int*, T*, int*, int, int, int64_t,          \
                                   const int*, const long long*, int, int, cudaStream_t,       \
                                   bf16*, int64_t, int);

@@ -308,7 +308,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int p = 0; p < kSplit; ++p) {
           uint8_t* sb = sb0 + p * Cfg::kBBytes;
           if (!kBMN) {
-            load(sb, &tmB, kc, n_tile * BN + b_row0, b_z, p, &full[s]);
+#pragma unroll
+            for (int c = 0; c < BN / kTcBoxN; ++c)
+              load(sb + c * (kTcBoxN * Cfg::kRowBytes), &tmB, kc,
+                   n_tile * BN + c * kTcBoxN + b_row0, b_z, p, &full[s]);
           } else {
 #pragma unroll
             for (int c = 0; c < BN / 64; ++c)
@@ -725,7 +728,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       float* sPart = sW3 + kHC * 128;
       float* sG = sPart + 8 * 16 * kHC;
       uint16_t* sMask = reinterpret_cast<uint16_t*>(sG + 32 * kHC);   // [owned chunk][thread]
-      const int nchk = (args.N + 31) / 32;
+      const int nchk = (args.N + 31) / 32, nc0 = n_tile * kNch;   // this tile's first chunk
       if (kEpi == kEpiFwdHead && have) {
 #pragma unroll
         for (int k = 0; k < kW3Per; ++k) sW3[threadIdx.x + k * kThreads] = w3v_reg[k];
@@ -744,7 +747,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < 16; ++i) tT[i * 32 + lane] = __uint_as_float(r[i]);
           __syncwarp();
-          if (kEpi == kEpiFwdHead && (c0 - co) / 32 < nchk) {
+          if (kEpi == kEpiFwdHead && nc0 + (c0 - co) / 32 < nchk) {
             // Pass 1 of the fused output layer, before this chunk's stores (so
             // that the release below orders only the partials): this CTA's
             // share of the chunk's logits, sum over its 128 features of
@@ -812,7 +815,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             sMask[o * kThreads + threadIdx.x] = (uint16_t)mbits;
             __syncthreads();
-            const int chunk = (c0 - co) / 32;
+            const int chunk = nc0 + (c0 - co) / 32;
             float* gp = args.head_part +
                         (((int64_t)slot * nchk + chunk) * gridDim.x + m_tile) * (32 * kHC);
             for (int i = threadIdx.x; i < 32 * kHC; i += kThreads) {
@@ -851,7 +854,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                   for (int e = 0; e < 4; ++e) v[e] = hv[e] > 0.f ? v[e] : 0.f;
                 }
                 const int64_t o4 = (int64_t)j * args.ldo + row4;
-                store4(out + o4, v);
+                if (kEpi == kEpiFwd && kSplit == 1 && args.out_f32)
+                  store4(static_cast<float*>(args.out) + (int64_t)slot * args.out_bstride + o4, v);
+                else
+                  store4(out + o4, v);
                 if (kSplit == 3 && args.out_pieces) {
                   uint2 q0, q1, q2;
                   split3_x4(v, q0, q1, q2);
@@ -880,7 +886,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int mtn = (int)gridDim.x;
 #pragma unroll 1
           for (int o = 0; o < n_own; ++o) {
-            const int chunk = own_rank + o * kstride;
+            const int chunk = nc0 + own_rank + o * kstride;
             if (chunk >= nchk) continue;   // CTA-uniform
             int* ctr = args.head_counter + slot * nchk + chunk;
             if (threadIdx.x == 0)
@@ -926,7 +932,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
               for (int hh = 0; hh < 2; ++hh) {
                 const int sl = 16 * hh + (threadIdx.x >> 4);   // sample within the chunk
-                const int j = n_tile * BN + 32 * chunk + sl;
+                const int j = 32 * chunk + sl;
                 const bool valid = j < args.N;
                 const float z = cv ? (hh ? zz[1] : zz[0]) + bc : -INFINITY;
                 float mx = z;
@@ -994,7 +1000,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               }
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
-                const int j = n_tile * BN + 32 * chunk + co + jl + 4 * u;
+                const int j = 32 * chunk + co + jl + 4 * u;
                 if (j < args.N) {
                   float dv[4];
 #pragma unroll
@@ -1188,7 +1194,7 @@ Status launch_tc(const CUtensorMap& a, const CUtensorMap& b, const TcArgs& args,
     AGN_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t tiles = (int64_t)ceil_div(args.M, 128) * ceil_div(args.N, BN) * slots;
     if (tiles * ks > sms) ks = 1;
-    if (kEpi == kEpiFwdHead && (tiles > sms || ceil_div(args.N, BN) != 1)) {
+    if (kEpi == kEpiFwdHead && tiles > sms) {
       if (launched) *launched = false;
       return Status::Ok();
     }
@@ -1333,7 +1339,7 @@ Status tc_forward_head(const CUtensorMap& w_k, const CUtensorMap& h_k, const TcA
   if (args.head_C < 1 || args.head_C > kHC || !args.head_part || !args.head_counter ||
       !args.dh || !args.dzl || !args.loss_parts)
     return Status::Err(AGN_E_INVALID, "fused output layer without its buffers");
-  if ((int64_t)ceil_div(args.M, 128) * slots > num_sms) return Status::Ok();
+  if (ceil_div(args.M, 128) * ceil_div(args.N, bn) * (int64_t)slots > num_sms) return Status::Ok();
   if (split) {
     if (bn == 64)
       return launch_tc<64, false, false, kEpiFwdHead, 6, 3>(w_k, h_k, args, slots, st, launched);

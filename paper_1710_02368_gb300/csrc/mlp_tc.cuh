@@ -16,6 +16,7 @@ struct TcArgs {
   int a_by_worker, b_by_worker;
   int* err;                // set to 1 when a bounded wait gives up
   void* out;               // forward / dX output (bf16) [slots][N rows][ldo]
+  int out_f32;             // forward, bf16 mode: the output is fp32 (the logits)
   int64_t ldo, out_bstride;
   const void* mask;        // dX: H_{l-1}, same layout and type as out
   int64_t mask_bstride;
@@ -94,9 +95,9 @@ struct TcArgs {
   int no_a_prefetch;
 };
 
-// Column tile used for an N: the tensor map of the operand that spans N
-// must have this many rows (K-major) or 64-element chunks summing to it.
-inline int tc_bn(int N) { return N <= 64 ? 64 : N <= 128 ? 128 : 256; }
+// Column tiles of the forward and dX are 64, 128 or 256 samples wide
+// (tc_bn); their activation operand lands in boxes of kTcBoxN rows.
+constexpr int kTcBoxN = 64;
 constexpr int kTcSplitBK = 32;      // forward / dX k per stage, split (fp32) mode
 constexpr int kTcDwBN = 256;        // dW column tile, bf16 mode
 constexpr int kTcDwBNSplit = 128;   // dW column tile, split (fp32) mode
@@ -119,11 +120,11 @@ Status make_tmap_bf16_4d(CUtensorMap* map, const void* base, uint64_t inner, uin
 // split = false: bf16 operands (3D maps), bf16 activations.
 // split = true : fp32 operands as three exact bf16 pieces (4D maps), fp32
 //                activations; dW writes the three pieces of the new weights.
-// forward: w_k box {64, 128} over W (K-major); h_k box {64, bn} over H_{l-1},
-// bn = tc_bn(N) the column tile.  Small waves split K instead (args.ksplit).
+// forward: w_k box {64, 128} over W (K-major); h_k box {64, kTcBoxN} over
+// H_{l-1}; bn the column tile (64, 128 or 256).  Small waves split K (args.ksplit).
 Status tc_forward(const CUtensorMap& w_k, const CUtensorMap& h_k, const TcArgs& args, int slots,
                   cudaStream_t st, bool split, int bn);
-// dX: w_mn box {64, 64} over W (MN-major view); dz_k box {64, bn} over dZ_l.
+// dX: w_mn box {64, 64} over W (MN-major view); dz_k box {64, kTcBoxN} over dZ_l.
 // The forward GEMM of the last hidden layer with the output layer fused
 // (args.head_* set, args.relu = 1).  Needs every CTA of the launch resident at
 // once; when the launch would exceed the SMs nothing is queued and *launched
