@@ -57,6 +57,7 @@ struct NvtxRange {
 struct Wave {
   int offset = 0;                 // first slot in the run's plan arrays
   int slots = 0;
+  int repulls = 0;                // slots whose worker pulls anew later in the run
   std::vector<CommitPlan> commits;
 };
 
@@ -246,6 +247,9 @@ struct agn_handle {
   // and H_{L-1}'s pieces kept
   bool fuse_out_dw = false;
   int ldz_out = 0;
+  // the first local step of a commit stores a_k = g, so no commit zeroes a_k
+  // (every layer's dW in the persistent tensor-core launch, or Adam)
+  bool acc_first = false;
   float* ce_partial = nullptr;    // [n][ceil(m / kHeadSamples)]
   int* head_counter = nullptr;    // [n]
   // the output layer fused into the last hidden layer's tensor-core forward
@@ -282,10 +286,12 @@ struct agn_handle {
   int64_t cap_commits = 0;
   float* loss_parts = nullptr;
   int64_t cap_parts = 0;
+  // the run's plan arrays, one entry per slot, in one buffer (one upload)
+  long long* plan_t0 = nullptr;
   int* plan_worker = nullptr;
   int* plan_commit = nullptr;
-  long long* plan_t0 = nullptr;
-  int64_t cap_plan = 0;
+  int* plan_repull = nullptr;
+  int64_t cap_plan = 0;       // entries of 20 bytes
   int* pull_list = nullptr;   // [n]
   // host state
   std::vector<float> hX, htheta0;
@@ -625,18 +631,24 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
                                          : reinterpret_cast<const T*>(h->rep);
   const float eta = (float)h->eta;
   const double es = (double)sizeof(T);
-  // bytes per parameter of the local step + accumulation: theta RMW, a RMW, and
-  // the low-precision copy (one bf16, or three pieces in the split mode)
-  // (with Adam the dW kernels only store the gradient, 4 bytes; the Adam
-  // kernel's own traffic is counted at its launch)
-  const double upd = h->adam ? 4.0
-                             : (h->elide ? 8.0 : 16.0) + (h->prec == AGN_PREC_BF16 ? 2.0 : 0.0);
   // pieces of dZ_l (split mode, hidden tensor-core layers), planes n m d_l apart
   auto dz_pieces = [&](int l) -> bf16* {
     return (h->split && l >= 1 && tc_layer(h, l)) ? h->dZp[l] : nullptr;
   };
   auto dz_plane = [&](int l) -> int64_t { return (int64_t)n * m * h->dims[l]; };
   for (int i = 0; i < h->lam; ++i) {
+    // The last local step before a worker's next pull: nothing reads theta_k
+    // between the two (the commit takes a_k), so its dW adds g to a_k only.
+    const bool last_acc = i == h->lam - 1 && h->acc_first && !h->adam && !h->elide;
+    const bool acc_only = last_acc && wv.repulls == s;
+    const double theta_share = last_acc ? (double)(s - wv.repulls) / s : 1.0;
+    // bytes per parameter of this step's dW: theta RMW (or none), a RMW (the
+    // first step stores only) and the low-precision copy; with Adam the dW
+    // kernels only store the gradient, 4 bytes (the Adam kernel's own traffic
+    // is counted at its launch)
+    const double acc_b = h->elide ? 0.0 : h->acc_first && i == 0 ? 4.0 : 8.0;
+    const double upd = h->adam ? 4.0
+                       : theta_share * (h->prec == AGN_PREC_BF16 ? 10.0 : 8.0) + acc_b;
     // this local step's buffer of layer 1's tensor-core operand
     const bool alt = h->early_gather && h->gparity;
     const agn_handle::LayerMaps& l1 = alt ? h->l1_alt : h->tmaps.empty() ? h->l1_alt : h->tmaps[0];
@@ -912,6 +924,12 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       Launch k(h, AGN_K_BACKWARD_DW, tc_flops, tc_bytes, launches);
       agn::TcArgs t = tc_args(h, sw, st0, i);
       t.K = m; t.eta = eta;
+      if (acc_only) {
+        t.grad_out = h->acc; t.grad_add = i > 0;
+      } else {
+        t.acc_set = h->acc_first && i == 0;
+        if (last_acc && wv.repulls > 0) t.slot_repull = h->plan_repull + wv.offset;
+      }
       AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
                                   h->num_sms));
     }
@@ -921,10 +939,11 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       ad.m = h->mom1; ad.v = h->mom2; ad.theta_b = h->rep_b; ad.piece_plane = h->piece_plane;
       ad.P = h->P_pad; ad.ld = h->P_pad;
       ad.slot_worker = sw; ad.slot_t0 = st0; ad.step = i;
+      ad.acc_set = i == 0;
       ad.eta = eta; ad.beta1 = h->beta1; ad.beta2 = h->beta2; ad.eps = h->eps;
       const double copy_b = h->rep_b ? 2.0 : 0.0;
       Launch k(h, AGN_K_BACKWARD_DW, 0.0,
-               (double)s * h->P * (4.0 + 16.0 + 8.0 + (h->elide ? 0.0 : 8.0) + copy_b), launches);
+               (double)s * h->P * (4.0 + 16.0 + 8.0 + acc_b + copy_b), launches);
       AGN_TRY(agn::adam_step(ad, s, h->num_sms, h->stream));
     }
   }
@@ -935,10 +954,13 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
 // Planning
 // ---------------------------------------------------------------------------
 
+// Bytes per slot of the plan buffer: slot_t0, then worker, commit and repull.
+constexpr int64_t kPlanEntry = sizeof(long long) + 3 * sizeof(int);
+
 struct RunPlan {
   std::vector<int> start_pulls;
   std::vector<Wave> waves;
-  std::vector<int> slot_worker, slot_commit;
+  std::vector<int> slot_worker, slot_commit, slot_repull;
   std::vector<long long> slot_t0;
   std::vector<int64_t> prev, pulled_v, steps;
 };
@@ -974,6 +996,7 @@ Status build_plan(const agn_handle* h, int k, const int32_t* worker, const int32
     else if (look[w] < 0) look[w] = i;
   }
   std::vector<std::vector<int>> pulls_at(k + 1);   // pulls at version V0 + j
+  std::vector<char> repulled(k, 0);   // commit i's worker pulls anew later in the run
   std::vector<int64_t> pulled = h->pulled_v;
   for (int w = 0; w < n; ++w) {
     std::vector<int> lst = q[w];
@@ -1000,6 +1023,7 @@ Status build_plan(const agn_handle* h, int k, const int32_t* worker, const int32
       if (vc <= V0 + k) {
         pulls_at[vc - V0].push_back(w);
         pulled[w] = vc;
+        if (e > 0) repulled[lst[e - 1]] = 1;
       }
     }
     if (!q[w].empty()) {
@@ -1028,6 +1052,8 @@ Status build_plan(const agn_handle* h, int k, const int32_t* worker, const int32
           steps[w] += h->lam;
           ++ptr[w];
           computed[i] = 1;
+          out->slot_repull.push_back(repulled[i]);
+          wv.repulls += repulled[i];
         }
       }
     }
@@ -1091,21 +1117,28 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
     h->cap_commits = c1;
   }
   AGN_TRY(grow(h, &h->loss_parts, &h->cap_parts, (int64_t)k * h->lam * h->loss_q, 0));
-  if (total_slots > h->cap_plan) {  // the three plan arrays share one capacity
-    int64_t c1 = h->cap_plan, c2 = h->cap_plan, c3 = h->cap_plan;
-    AGN_TRY(grow(h, &h->plan_worker, &c1, total_slots, 0));
-    AGN_TRY(grow(h, &h->plan_commit, &c2, total_slots, 0));
-    AGN_TRY(grow(h, &h->plan_t0, &c3, total_slots, 0));
-    h->cap_plan = c1;
+  if (total_slots > h->cap_plan) {
+    const int64_t cap = std::max(total_slots, 2 * h->cap_plan);
+    char* buf = nullptr;
+    AGN_TRY(dalloc_t(h, &buf, (size_t)cap * kPlanEntry));
+    AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+    dfree(h, h->plan_t0);
+    h->plan_t0 = reinterpret_cast<long long*>(buf);
+    h->cap_plan = cap;
   }
   AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build: buffers as grown
+  std::vector<char> packed((size_t)(total_slots * kPlanEntry));
   if (total_slots > 0) {
-    AGN_TRY_CUDA(cudaMemcpyAsync(h->plan_worker, plan.slot_worker.data(), total_slots * sizeof(int),
-                                 cudaMemcpyHostToDevice, h->stream));
-    AGN_TRY_CUDA(cudaMemcpyAsync(h->plan_commit, plan.slot_commit.data(), total_slots * sizeof(int),
-                                 cudaMemcpyHostToDevice, h->stream));
-    AGN_TRY_CUDA(cudaMemcpyAsync(h->plan_t0, plan.slot_t0.data(), total_slots * sizeof(long long),
-                                 cudaMemcpyHostToDevice, h->stream));
+    const size_t ts = (size_t)total_slots;
+    h->plan_worker = reinterpret_cast<int*>(h->plan_t0 + ts);
+    h->plan_commit = h->plan_worker + ts;
+    h->plan_repull = h->plan_commit + ts;
+    std::memcpy(packed.data(), plan.slot_t0.data(), ts * sizeof(long long));
+    std::memcpy(packed.data() + ts * 8, plan.slot_worker.data(), ts * sizeof(int));
+    std::memcpy(packed.data() + ts * 12, plan.slot_commit.data(), ts * sizeof(int));
+    std::memcpy(packed.data() + ts * 16, plan.slot_repull.data(), ts * sizeof(int));
+    AGN_TRY_CUDA(cudaMemcpyAsync(h->plan_t0, packed.data(), packed.size(), cudaMemcpyHostToDevice,
+                                 h->stream));
   }
   int64_t launches = 0;
   AGN_TRY_CUDA(cudaEventRecord(h->ev0, h->stream));
@@ -1138,11 +1171,11 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
       {
         const double copy_b = h->rep_b ? 2.0 : 0.0;
         Launch kc(h, AGN_K_COMMIT, 2.0 * cp.n_commits * h->P,
-                  (double)h->P * (8.0 + 8.0 * cp.n_commits +
+                  (double)h->P * (8.0 + (h->elide || !h->acc_first ? 8.0 : 4.0) * cp.n_commits +
                                   pulls * (4.0 + copy_b + (h->elide ? 4.0 : 0.0))),
                   &launches);
         AGN_TRY(agn::launch_commit_pull(cp, h->theta_c, h->acc, h->rep, h->rep_b, h->P_pad,
-                                        h->P_pad, scale, true, h->partials, h->grid, nullptr,
+                                        h->P_pad, scale, !h->acc_first, h->partials, h->grid, nullptr,
                                         nullptr, h->stream, /*norms=*/false, h->piece_plane,
                                         h->elide));
       }
@@ -1377,6 +1410,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
       AGN_TRY_CUDA(cudaMemset(p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
   }
   h->fuse_out_dw = h->use_tc && (h->use_head || h->out_tc) && (h->tc_mask & 4) && !(h->tc_mask & 8);
+  h->acc_first = h->fuse_out_dw || h->adam;
   h->ldz_out = h->fuse_out_dw ? (int)round_up(dims[h->L], 8) : dims[h->L];
   h->fuse_head = h->use_tc && h->use_head && (h->tc_mask & 1) &&
                  !(h->tc_mask & 32) && dims[h->L] <= agn::kHeadMaxClasses;

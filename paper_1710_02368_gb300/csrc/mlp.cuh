@@ -139,6 +139,7 @@ struct AdamArgs {
   const float* grad;       // [n][ld] raw minibatch gradients of this local step
   float* theta;            // [n][ld] fp32 replicas
   float* acc;              // [n][ld] accumulators (of the steps), or null
+  int acc_set;             // 1: a_k = the step (a commit's first), whatever a_k held
   float* m;                // [n][ld] first moments
   float* v;                // [n][ld] second moments
   bf16* theta_b;           // bf16 copies / piece 0 of three planes, or null

@@ -45,9 +45,11 @@ struct TcArgs {
   int* counter_clear;
   int counter_clear_n;
   // dW: store the raw gradient at grad_out [n][ld_param] (same layout as the
-  // replicas) instead of taking the local step (the optimizer runs after);
-  // null = fused local step
+  // replicas) instead of taking the local step (the optimizer runs after, or
+  // the replica is pulled anew before anything reads it); null = fused local
+  // step.  grad_add: add it to what is there instead.
   float* grad_out;
+  int grad_add;
   // Forward of the last hidden layer with the output layer fused into its
   // epilogue (tc_forward_head): the d_L <= 16 logits of every sample from the
   // CTAs' partial sums over their 128 features, softmax cross-entropy, dZ_L and
@@ -91,6 +93,11 @@ struct TcArgs {
   // dW: 1 reads a_k's chunks through the parameter ring and stores a_k + g;
   // 0 adds g to a_k in the L2 (red.add) and keeps the ring for theta_k
   int acc_ring;
+  // dW: 1 stores a_k = g (the first local step of a commit), whatever a_k held
+  int acc_set;
+  // dW: slots with slot_repull[slot] != 0 take no local step, only a_k (their
+  // replica is pulled anew before anything reads it); null = none
+  const int* slot_repull;
   // forward / dX: 1 requests no weight stage before the dependency wait
   int no_a_prefetch;
 };

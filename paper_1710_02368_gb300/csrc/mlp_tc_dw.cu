@@ -85,7 +85,7 @@ struct DwCfg {
   static constexpr bool kAccRing = kMode == kDwUpdAcc;                     // a_k via the ring
   static constexpr int kArrays = kAccRing ? 2 : 1;
   static constexpr int kSlotBytes = kArrays * (kChunkBytes + kBiasHalf);
-  static constexpr int kRing = kAccRing ? 3 : 6;
+  static constexpr int kRing = kMode == kDwGrad ? 1 : kAccRing ? 3 : 6;   // (kDwGrad: unused)
   static constexpr int kBK = kBKs;
   static constexpr int kBox = kBK * 128;
   static constexpr int kABytes = 2 * kBox;
@@ -184,6 +184,10 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int T = B.total_tiles;
+  // a slot whose replica nothing reads before its next pull: a_k only
+  auto acc_only = [&](int slot) -> bool {
+    return kMode == kDwUpdRed && args.slot_repull && AGN_LD(args.slot_repull + slot) != 0;
+  };
   const int KT = (args.K + kBK - 1) / kBK;
 
   if (threadIdx.x == 0) {
@@ -339,7 +343,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       // a pull, two or more launches back: the first tile's first chunks are
       // requested before waiting for the preceding kernel
       int npre = 0;
-      if (!kGrad && (int)blockIdx.x < T) {
+      if (!kGrad && (int)blockIdx.x < T && !acc_only(decode(B, blockIdx.x).slot)) {
         const TileIdx t0 = decode(B, blockIdx.x);
         const DwLayer& L0 = B.layer[t0.layer];
         npre = min(kRing, min(Cfg::kChunks, (L0.N - t0.n_tile * BN + kCF - 1) / kCF));
@@ -354,7 +358,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         const TileIdx ti = decode(B, t);
         const DwLayer& L = B.layer[ti.layer];
         const int worker = AGN_LD(args.slot_worker + ti.slot);
-        const int nch = min(Cfg::kChunks, (L.N - ti.n_tile * BN + kCF - 1) / kCF);
+        const int nch = acc_only(ti.slot)
+                            ? 0 : min(Cfg::kChunks, (L.N - ti.n_tile * BN + kCF - 1) / kCF);
         for (int c = t == (int)blockIdx.x ? npre : 0; c < nch; ++c) {
           const int r = ch % kRing;
           if (ch >= kRing &&
@@ -466,6 +471,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       float* acc = kAcc ? args.acc + rbase : nullptr;
       bf16* tb = args.theta_b ? args.theta_b + rbase : nullptr;   // bf16 mode only
       const int nch = min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
+      const bool grad_only = kGrad || acc_only(ti.slot);
+      const bool grad_add = kGrad ? args.grad_add != 0 : !args.acc_set;
       for (int c = 0; c < nch; ++c) {
         const int r = ch % kRing;
         uint32_t v[16];
@@ -482,21 +489,26 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         }
 #pragma unroll
         for (int i = 0; i < 16; ++i) gS[i * 32 + lane] = __uint_as_float(v[i]);
-        if (kGrad) {   // raw gradient out: grad[w][p] = g, coalesced 16-byte stores
+        if (grad_only) {   // raw gradient out: grad (or a_k) = g or += g, coalesced 16 bytes
           __syncwarp();
           const int fbase = ti.n_tile * BN + c * kCF + 16 * hf;
-          float* gout = args.grad_out + rbase;
+          float* gout = kGrad ? args.grad_out + rbase : acc;
           if (quad_ok) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const int i = i0 + 4 * u;
-              if (fbase + i < N)
-                AGN_ST(reinterpret_cast<float4*>(gout + L.woff + (int64_t)(fbase + i) * M + k0 + k4),
-                       *reinterpret_cast<const float4*>(gS + i * 32 + k4));
+              if (fbase + i >= N) continue;
+              float* go = gout + L.woff + (int64_t)(fbase + i) * M + k0 + k4;
+              const float4 gv = *reinterpret_cast<const float4*>(gS + i * 32 + k4);
+              if (grad_add) AGN_RED4(go, gv);
+              else AGN_ST(reinterpret_cast<float4*>(go), gv);
             }
           }
-          if (kb >= 0 && kb < 32 && lane < 16 && fbase + lane < N)
-            AGN_ST(gout + L.boff + fbase + lane, gS[lane * 32 + kb]);
+          if (kb >= 0 && kb < 32 && lane < 16 && fbase + lane < N) {
+            float* go = gout + L.boff + fbase + lane;
+            if (grad_add) AGN_RED(go, gS[lane * 32 + kb]);
+            else AGN_ST(go, gS[lane * 32 + kb]);
+          }
           __syncwarp();
           continue;
         }
@@ -528,7 +540,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
                 AGN_ST(reinterpret_cast<float4*>(acc + p),
                        make_float4(av.x + gv.x, av.y + gv.y, av.z + gv.z, av.w + gv.w));
               } else if (kAcc) {   // a_k += g in the L2 (one add per element and launch)
-                AGN_RED4(reinterpret_cast<float*>(acc + p), gv);
+                if (args.acc_set) AGN_ST(reinterpret_cast<float4*>(acc + p), gv);
+                else AGN_RED4(acc + p, gv);
               }
               // the bf16 copy (bf16 mode); the fp32 mode's GEMMs split the
               // fp32 weights themselves
@@ -544,6 +557,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           const float tn = local_step(sTb[16 * hf + lane], eta, gb);
           AGN_ST(theta + pb, tn);
           if (kAccRing) AGN_ST(acc + pb, sTb[kCF + 16 * hf + lane] + gb);
+          else if (kAcc && args.acc_set) AGN_ST(acc + pb, gb);
           else if (kAcc) AGN_RED(acc + pb, gb);
           if (kSplit == 1) AGN_ST(tb + pb, __float2bfloat16_rn(tn));
         }
@@ -636,19 +650,22 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     // at the copy bandwidth: there the L2's adds slowed the stream by 4 %;
     // and always with args.acc_ring)
     constexpr int64_t kRedAccBytes = 64ll << 20;
-    const bool ring = args.acc_ring || acc_bytes > kRedAccBytes;
+    // (a first local step only stores a_k, and slots about to pull only add to
+    // it: the ring stays with theta_k)
+    const bool ring = !args.acc_set && !args.slot_repull &&
+                      (args.acc_ring || acc_bytes > kRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
                                    : kDwUpdRed;
     Status r = Status::Ok();
     if (split) {
-      r = mode == kDwGrad     ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwGrad>(batch, args, num_sms, st)
+      r = mode == kDwGrad     ? launch_dw<kTcDwBNSplit, 3, 4, 32, kDwGrad>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpd>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdAcc>(batch, args, num_sms, st)
                               : launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdRed>(batch, args, num_sms, st);
     } else {
-      r = mode == kDwGrad     ? launch_dw<kTcDwBN, 1, 2, 64, kDwGrad>(batch, args, num_sms, st)
+      r = mode == kDwGrad     ? launch_dw<kTcDwBN, 1, 4, 64, kDwGrad>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpd>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpdAcc>(batch, args, num_sms, st)
                               : launch_dw<kTcDwBN, 1, 2, 64, kDwUpdRed>(batch, args, num_sms, st);

@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(kOptThreads) adam_kernel(const AdamArgs a) {
     AGN_ST(reinterpret_cast<float4*>(a.v + p), make_float4(vv[0], vv[1], vv[2], vv[3]));
     AGN_ST(reinterpret_cast<float4*>(a.theta + p), make_float4(th[0], th[1], th[2], th[3]));
     if (a.acc) {
-      const float4 c4 = AGN_LD(reinterpret_cast<const float4*>(a.acc + p));
+      const float4 c4 = a.acc_set ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                  : AGN_LD(reinterpret_cast<const float4*>(a.acc + p));
       AGN_ST(reinterpret_cast<float4*>(a.acc + p),
              make_float4(c4.x + u[0], c4.y + u[1], c4.z + u[2], c4.w + u[3]));
     }
