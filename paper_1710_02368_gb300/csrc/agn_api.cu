@@ -247,6 +247,9 @@ struct agn_handle {
   // and H_{L-1}'s pieces kept
   bool fuse_out_dw = false;
   int ldz_out = 0;
+  // local steps whose activations and dZ the buffers keep ([hist][n][m][d]; 1:
+  // only the current one's), see run_wave_steps
+  int hist = 1;
   // the first local step of a commit stores a_k = g, so no commit zeroes a_k
   // (every layer's dW in the persistent tensor-core launch, or Adam)
   bool acc_first = false;
@@ -425,8 +428,9 @@ void collect_profile(agn_handle* h) {
 // layer too wide for the output-layer kernels.
 bool tc_layer(const agn_handle* h, int l) { return h->use_tc && (l < h->L || h->out_tc); }
 
-agn::TcArgs tc_args(agn_handle* h, const int* sw, const long long* st0, int step) {
+agn::TcArgs tc_args(agn_handle* h, const int* sw, const long long* st0, int step, int z0) {
   agn::TcArgs t{};
+  t.z0 = z0;
   t.slot_worker = sw;
   t.slot_t0 = st0;
   t.step = step;
@@ -460,6 +464,7 @@ void next_counters(agn_handle* h, agn::TcArgs* t) {
 // Tensor maps of the tcgen05 path (addresses are fixed for the handle's life).
 Status build_tc_maps(agn_handle* h) {
   const int n = h->n, m = h->m, L = h->L;
+  const int nh = n * h->hist;   // activation batches: slots of every kept local step
   constexpr uint32_t bn = agn::kTcBoxN;
   h->tmaps.assign(L - 1, {});
   for (int l = 1; l < L; ++l) {
@@ -497,11 +502,12 @@ Status build_tc_maps(agn_handle* h) {
     AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, 64, 128));
     AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 64, 64));
     const void* Hin = l == 1 ? h->Xb : h->H[l - 1];
-    AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, Hin, fi, m, n, fi, (uint64_t)m * fi, 64, bn));
-    AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_mn, Hin, fi, m, n, fi, (uint64_t)m * fi, 64, 64));
+    const int nl = l == 1 ? n : nh;
+    AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, Hin, fi, m, nl, fi, (uint64_t)m * fi, 64, bn));
+    AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_mn, Hin, fi, m, nl, fi, (uint64_t)m * fi, 64, 64));
     const void* dZ = h->dZ[l];
-    AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, dZ, fo, m, n, fo, (uint64_t)m * fo, 64, bn));
-    AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_mn, dZ, fo, m, n, fo, (uint64_t)m * fo, 64, 64));
+    AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, dZ, fo, m, nh, fo, (uint64_t)m * fo, 64, bn));
+    AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_mn, dZ, fo, m, nh, fo, (uint64_t)m * fo, 64, 64));
   }
   if (h->direct_x) {   // layer 1's operand maps over the padded shards
     const uint64_t fi = h->dims[0], rows = (uint64_t)(h->S + m);
@@ -558,8 +564,8 @@ Status build_tc_maps(agn_handle* h) {
         const bf16* W = h->rep_b + h->woff[L - 1];
         AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, 64, 128));
         AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 64, 64));
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, h->H[L - 1], fi, m, n, fi, (uint64_t)m * fi, 64, bn));
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, h->dZ[L], lz, m, n, lz, (uint64_t)m * lz, 64, bn));
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, h->H[L - 1], fi, m, nh, fi, (uint64_t)m * fi, 64, bn));
+        AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, h->dZ[L], lz, m, nh, lz, (uint64_t)m * lz, 64, bn));
       }
     }
     if (h->split) {
@@ -569,8 +575,8 @@ Status build_tc_maps(agn_handle* h) {
       AGN_TRY(agn::make_tmap_bf16_4d(&mp.dz_mn32, h->dZp[L], lz, m, n, lz, (uint64_t)m * lz,
                                      (uint64_t)n * m * lz, 64, 32));
     } else {
-      AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_mn, h->H[L - 1], fi, m, n, fi, (uint64_t)m * fi, 64, 64));
-      AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_mn, h->dZ[L], lz, m, n, lz, (uint64_t)m * lz, 64, 64));
+      AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_mn, h->H[L - 1], fi, m, nh, fi, (uint64_t)m * fi, 64, 64));
+      AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_mn, h->dZ[L], lz, m, nh, lz, (uint64_t)m * lz, 64, 64));
     }
   }
   return Status::Ok();
@@ -620,6 +626,9 @@ Status split_act(agn_handle* h, const void* src, bf16* dst, int d, int slots, in
 // One wave: lambda local steps of every slot (Algorithm 1's inner loop)
 // ---------------------------------------------------------------------------
 
+// The history of a wave's local steps: see agn_handle::hist.
+constexpr int kHistMaxSteps = 16, kHistMaxBatch = 256;
+
 template <typename T>
 Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
   const int s = wv.slots;
@@ -636,7 +645,19 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     return (h->split && l >= 1 && tc_layer(h, l)) ? h->dZp[l] : nullptr;
   };
   auto dz_plane = [&](int l) -> int64_t { return (int64_t)n * m * h->dims[l]; };
+  // bf16 waves whose accumulators stream from DRAM: each step's activations
+  // and dZ stay in the history, the steps' dW updates theta_k alone, and one
+  // launch sums the gradients of up to `hist` steps into a_k (K = steps m).
+  const bool defer = h->hist > 1 && (int64_t)s * h->P * 4 > agn::kTcRedAccBytes;
   for (int i = 0; i < h->lam; ++i) {
+    const int hi = defer ? i % h->hist : 0;   // this step's place in the history
+    auto Hl = [&](int l) -> void* {
+      return static_cast<char*>(h->H[l]) + (int64_t)hi * n * m * h->dims[l] * (int64_t)sizeof(T);
+    };
+    auto dZl = [&](int l) -> void* {
+      return static_cast<char*>(h->dZ[l]) +
+             (int64_t)hi * n * m * (l == L ? h->ldz_out : h->dims[l]) * (int64_t)sizeof(T);
+    };
     // The last local step before a worker's next pull: nothing reads theta_k
     // between the two (the commit takes a_k), so its dW adds g to a_k only.
     const bool last_acc = i == h->lam - 1 && h->acc_first && !h->adam && !h->elide;
@@ -646,7 +667,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // first step stores only) and the low-precision copy; with Adam the dW
     // kernels only store the gradient, 4 bytes (the Adam kernel's own traffic
     // is counted at its launch)
-    const double acc_b = h->elide ? 0.0 : h->acc_first && i == 0 ? 4.0 : 8.0;
+    const double acc_b = h->elide || defer ? 0.0 : h->acc_first && i == 0 ? 4.0 : 8.0;
     const double upd = h->adam ? 4.0
                        : theta_share * (h->prec == AGN_PREC_BF16 ? 10.0 : 8.0) + acc_b;
     // this local step's buffer of layer 1's tensor-core operand
@@ -684,16 +705,16 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       if (l == L && h->use_head) {   // output layer: forward + softmax-CE + dX, one kernel
         agn::HeadArgs a{};
         const int fi = h->dims[L - 1], C = h->dims[L];
-        a.H = L == 1 ? h->Xb : h->H[L - 1];
+        a.H = L == 1 ? h->Xb : Hl(L - 1);
         a.W = W; a.theta = h->rep; a.ld_param = h->P_pad;
         a.woff = h->woff[L - 1]; a.boff = h->boff[L - 1];
         a.K = fi; a.C = C; a.m = m;
         a.slot_worker = sw; a.yb = h->yb;
         a.slot_t0 = st0; a.x_shard = h->direct_x ? h->S : 0;
-        a.dZL = h->dZ[L]; a.ldz = h->ldz_out;
+        a.dZL = dZl(L); a.ldz = h->ldz_out;
         a.dZL_pieces = (h->fuse_out_dw && h->split) ? h->dZp[L] : nullptr;
         a.dZL_plane = (int64_t)n * m * h->ldz_out;
-        a.dH = L > 1 ? h->dZ[L - 1] : nullptr;
+        a.dH = L > 1 ? dZl(L - 1) : nullptr;
         a.dH_pieces = L > 1 ? dz_pieces(L - 1) : nullptr;
         a.dH_plane = L > 1 ? dz_plane(L - 1) : 0;
         a.ce_partial = h->ce_partial; a.counter = h->head_counter;
@@ -708,10 +729,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       agn::GemmArgs g{};
       const int fi = h->dims[l - 1], fo = h->dims[l];
       g.M = m; g.N = fo; g.K = fi;
-      g.a = l == 1 ? h->Xb : h->H[l - 1]; g.lda = fi; g.a_bstride = (int64_t)m * fi;
+      g.a = l == 1 ? h->Xb : Hl(l - 1); g.lda = fi; g.a_bstride = (int64_t)m * fi;
       g.b = W + h->woff[l - 1]; g.ldb = fi; g.b_bstride = h->P_pad; g.b_by_worker = 1;
       g.slot_worker = sw;
-      g.out = l == L ? static_cast<void*>(h->Z) : h->H[l];
+      g.out = l == L ? static_cast<void*>(h->Z) : Hl(l);
       g.ldo = fo; g.out_bstride = (int64_t)m * fo;
       g.relu = l < L;
       g.theta = h->rep; g.ld_param = h->P_pad; g.boff = h->boff[l - 1];
@@ -736,18 +757,18 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
                            : 0.0),
                  launches);
         if (fuse) {
-          agn::TcArgs t = tc_args(h, sw, st0, i);
+          agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
           t.M = fo; t.N = m; t.K = fi;
           t.a_by_worker = 1;
-          t.out = h->H[l]; t.ldo = fo; t.out_bstride = (int64_t)m * fo;
+          t.out = Hl(l); t.ldo = fo; t.out_bstride = (int64_t)m * fo;
           t.relu = 1; t.boff = h->boff[l - 1];
           t.out_pieces = h_pieces; t.out_plane = (int64_t)n * m * fo;
           t.head_woff = h->woff[L - 1]; t.head_boff = h->boff[L - 1]; t.head_C = C;
           t.yb = h->yb;
-          t.dzl = h->dZ[L]; t.ldz = h->ldz_out;
+          t.dzl = dZl(L); t.ldz = h->ldz_out;
           t.dzl_pieces = (h->fuse_out_dw && h->split) ? h->dZp[L] : nullptr;
           t.dzl_plane = (int64_t)n * m * h->ldz_out;
-          t.dh = h->dZ[L - 1]; t.dh_pieces = dz_pieces(L - 1); t.dh_plane = dz_plane(L - 1);
+          t.dh = dZl(L - 1); t.dh_pieces = dz_pieces(L - 1); t.dh_plane = dz_plane(L - 1);
           t.head_part = h->fh_part;
           {   // the fused output layer's counters alternate like the split-K ones
             const int hn = n * (int)ceil_div(m, 32);
@@ -772,10 +793,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           head_done = true;
           dz_ready = t.dh_pieces != nullptr;
         } else if (tc_layer(h, l) && (h->tc_mask & 1)) {
-          agn::TcArgs t = tc_args(h, sw, st0, i);
+          agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
           t.M = fo; t.N = m; t.K = fi;
           t.a_by_worker = 1;
-          t.out = l == L ? static_cast<void*>(h->Z) : h->H[l];
+          t.out = l == L ? static_cast<void*>(h->Z) : Hl(l);
           t.out_f32 = l == L;
           t.ldo = fo; t.out_bstride = (int64_t)m * fo;
           t.relu = l < L; t.boff = h->boff[l - 1];
@@ -793,13 +814,13 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           AGN_TRY(agn::simt_forward<T>(g, l == L, s, h->stream));
         }
       }
-      if (h_pieces && !pieces_done) AGN_TRY(split_act(h, h->H[l], h_pieces, fo, s, launches));
+      if (h_pieces && !pieces_done) AGN_TRY(split_act(h, Hl(l), h_pieces, fo, s, launches));
     }
     if (!h->use_head) {
       agn::SoftmaxArgs a{};
       a.Z = h->Z; a.m = m; a.C = h->C; a.ld = h->dims[L];
       a.yb = h->yb; a.slot_worker = sw; a.slot_t0 = st0; a.x_shard = h->direct_x ? h->S : 0;
-      a.dZ = h->dZ[L];
+      a.dZ = dZl(L);
       a.dZ_pieces = dz_pieces(L); a.dZ_plane = dz_plane(L);
       a.loss_parts = h->loss_parts; a.slot_commit = sc; a.lam = h->lam; a.step = i;
       a.flag = h->flag;
@@ -814,7 +835,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     have_pieces[L] = dz_pieces(L) != nullptr;   // by the softmax kernel
     auto ensure_pieces = [&](int l) -> Status {
       if (dz_pieces(l) && !have_pieces[l]) {
-        AGN_TRY(split_act(h, h->dZ[l], dz_pieces(l), h->dims[l], s, launches, dz_plane(l)));
+        AGN_TRY(split_act(h, dZl(l), dz_pieces(l), h->dims[l], s, launches, dz_plane(l)));
         have_pieces[l] = 1;
       }
       return Status::Ok();
@@ -822,7 +843,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     for (int l = L; l >= 2; --l) {
       if (l == L && h->use_head) continue;   // the head already wrote dZ_{L-1}
       const int fi = h->dims[l - 1], fo = h->dims[l];
-      const void* Hprev = h->H[l - 1];
+      const void* Hprev = Hl(l - 1);
       bf16* next_pieces = dz_pieces(l - 1);
       Launch k(h, AGN_K_BACKWARD_DX, 2.0 * s * m * fo * fi,
                (double)s * ((double)fo * fi * es + (double)m * fo * es +
@@ -830,10 +851,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
                launches);
       if (tc_layer(h, l) && (h->tc_mask & 2)) {
         AGN_TRY(ensure_pieces(l));
-        agn::TcArgs t = tc_args(h, sw, st0, i);
+        agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
         t.M = fi; t.N = m; t.K = fo;
         t.a_by_worker = 1;
-        t.out = h->dZ[l - 1]; t.ldo = fi; t.out_bstride = (int64_t)m * fi;
+        t.out = dZl(l - 1); t.ldo = fi; t.out_bstride = (int64_t)m * fi;
         t.mask = Hprev; t.mask_bstride = (int64_t)m * fi;
         t.out_pieces = next_pieces; t.out_plane = dz_plane(l - 1);
         const auto& mp = maps_of(l);
@@ -845,10 +866,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       } else {
         agn::GemmArgs g{};
         g.M = m; g.N = fi; g.K = fo;
-        g.a = h->dZ[l]; g.lda = fo; g.a_bstride = (int64_t)m * fo;
+        g.a = dZl(l); g.lda = fo; g.a_bstride = (int64_t)m * fo;
         g.b = W + h->woff[l - 1]; g.ldb = fi; g.b_bstride = h->P_pad; g.b_by_worker = 1;
         g.slot_worker = sw;
-        g.out = h->dZ[l - 1]; g.ldo = fi; g.out_bstride = (int64_t)m * fi;
+        g.out = dZl(l - 1); g.ldo = fi; g.out_bstride = (int64_t)m * fi;
         g.mask = Hprev; g.mask_bstride = (int64_t)m * fi;
         g.theta = h->rep; g.ld_param = h->P_pad;
         AGN_TRY(agn::simt_backward_dx<T>(g, s, h->stream));
@@ -860,7 +881,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     double tc_flops = 0.0, tc_bytes = 0.0;
     for (int l = L; l >= 1; --l) {
       const int fi = h->dims[l - 1], fo = h->dims[l];
-      const void* Hprev = l == 1 ? h->Xb : h->H[l - 1];
+      const void* Hprev = l == 1 ? h->Xb : Hl(l - 1);
       const double flops = 2.0 * s * m * fo * fi;
       const double bytes =
           (double)s * (((double)fo * fi + fo) * upd + (double)m * fo * es + (double)m * fi * es);
@@ -868,12 +889,12 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         AGN_TRY(ensure_pieces(l));
         if (h->tc_mask & 8) {   // the earlier one-tile-per-CTA kernel, layer by layer
           Launch k(h, AGN_K_BACKWARD_DW, flops, bytes, launches);
-          agn::TcArgs t = tc_args(h, sw, st0, i);
+          agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
           t.M = fi; t.N = fo; t.K = m;
           t.woff = h->woff[l - 1]; t.eta = eta;
           const auto& mp = h->tmaps[l - 1];
           AGN_TRY(agn::tc_backward_dw_tiled(mp.h_mn, mp.dz_mn, t, s, h->stream, h->split));
-          AGN_TRY(agn::bias_update(h->dZ[l], m, fo, (int64_t)m * fo, sw, h->rep, h->acc,
+          AGN_TRY(agn::bias_update(dZl(l), m, fo, (int64_t)m * fo, sw, h->rep, h->acc,
                                    h->rep_b, h->P_pad, h->boff[l - 1], eta, s, h->stream,
                                    h->split, h->piece_plane));
         } else {
@@ -898,7 +919,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       Launch k(h, AGN_K_BACKWARD_DW, flops, bytes, launches);
       if (l == L && h->use_head) {   // narrow output layer
         agn::HeadDwArgs d{};
-        d.H = Hprev; d.dZL = h->dZ[l]; d.slot_worker = sw;
+        d.H = Hprev; d.dZL = dZl(l); d.slot_worker = sw;
         d.theta = h->rep; d.acc = h->elide ? nullptr : h->acc; d.theta_b = h->rep_b;
         d.piece_plane = h->piece_plane;
         d.ld_param = h->P_pad; d.woff = h->woff[l - 1]; d.boff = h->boff[l - 1];
@@ -909,7 +930,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       } else {
         agn::GemmArgs g{};
         g.M = fo; g.N = fi; g.K = m;
-        g.a = h->dZ[l]; g.lda = fo; g.a_bstride = (int64_t)m * fo;
+        g.a = dZl(l); g.lda = fo; g.a_bstride = (int64_t)m * fo;
         g.b = Hprev; g.ldb = fi; g.b_bstride = (int64_t)m * fi;
         g.slot_worker = sw;
         g.theta = h->rep; g.acc = h->elide ? nullptr : h->acc; g.theta_bf16 = h->rep_b;
@@ -920,16 +941,27 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         AGN_TRY(agn::simt_backward_dw<T>(g, s, h->stream));
       }
     }
-    if (!tc_dw.empty()) {
+    if (!tc_dw.empty() && !(defer && acc_only)) {
       Launch k(h, AGN_K_BACKWARD_DW, tc_flops, tc_bytes, launches);
-      agn::TcArgs t = tc_args(h, sw, st0, i);
+      agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
       t.K = m; t.eta = eta;
+      if (defer) t.acc = nullptr;
       if (acc_only) {
         t.grad_out = h->acc; t.grad_add = i > 0;
       } else {
         t.acc_set = h->acc_first && i == 0;
         if (last_acc && wv.repulls > 0) t.slot_repull = h->plan_repull + wv.offset;
       }
+      AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
+                                  h->num_sms));
+    }
+    if (defer && (hi == h->hist - 1 || i == h->lam - 1)) {   // a_k of the kept steps
+      Launch k(h, AGN_K_BACKWARD_DW, tc_flops * (hi + 1), (double)s * h->P * (i > hi ? 8.0 : 4.0),
+               launches);
+      agn::TcArgs t = tc_args(h, sw, st0, i - hi, 0);
+      t.K = m;
+      t.hist_steps = hi + 1; t.z_step = n;
+      t.grad_out = h->acc; t.grad_add = i > hi;
       AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
                                   h->num_sms));
     }
@@ -1448,13 +1480,22 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     else AGN_TRY(dalloc(h, &h->Xb_alt, (size_t)(n * m * d0) * es));
   }
   AGN_TRY(dalloc_t(h, &h->yb, (size_t)(n * (h->direct_x ? h->S + m : m))));
+  if (h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam && !h->elide &&
+      h->lam > 1 && m <= kHistMaxBatch && n * h->P * 4 > agn::kTcRedAccBytes) {
+    // no more than twice the accumulators' memory
+    int64_t per = h->ldz_out;
+    for (int l = 1; l < h->L; ++l) per += 2 * dims[l];
+    h->hist = (int)std::min<int64_t>(std::min(h->lam, kHistMaxSteps),
+                                     std::max<int64_t>(1, 8 * h->P / (2 * m * per)));
+  }
+  const int64_t nh = n * h->hist;
   h->H.assign(h->L, nullptr);
-  for (int l = 1; l < h->L; ++l) AGN_TRY(dalloc(h, &h->H[l], (size_t)(n * m * dims[l]) * es));
+  for (int l = 1; l < h->L; ++l) AGN_TRY(dalloc(h, &h->H[l], (size_t)(nh * m * dims[l]) * es));
   AGN_TRY(dalloc_t(h, &h->Z, (size_t)(n * m * dims[h->L])));
   h->dZ.assign(h->L + 1, nullptr);
-  for (int l = 1; l < h->L; ++l) AGN_TRY(dalloc(h, &h->dZ[l], (size_t)(n * m * dims[l]) * es));
-  AGN_TRY(dalloc(h, &h->dZ[h->L], (size_t)(n * m * h->ldz_out) * es));
-  AGN_TRY_CUDA(cudaMemset(h->dZ[h->L], 0, (size_t)(n * m * h->ldz_out) * es));
+  for (int l = 1; l < h->L; ++l) AGN_TRY(dalloc(h, &h->dZ[l], (size_t)(nh * m * dims[l]) * es));
+  AGN_TRY(dalloc(h, &h->dZ[h->L], (size_t)(nh * m * h->ldz_out) * es));
+  AGN_TRY_CUDA(cudaMemset(h->dZ[h->L], 0, (size_t)(nh * m * h->ldz_out) * es));
   AGN_TRY(dalloc_t(h, &h->flag, 2));
   AGN_TRY(dalloc_t(h, &h->ce_partial, (size_t)(n * ceil_div(m, agn::kHeadSamples))));
   AGN_TRY(dalloc_t(h, &h->head_counter, (size_t)n));

@@ -214,7 +214,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // slot's minibatch row (tile rows past m belong to the next rows of the
   // shard; their accumulator columns are never stored)
   const bool b_direct = !kBMN && args.x_b_direct && args.x_shard > 0;
-  const int b_z = b_direct ? worker : args.b_by_worker ? worker : slot;
+  const int b_z = b_direct || args.b_by_worker ? worker : args.z0 + slot;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {

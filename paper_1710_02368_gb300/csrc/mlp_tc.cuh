@@ -50,6 +50,12 @@ struct TcArgs {
   // step.  grad_add: add it to what is there instead.
   float* grad_out;
   int grad_add;
+  // dW: the operands of hist_steps (0 or 1: one) consecutive local steps
+  // beginning with `step`, kept z_step batches apart: their gradients summed
+  int hist_steps, z_step;
+  // batch coordinate of slot 0 in the activation maps (forward and dX: B; dW:
+  // both operands), the local step's place in the kept history
+  int z0;
   // Forward of the last hidden layer with the output layer fused into its
   // epilogue (tc_forward_head): the d_L <= 16 logits of every sample from the
   // CTAs' partial sums over their 128 features, softmax cross-entropy, dZ_L and
@@ -152,6 +158,10 @@ struct DwLayerMaps {
   int64_t woff, boff;
   int a_direct = 0;   // h_mn is a padded-shard map (layer 1; args.x_shard > 0)
 };
+// Accumulators (bytes) above which a wave streams them from DRAM: a dW launch
+// then takes a_k through the parameter ring, not by L2 adds, or, in bf16 mode,
+// leaves it to one launch over several local steps' operands.
+constexpr int64_t kTcRedAccBytes = 64ll << 20;
 // dW with the local step and accumulation of the weights and biases of all
 // `layers` in one persistent launch (mlp_tc_dw.cu, grid min(tiles, num_sms)).
 // args supplies slot_worker, err, theta, acc, theta_b, ld_param, piece_plane,

@@ -184,11 +184,15 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int T = B.total_tiles;
-  // a slot whose replica nothing reads before its next pull: a_k only
+  // a slot whose replica nothing reads before its next pull: a_k only (or,
+  // where this launch keeps no a_k, nothing)
   auto acc_only = [&](int slot) -> bool {
-    return kMode == kDwUpdRed && args.slot_repull && AGN_LD(args.slot_repull + slot) != 0;
+    return (kMode == kDwUpdRed || kMode == kDwUpd) && args.slot_repull &&
+           AGN_LD(args.slot_repull + slot) != 0;
   };
-  const int KT = (args.K + kBK - 1) / kBK;
+  // k steps of one local step's minibatch, and of the whole launch
+  const int KTs = (args.K + kBK - 1) / kBK;
+  const int KT = KTs * max(1, args.hist_steps);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -248,9 +252,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         // layer 1's A from the padded shards: the worker's shard at the slot's
         // minibatch row (samples past m multiply dZ rows that are zero fill)
         const bool a_direct = B.layer[ti.layer].a_direct && args.x_shard > 0;
-        const int a_row0 =
-            a_direct ? (int)batch_row0(args.slot_t0, ti.slot, args.step, args.K, args.x_shard) : 0;
-        const int a_z = a_direct ? AGN_LD(args.slot_worker + ti.slot) : ti.slot;
+        int a_row0 = 0, b_z = 0, a_z = 0;
         if (throttle && itp > 0 && *chunk_tiles < itp) {
           const uint64_t t0 = tc::globaltimer_ns();
           while (*chunk_tiles < itp) {
@@ -262,7 +264,13 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           }
           if (!ok) break;
         }
-        for (int kt = 0; kt < KT; ++kt) {
+        for (int kt = 0, kr = 0, st = 0; kt < KT; ++kt) {
+          if (kr == 0) {   // the next local step's operands
+            b_z = args.z0 + st * args.z_step + ti.slot;
+            a_z = a_direct ? AGN_LD(args.slot_worker + ti.slot) : b_z;
+            if (a_direct)
+              a_row0 = (int)batch_row0(args.slot_t0, ti.slot, args.step + st, args.K, args.x_shard);
+          }
           const int s = ml % kStages;
           if (ml >= kStages &&
               !tc::wait_or_abort(&empty[s], ((ml / kStages) - 1) & 1, abort_flag, kWaitNs)) {
@@ -277,24 +285,28 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
             uint8_t* sa = sa0 + p * kABytes;
             uint8_t* sb = sb0 + p * Cfg::kBBytes;
             if (kSplit == 1) {
-              tc::tma_load_3d(sa, tmA, &full[s], ti.m_tile * 128, kt * kBK + a_row0, a_z);
-              tc::tma_load_3d(sa + kBox, tmA, &full[s], ti.m_tile * 128 + 64, kt * kBK + a_row0,
+              tc::tma_load_3d(sa, tmA, &full[s], ti.m_tile * 128, kr * kBK + a_row0, a_z);
+              tc::tma_load_3d(sa + kBox, tmA, &full[s], ti.m_tile * 128 + 64, kr * kBK + a_row0,
                               a_z);
   #pragma unroll
               for (int c = 0; c < BN / 64; ++c)
-                tc::tma_load_3d(sb + c * kBox, tmB, &full[s], ti.n_tile * BN + c * 64, kt * kBK,
-                                ti.slot);
+                tc::tma_load_3d(sb + c * kBox, tmB, &full[s], ti.n_tile * BN + c * 64, kr * kBK,
+                                b_z);
             } else {
-              tc::tma_load_4d(sa, tmA, &full[s], ti.m_tile * 128, kt * kBK + a_row0, a_z, p);
-              tc::tma_load_4d(sa + kBox, tmA, &full[s], ti.m_tile * 128 + 64, kt * kBK + a_row0,
+              tc::tma_load_4d(sa, tmA, &full[s], ti.m_tile * 128, kr * kBK + a_row0, a_z, p);
+              tc::tma_load_4d(sa + kBox, tmA, &full[s], ti.m_tile * 128 + 64, kr * kBK + a_row0,
                               a_z, p);
   #pragma unroll
               for (int c = 0; c < BN / 64; ++c)
-                tc::tma_load_4d(sb + c * kBox, tmB, &full[s], ti.n_tile * BN + c * 64, kt * kBK,
-                                ti.slot, p);
+                tc::tma_load_4d(sb + c * kBox, tmB, &full[s], ti.n_tile * BN + c * 64, kr * kBK,
+                                b_z, p);
             }
           }
           ++ml;
+          if (++kr == KTs) {
+            kr = 0;
+            ++st;
+          }
         }
       }
       if (!ok) {
@@ -470,8 +482,9 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       float* theta = args.theta + rbase;
       float* acc = kAcc ? args.acc + rbase : nullptr;
       bf16* tb = args.theta_b ? args.theta_b + rbase : nullptr;   // bf16 mode only
-      const int nch = min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
       const bool grad_only = kGrad || acc_only(ti.slot);
+      const int nch = grad_only && kMode == kDwUpd
+                          ? 0 : min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
       const bool grad_add = kGrad ? args.grad_add != 0 : !args.acc_set;
       for (int c = 0; c < nch; ++c) {
         const int r = ch % kRing;
@@ -649,11 +662,10 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     // through the ring (large waves, which stream theta_k and a_k from DRAM
     // at the copy bandwidth: there the L2's adds slowed the stream by 4 %;
     // and always with args.acc_ring)
-    constexpr int64_t kRedAccBytes = 64ll << 20;
     // (a first local step only stores a_k, and slots about to pull only add to
     // it: the ring stays with theta_k)
     const bool ring = !args.acc_set && !args.slot_repull &&
-                      (args.acc_ring || acc_bytes > kRedAccBytes);
+                      (args.acc_ring || acc_bytes > kTcRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
