@@ -18,7 +18,9 @@
 #include <cstdint>
 #include <new>
 #include <cstring>
+#include <exception>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -201,6 +203,7 @@ struct agn_handle {
   std::vector<void*> allocs;
   // device state
   float* theta_c = nullptr;   // [P_pad]
+  float* flat = nullptr;      // [P]: parameters packed for a read (read_params)
   float* rep = nullptr;       // [n][P_pad] fp32 master replicas
   float* acc = nullptr;       // [n][P_pad] accumulators (sum of raw gradients)
   bf16* rep_b = nullptr;      // [n][P_pad] bf16 working copies (bf16 mode)
@@ -1431,6 +1434,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   const size_t es = elem_size(h);
   const int64_t n = h->n, m = h->m;
   AGN_TRY(dalloc_t(h, &h->theta_c, (size_t)h->P_pad));
+  AGN_TRY(dalloc_t(h, &h->flat, (size_t)h->P));
   AGN_TRY(dalloc_t(h, &h->rep, (size_t)(n * h->P_pad)));
   AGN_TRY(dalloc_t(h, &h->acc, (size_t)(n * h->P_pad)));
   if (h->prec == AGN_PREC_BF16) AGN_TRY(dalloc_t(h, &h->rep_b, (size_t)(n * h->P_pad)));
@@ -1633,19 +1637,46 @@ Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int6
   return Status::Ok();
 }
 
+// Write one byte of every page of a caller's output buffer from a few threads.
+// A fresh buffer's pages are mapped (and zeroed by the system) on first touch,
+// which one thread, or the copy itself, does at 20-25 GB/s: 84 MB took 3.3 ms
+// with the copy alone and the copy into touched pages 0.46 ms.
+void touch_pages(void* p, size_t bytes) {
+  constexpr size_t kMin = 4 << 20;   // below it a thread costs more than it saves
+  const size_t parts = std::min<size_t>({8, bytes / kMin, std::thread::hardware_concurrency()});
+  if (parts < 2) return;
+  volatile char* c = static_cast<volatile char*>(p);
+  auto work = [=](size_t i) {
+    const size_t lo = bytes / parts * i, hi = i + 1 == parts ? bytes : bytes / parts * (i + 1);
+    for (size_t o = lo; o < hi; o += 4096) c[o] = 0;
+  };
+  std::vector<std::thread> ts;
+  try {
+    ts.reserve(parts);
+    for (size_t i = 1; i < parts; ++i) ts.emplace_back(work, i);
+  } catch (const std::exception&) {   // no more threads: the copy touches the rest
+  }
+  work(0);
+  for (auto& t : ts) t.join();
+}
+
+// A replica's (or theta~'s) parameters in the ABI's flat order: packed on the
+// device (the device pads widths and aligns tensors), then one copy straight
+// into the caller's buffer while a few threads map its pages.  (Before: the
+// padded vector into a host vector, then per-row copies: 10.7 ms for 84 MB.)
 Status read_params(agn_handle* h, const float* dev, float* out, int64_t cap) {
   if (!out || cap < h->P) return Status::Err(AGN_E_INVALID, "output buffer shorter than P");
-  std::vector<float> tpad((size_t)h->P_pad);
+  std::vector<agn::PackLayer> layers;
+  for (int l = 0; l < h->L; ++l)
+    layers.push_back({h->woff_flat[l], h->boff_flat[l], h->woff[l], h->boff[l], h->udims[l],
+                      h->udims[l + 1], h->dims[l]});
+  AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build only
+  AGN_TRY(agn::pack_params(dev, h->flat, layers.data(), h->L, h->stream));
+  touch_pages(out, (size_t)h->P * sizeof(float));
+  AGN_TRY_CUDA(cudaMemcpyAsync(out, h->flat, (size_t)h->P * sizeof(float), cudaMemcpyDeviceToHost,
+                               h->stream));
   AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
-  AGN_TRY_CUDA(cudaMemcpy(tpad.data(), dev, tpad.size() * sizeof(float), cudaMemcpyDeviceToHost));
-  for (int l = 0; l < h->L; ++l) {
-    const int64_t fi = h->udims[l], fo = h->udims[l + 1], ld = h->dims[l];
-    for (int64_t f = 0; f < fo; ++f)
-      std::memcpy(out + h->woff_flat[l] + f * fi, &tpad[h->woff[l] + f * ld],
-                  (size_t)fi * sizeof(float));
-    std::memcpy(out + h->boff_flat[l], &tpad[h->boff[l]], (size_t)fo * sizeof(float));
-  }
-  return Status::Ok();
+  return agn::bounds_collect(h->stream);
 }
 
 Status read_commit_array(agn_handle* h, const float* dev, float* out, int64_t cap) {
@@ -1844,16 +1875,24 @@ int agn_run(agn_handle* h, int32_t n_commits, const int32_t* worker, const int32
 int agn_central(agn_handle* h, float* out, int64_t cap) {
   if (!h) return fail(nullptr, AGN_E_INVALID, "null handle");
   DeviceGuard g(h->device);
-  Status s = read_params(h, h->theta_c, out, cap);
-  return s.ok() ? AGN_OK : fail(h, s);
+  try {
+    Status s = read_params(h, h->theta_c, out, cap);
+    return s.ok() ? AGN_OK : fail(h, s);
+  } catch (const std::bad_alloc&) {
+    return fail(h, AGN_E_OOM, "host allocation failed");
+  }
 }
 
 int agn_replica(agn_handle* h, int32_t k, float* out, int64_t cap) {
   if (!h) return fail(nullptr, AGN_E_INVALID, "null handle");
   if (k < 0 || k >= h->n) return fail(h, AGN_E_INVALID, "replica index out of range");
   DeviceGuard g(h->device);
-  Status s = read_params(h, h->rep + (int64_t)k * h->P_pad, out, cap);
-  return s.ok() ? AGN_OK : fail(h, s);
+  try {
+    Status s = read_params(h, h->rep + (int64_t)k * h->P_pad, out, cap);
+    return s.ok() ? AGN_OK : fail(h, s);
+  } catch (const std::bad_alloc&) {
+    return fail(h, AGN_E_OOM, "host allocation failed");
+  }
 }
 
 int agn_loss(agn_handle* h, float* out, int64_t cap) {

@@ -357,7 +357,41 @@ __global__ void reduce_losses_kernel(const float* __restrict__ parts, int lambda
   AGN_ST(loss + c, s / (float)lambda);
 }
 
+// One layer's weights and biases from the device layout to the flat one
+// (rows of fi, unpadded).  A block copies whole rows, coalesced on both sides.
+__global__ void __launch_bounds__(kThreads)
+pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayer L) {
+  pdl_begin();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kWarps = kThreads / 32;
+  for (int64_t f = (int64_t)blockIdx.x * kWarps + warp; f < L.fo; f += (int64_t)gridDim.x * kWarps) {
+    const float* s = src + L.woff + f * L.ld;
+    float* d = dst + L.woff_flat + f * L.fi;
+    for (int k0 = lane; k0 < L.fi; k0 += 32 * 8) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k0 + 32 * u < L.fi) v[u] = AGN_LD(s + k0 + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k0 + 32 * u < L.fi) AGN_ST(d + k0 + 32 * u, v[u]);
+    }
+    if (lane == 0) AGN_ST(dst + L.boff_flat + f, AGN_LD(src + L.boff + f));
+  }
+}
+
 }  // namespace
+
+Status pack_params(const float* src, float* dst, const PackLayer* layers, int n_layers,
+                   cudaStream_t st) {
+  for (int l = 0; l < n_layers; ++l) {
+    const int grid = (int)std::min<int64_t>(ceil_div(layers[l].fo, kThreads / 32), 152 * 8);
+    auto kf = pack_kernel;
+    AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, 0, st, src, dst, layers[l]));
+  }
+  AGN_TRY_CUDA(cudaGetLastError());
+  return Status::Ok();
+}
 
 Status pull_replicas(const float* theta_c, float* replicas, bf16* replicas_bf16, int64_t P,
                      int64_t ld, const int* workers, int count, cudaStream_t st,

@@ -169,6 +169,15 @@ Status temporal_efficiency(const double* ta, const double* fa, int64_t na, const
 Status pull_replicas(const float* theta_c, float* replicas, bf16* replicas_bf16, int64_t P,
                      int64_t ld, const int* workers, int count, cudaStream_t st,
                      int64_t piece_plane = 0, float* snapshot = nullptr);
+// One layer of pack_params: offsets of W_l and b_l in the flat and in the
+// device layout, their inputs, outputs and the device's row length.
+struct PackLayer {
+  int64_t woff_flat, boff_flat, woff, boff;
+  int fi, fo, ld;
+};
+// dst (flat order, unpadded) = the parameters at src (device layout).
+Status pack_params(const float* src, float* dst, const PackLayer* layers, int n_layers,
+                   cudaStream_t st);
 // loss[c] = mean_i parts[c * lambda + i] for c < count.
 // loss[c] = (1/lambda) sum_i sum_q parts[(c lambda + i) q_per + q] (fixed order).
 Status reduce_losses(const float* parts, int lambda, int q_per, int count, float* loss,

@@ -1,0 +1,52 @@
+"""A standalone call writes a replica once, at its worker's last pull
+(csrc/common.cuh, LastPulls): random pull lists with repeats within a commit and
+across commits, against the float32 oracle that performs every pull in order;
+both entry points, with and without bf16 copies."""
+
+import numpy as np
+import pytest
+
+import agn_inputs as I  # noqa: F401  (path set-up)
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import __graft_entry__ as g
+    g.build()
+    import torch
+    import paper_1710_02368_gb300 as agn
+    return agn, torch, torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("P,n,C,most", [(1, 1, 1, 3), (1003, 3, 7, 4), (4099, 40, 33, 9),
+                                        (260, 300, 5, 200)])
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("low", [False, True])
+def test_last_pull_wins(env, P, n, C, most, noalloc, low):
+    agn, torch, dev = env
+    rng = np.random.default_rng(P + C)
+    ld = (P + 3) // 4 * 4
+    theta = torch.empty(P, device=dev)
+    acc = torch.empty(n, ld, device=dev)
+    reps = torch.full((n, ld), 5.0, device=dev)
+    repb = torch.full((n, ld), 5.0, dtype=torch.bfloat16, device=dev) if low else None
+    agn.agn_fill_commit_inputs(theta, acc, None, P, ld, n, 11)
+    th_h, acc_h = theta.cpu().numpy().copy(), acc[:, :P].cpu().numpy().copy()
+    order = rng.integers(0, n, C).tolist()
+    pulls = [rng.integers(0, n, rng.integers(0, most + 1)).tolist() for _ in range(C)]
+    offs = np.cumsum([0] + [len(p) for p in pulls])
+    call = agn.agn_commit_pull_noalloc if noalloc else agn.agn_commit_pull
+    call(theta, acc, reps, repb, P, ld, n, order, offs, [p for ps in pulls for p in ps], 0.01, 10)
+    torch.cuda.synchronize()
+    t, _, r, _ = O.commit_pull_fp32(th_h, {k: acc_h[k] for k in range(n)}, order, pulls, 0.01, 10)
+    assert np.array_equal(theta.cpu().numpy(), t)
+    pulled = {p for ps in pulls for p in ps}
+    for k in range(n):
+        got = reps[k, :P].cpu()
+        want = torch.from_numpy(r[k]) if k in pulled else torch.full((P,), 5.0)
+        assert torch.equal(got, want), k
+        if low:
+            assert torch.equal(repb[k, :P].cpu(), want.to(torch.bfloat16)), k
