@@ -55,21 +55,20 @@ extern "C" {
 #define AGN_DIST_UNIFORM 0     /* x ~ U[0,1)^d0 */
 #define AGN_DIST_NORMAL 1      /* x ~ N(0,1)^d0 */
 
-#define AGN_GEMM_AUTO 0        /* tcgen05 for every net with a hidden layer
-                                  (any widths: the device pads d_0 .. d_{L-1}
-                                  to multiples of 8 with zeros that stay zero;
-                                  any batch), else CUDA cores               */
+#define AGN_GEMM_AUTO 0        /* tcgen05 for nets with a hidden layer and
+                                  d_0 .. d_{L-1} multiples of 8 (any batch),
+                                  else CUDA cores                           */
 #define AGN_GEMM_SIMT 1        /* CUDA-core GEMM kernels only                */
 #define AGN_GEMM_TCGEN05 2     /* tcgen05/TMEM GEMMs in either precision (fp32
                                   mode feeds every fp32 operand as three exact
                                   bf16 pieces, fp32 accumulation); needs at
                                   least one hidden layer, batch <= 256 and
                                   d_0 .. d_{L-1} multiples of 8 (else
-                                  AGN_E_UNSUPPORTED).  A narrow output layer's
-                                  (d_L <= 16) forward, softmax-CE and dX run
-                                  on CUDA cores and its dW joins the
-                                  tensor-core dW launch; a wider one is a
-                                  tensor-core layer too */
+                                  AGN_E_UNSUPPORTED).  The output layer's
+                                  forward, softmax-CE and dX run on CUDA cores
+                                  or in the last hidden layer's forward; a
+                                  narrow one's dW (d_L <= 16) joins the
+                                  tensor-core dW launch                     */
 
 /* Local optimizers (agn_options.local_optimizer) */
 #define AGN_OPT_SGD 0

@@ -159,9 +159,8 @@ Status bounds_collect(cudaStream_t st) {
 #endif
 
 struct agn_handle {
-  // problem: the caller's layer dims and the device's (d_0 .. d_{L-1} padded to
-  // multiples of 8 on the tensor-core path, see create)
-  std::vector<int> udims, dims;
+  // problem
+  std::vector<int> dims;
   int L = 0, n = 0, lam = 0;
   double eta = 0.0;
   uint64_t seed = 0;
@@ -193,7 +192,6 @@ struct agn_handle {
   int64_t N = 0, S = 0;
   std::vector<int> tdims;
   int64_t P = 0, P_pad = 0;
-  int C = 0;                  // classes d_L
   std::vector<int64_t> woff, boff, woff_flat, boff_flat;   // per layer (index l-1)
   // CUDA
   int device = 0;
@@ -242,9 +240,6 @@ struct agn_handle {
   std::vector<bf16*> dZp;         // pieces of dZ_l, l = 1..L-1: [3][n][m][d_l]
   // output layer fused into one kernel (forward + softmax-CE + dX) when narrow
   bool use_head = false;
-  // a wide output layer (!use_head) on the tensor cores: dims[L] is then its
-  // classes padded to a multiple of 8
-  bool out_tc = false;
   // the output layer's dW runs as tiles of the persistent tensor-core dW
   // launch: dZ_L padded to ldz_out columns (zero beyond d_L) with its pieces,
   // and H_{L-1}'s pieces kept
@@ -427,9 +422,8 @@ void collect_profile(agn_handle* h) {
   h->ev_used = 0;
 }
 
-// Layer l (1-based) runs on the tensor cores: a hidden layer, or an output
-// layer too wide for the output-layer kernels.
-bool tc_layer(const agn_handle* h, int l) { return h->use_tc && (l < h->L || h->out_tc); }
+// Layer l (1-based) runs on the tensor cores: a hidden layer.
+bool tc_layer(const agn_handle* h, int l) { return h->use_tc && l < h->L; }
 
 agn::TcArgs tc_args(agn_handle* h, const int* sw, const long long* st0, int step, int z0) {
   agn::TcArgs t{};
@@ -552,25 +546,6 @@ Status build_tc_maps(agn_handle* h) {
                                   128, 32));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.acc, h->acc + h->woff[L - 1], fi, fo, n, fi, h->P_pad,
                                   128, 32));
-    if (h->out_tc) {   // and its forward and dX
-      if (h->split) {
-        constexpr uint32_t bk = agn::kTcSplitBK;
-        const float* W = h->rep + h->woff[L - 1];
-        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, bk, 128, true));
-        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k256, W, fi, fo, n, fi, h->P_pad, bk, 128));
-        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 128, bk));
-        AGN_TRY(agn::make_tmap_bf16_4d(&mp.h_k, h->Hs[L - 1], fi, m, n, fi, (uint64_t)m * fi,
-                                       (uint64_t)n * m * fi, bk, bn));
-        AGN_TRY(agn::make_tmap_bf16_4d(&mp.dz_k, h->dZp[L], lz, m, n, lz, (uint64_t)m * lz,
-                                       (uint64_t)n * m * lz, bk, bn));
-      } else {
-        const bf16* W = h->rep_b + h->woff[L - 1];
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_k, W, fi, fo, n, fi, h->P_pad, 64, 128));
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.w_mn, W, fi, fo, n, fi, h->P_pad, 64, 64));
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.h_k, h->H[L - 1], fi, m, nh, fi, (uint64_t)m * fi, 64, bn));
-        AGN_TRY(agn::make_tmap_bf16_3d(&mp.dz_k, h->dZ[L], lz, m, nh, lz, (uint64_t)m * lz, 64, bn));
-      }
-    }
     if (h->split) {
       const bf16* Hp = h->Hs[L - 1];
       AGN_TRY(agn::make_tmap_bf16_4d(&mp.h_mn32, Hp, fi, m, n, fi, (uint64_t)m * fi,
@@ -677,7 +652,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     const bool alt = h->early_gather && h->gparity;
     const agn_handle::LayerMaps& l1 = alt ? h->l1_alt : h->tmaps.empty() ? h->l1_alt : h->tmaps[0];
     auto maps_of = [&](int l) -> const agn_handle::LayerMaps& {
-      return l == 1 ? l1 : l == L ? h->out_maps : h->tmaps[l - 1];
+      return l == 1 ? l1 : h->tmaps[l - 1];
     };
     if (!h->direct_x) {
       // fp32 mode with the early gather: the fp32 rows are not read by the
@@ -799,10 +774,9 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
           t.M = fo; t.N = m; t.K = fi;
           t.a_by_worker = 1;
-          t.out = l == L ? static_cast<void*>(h->Z) : Hl(l);
-          t.out_f32 = l == L;
+          t.out = Hl(l);
           t.ldo = fo; t.out_bstride = (int64_t)m * fo;
-          t.relu = l < L; t.boff = h->boff[l - 1];
+          t.relu = 1; t.boff = h->boff[l - 1];
           t.out_pieces = h_pieces; t.out_plane = (int64_t)n * m * fo;
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
@@ -821,21 +795,19 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     }
     if (!h->use_head) {
       agn::SoftmaxArgs a{};
-      a.Z = h->Z; a.m = m; a.C = h->C; a.ld = h->dims[L];
+      a.Z = h->Z; a.m = m; a.C = h->dims[L];
       a.yb = h->yb; a.slot_worker = sw; a.slot_t0 = st0; a.x_shard = h->direct_x ? h->S : 0;
       a.dZ = dZl(L);
-      a.dZ_pieces = dz_pieces(L); a.dZ_plane = dz_plane(L);
       a.loss_parts = h->loss_parts; a.slot_commit = sc; a.lam = h->lam; a.step = i;
       a.flag = h->flag;
       Launch k(h, AGN_K_SOFTMAX, 0.0,
-               (double)s * m * (h->C * (4.0 + es + (a.dZ_pieces ? 6.0 : 0.0)) + 4.0), launches);
+               (double)s * m * (h->dims[L] * (4.0 + es) + 4.0), launches);
       AGN_TRY(agn::softmax_xent<T>(a, s, h->stream));
     }
     // backward: dX for l = L..2 (each reads W_l before its update), then the
     // weight and bias gradients with the local step of every layer
     std::vector<char> have_pieces(L + 1, 0);   // pieces of dZ_l written by its producer
     if (L > 1) have_pieces[L - 1] = dz_ready;
-    have_pieces[L] = dz_pieces(L) != nullptr;   // by the softmax kernel
     auto ensure_pieces = [&](int l) -> Status {
       if (dz_pieces(l) && !have_pieces[l]) {
         AGN_TRY(split_act(h, dZl(l), dz_pieces(l), h->dims[l], s, launches, dz_plane(l)));
@@ -1261,18 +1233,6 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
   return bounds;
 }
 
-// Host rows of `width` elements into device rows of `ld` >= width, zero beyond.
-Status upload_rows(void* dst, const void* src, int64_t rows, int64_t width, int64_t ld, size_t es) {
-  if (width == ld) {
-    AGN_TRY_CUDA(cudaMemcpy(dst, src, (size_t)(rows * ld) * es, cudaMemcpyHostToDevice));
-    return Status::Ok();
-  }
-  AGN_TRY_CUDA(cudaMemset(dst, 0, (size_t)(rows * ld) * es));
-  AGN_TRY_CUDA(cudaMemcpy2D(dst, (size_t)ld * es, src, (size_t)width * es, (size_t)width * es,
-                            (size_t)rows, cudaMemcpyHostToDevice));
-  return Status::Ok();
-}
-
 Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_workers, int32_t lambda,
               double eta, uint64_t seed, const agn_options& o) {
   if (!dims || n_dims < 2) return Status::Err(AGN_E_INVALID, "need at least two layer dims");
@@ -1310,9 +1270,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   if (o.elide_accumulator && (o.tc_mask & 8))
     return Status::Err(AGN_E_UNSUPPORTED,
                        "the one-tile-per-CTA dW kernel (tc_mask bit 3) keeps the accumulator");
-  h->udims.assign(dims, dims + n_dims);
+  h->dims.assign(dims, dims + n_dims);
   h->L = n_dims - 1;
-  h->C = dims[h->L];
   h->n = n_workers;
   h->lam = lambda;
   h->eta = eta;
@@ -1344,33 +1303,19 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   // tcgen05 path: a hidden layer and every TMA row 16-byte aligned.  bf16 mode
   // feeds bf16 operands; fp32 mode feeds each fp32 operand as three exact bf16
   // pieces (split mode).
-  bool tc_ok = h->m <= 256 && h->L >= 2;
+  bool tc_ok = h->L >= 2;
   for (int l = 0; l < h->L; ++l) tc_ok = tc_ok && dims[l] % 8 == 0;
-  if (o.gemm == AGN_GEMM_TCGEN05 && !tc_ok)
+  if (o.gemm == AGN_GEMM_TCGEN05 && !(tc_ok && h->m <= 256))
     return Status::Err(AGN_E_UNSUPPORTED,
                        "tcgen05 GEMMs need batch <= 256, at least one hidden layer "
                        "and d_0 .. d_{L-1} multiples of 8");
-  h->use_tc = h->L >= 2 && o.gemm != AGN_GEMM_SIMT;
+  h->use_tc = tc_ok && o.gemm != AGN_GEMM_SIMT;
   h->split = h->use_tc && h->prec == AGN_PREC_FP32;
   h->tc_mask = (o.tc_mask & 7) == 0 ? (o.tc_mask | 7) : o.tc_mask;
-  // Device dims.  The tensor-core path pads d_0 .. d_{L-1} to multiples of 8
-  // with inputs, features and weights that are zero and stay zero: a padded
-  // feature's pre-activation and gradient are zero, and so are the gradients
-  // of the weights into and out of it (SGD, Adam and the commits leave a zero
-  // with a zero gradient unchanged).  Every size gains over the CUDA-core
-  // kernels, us per local step of either: 3-5-2 17.0 / 18.4, 37-65-13-7 at 5
-  // workers 30 / 38, 613-301-150-26 (m = 100, 8 workers) 64 / 170,
-  // 784-1000-1000-10 (m = 512, 4 workers) 178 / 888.
-  h->dims = h->udims;
-  if (h->use_tc)
-    for (int l = 0; l < h->L; ++l) h->dims[l] = (int)round_up(dims[l], 8);
-  const int dl1 = h->dims[h->L - 1];
-  h->use_head = h->prec == AGN_PREC_BF16 ? agn::head_fits<bf16>(dl1, h->C)
-                                         : agn::head_fits<float>(dl1, h->C);
-  h->out_tc = h->use_tc && !h->use_head && (h->tc_mask & 7) == 7 && !(h->tc_mask & 8);
-  if (h->out_tc) h->dims[h->L] = (int)round_up(h->C, 8);
-  // parameter layouts: flat (the ABI's order, the caller's dims) and the
-  // device's (the device dims, 64-element aligned tensors)
+  h->use_head = h->prec == AGN_PREC_BF16 ? agn::head_fits<bf16>(dims[h->L - 1], dims[h->L])
+                                         : agn::head_fits<float>(dims[h->L - 1], dims[h->L]);
+  // parameter layouts: flat (the ABI's order) and padded (device, 64-element
+  // aligned tensors)
   int64_t off = 0, offp = 0;
   for (int l = 1; l <= h->L; ++l) {
     const int64_t fi = dims[l - 1], fo = dims[l];
@@ -1379,9 +1324,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     off += fo * fi + fo;
     offp = round_up(offp, 64);
     h->woff.push_back(offp);
-    offp = round_up(offp + (int64_t)h->dims[l] * h->dims[l - 1], 64);
+    offp = round_up(offp + fo * fi, 64);
     h->boff.push_back(offp);
-    offp += h->dims[l];
+    offp += fo;
   }
   h->P = off;
   h->P_pad = round_up(offp, 64);
@@ -1401,36 +1346,34 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   AGN_TRY_CUDA(cudaEventCreate(&h->ev1));
 
   // host inputs
-  const int u0 = dims[0];
-  h->hX.resize((size_t)h->N * u0);
+  const int d0 = dims[0];
+  h->hX.resize((size_t)h->N * d0);
   h->hy.resize((size_t)h->N);
   h->htheta0.resize((size_t)h->P);
   if (o.x_init) std::memcpy(h->hX.data(), o.x_init, h->hX.size() * sizeof(float));
-  else agn::gen_dataset(seed, u0, h->N, h->dist, h->hX.data());
+  else agn::gen_dataset(seed, d0, h->N, h->dist, h->hX.data());
   if (o.y_init) {
     std::memcpy(h->hy.data(), o.y_init, h->hy.size() * sizeof(int32_t));
     for (int32_t v : h->hy)
       if (v < 0 || v >= dims[n_dims - 1]) return Status::Err(AGN_E_INVALID, "label out of range");
   } else {
     auto Ws = agn::gen_teacher(seed, h->tdims);
-    agn::gen_teacher_labels(h->hX.data(), h->N, u0, h->dist, h->tdims, Ws, h->hy.data());
+    agn::gen_teacher_labels(h->hX.data(), h->N, d0, h->dist, h->tdims, Ws, h->hy.data());
   }
   if (o.theta_init) std::memcpy(h->htheta0.data(), o.theta_init, h->htheta0.size() * sizeof(float));
-  else agn::gen_init(seed, h->udims, h->htheta0.data());
+  else agn::gen_init(seed, h->dims, h->htheta0.data());
   std::vector<float> hXe;
   std::vector<int32_t> hye;
   if (o.n_eval > 0) {   // held-out rows of the same generator, labelled by the same teacher
     h->n_eval = o.n_eval;
-    hXe.resize((size_t)(o.n_eval * u0));
+    hXe.resize((size_t)(o.n_eval * d0));
     hye.resize((size_t)o.n_eval);
-    agn::gen_dataset_rows(seed, u0, h->N, o.n_eval, h->dist, hXe.data());
+    agn::gen_dataset_rows(seed, d0, h->N, o.n_eval, h->dist, hXe.data());
     auto Ws = agn::gen_teacher(seed, h->tdims);
-    agn::gen_teacher_labels(hXe.data(), o.n_eval, u0, h->dist, h->tdims, Ws, hye.data());
+    agn::gen_teacher_labels(hXe.data(), o.n_eval, d0, h->dist, h->tdims, Ws, hye.data());
   }
 
-  // device buffers (the device dims from here on)
-  dims = h->dims.data();
-  const int d0 = dims[0];
+  // device buffers
   const size_t es = elem_size(h);
   const int64_t n = h->n, m = h->m;
   AGN_TRY(dalloc_t(h, &h->theta_c, (size_t)h->P_pad));
@@ -1445,7 +1388,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     for (float* p : {h->grad, h->mom1, h->mom2})
       AGN_TRY_CUDA(cudaMemset(p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
   }
-  h->fuse_out_dw = h->use_tc && (h->use_head || h->out_tc) && (h->tc_mask & 4) && !(h->tc_mask & 8);
+  h->fuse_out_dw = h->use_tc && h->use_head && (h->tc_mask & 4) && !(h->tc_mask & 8);
   h->acc_first = h->fuse_out_dw || h->adam;
   h->ldz_out = h->fuse_out_dw ? (int)round_up(dims[h->L], 8) : dims[h->L];
   h->fuse_head = h->use_tc && h->use_head && (h->tc_mask & 1) &&
@@ -1518,7 +1461,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY(dalloc_t(h, &h->e_pred, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->e_out, 2));
     AGN_TRY(dalloc_t(h, &h->e_sw, 1));
-    AGN_TRY(upload_rows(h->Xe, hXe.data(), E, h->udims[0], d0, sizeof(float)));
+    AGN_TRY_CUDA(cudaMemcpy(h->Xe, hXe.data(), hXe.size() * sizeof(float), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemcpy(h->ye, hye.data(), hye.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemset(h->e_sw, 0, sizeof(int)));
   }
@@ -1541,10 +1484,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   // uploads
   std::vector<float> tpad((size_t)h->P_pad, 0.f);
   for (int l = 0; l < h->L; ++l) {
-    const int64_t fi = h->udims[l], fo = h->udims[l + 1], ld = dims[l];
-    for (int64_t f = 0; f < fo; ++f)
-      std::memcpy(&tpad[h->woff[l] + f * ld], &h->htheta0[h->woff_flat[l] + f * fi],
-                  (size_t)fi * sizeof(float));
+    const int64_t fi = dims[l], fo = dims[l + 1];
+    std::memcpy(&tpad[h->woff[l]], &h->htheta0[h->woff_flat[l]], (size_t)(fo * fi) * sizeof(float));
     std::memcpy(&tpad[h->boff[l]], &h->htheta0[h->boff_flat[l]], (size_t)fo * sizeof(float));
   }
   AGN_TRY_CUDA(cudaMemcpy(h->theta_c, tpad.data(), tpad.size() * sizeof(float),
@@ -1552,9 +1493,9 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   if (h->prec == AGN_PREC_BF16) {
     std::vector<bf16> xb(h->hX.size());
     for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16_rn(h->hX[i]);
-    AGN_TRY(upload_rows(h->X, xb.data(), h->N, h->udims[0], d0, es));
+    AGN_TRY_CUDA(cudaMemcpy(h->X, xb.data(), xb.size() * es, cudaMemcpyHostToDevice));
   } else {
-    AGN_TRY(upload_rows(h->X, h->hX.data(), h->N, h->udims[0], d0, es));
+    AGN_TRY_CUDA(cudaMemcpy(h->X, h->hX.data(), h->hX.size() * es, cudaMemcpyHostToDevice));
   }
   AGN_TRY_CUDA(cudaMemcpy(h->y, h->hy.data(), h->hy.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice));
@@ -1621,7 +1562,7 @@ Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int6
       AGN_TRY(agn::simt_forward<float>(g, l == L, 1, h->stream));
       in = out;
     }
-    AGN_TRY(agn::eval_logits(h->Ze, h->ye + r0, rows, h->C, h->dims[L], h->e_loss + r0,
+    AGN_TRY(agn::eval_logits(h->Ze, h->ye + r0, rows, h->dims[L], h->e_loss + r0,
                              h->e_correct + r0, h->e_pred + r0, h->stream));
   }
   AGN_TRY(agn::eval_reduce(h->e_loss, h->e_correct, h->n_eval, h->e_out, h->stream));
@@ -1661,15 +1602,15 @@ void touch_pages(void* p, size_t bytes) {
 }
 
 // A replica's (or theta~'s) parameters in the ABI's flat order: packed on the
-// device (the device pads widths and aligns tensors), then one copy straight
+// device (which aligns its tensors), then one copy straight
 // into the caller's buffer while a few threads map its pages.  (Before: the
-// padded vector into a host vector, then per-row copies: 10.7 ms for 84 MB.)
+// padded vector into a host vector, then per-tensor copies: 10.7 ms for 84 MB.)
 Status read_params(agn_handle* h, const float* dev, float* out, int64_t cap) {
   if (!out || cap < h->P) return Status::Err(AGN_E_INVALID, "output buffer shorter than P");
   std::vector<agn::PackLayer> layers;
   for (int l = 0; l < h->L; ++l)
-    layers.push_back({h->woff_flat[l], h->boff_flat[l], h->woff[l], h->boff[l], h->udims[l],
-                      h->udims[l + 1], h->dims[l]});
+    layers.push_back({h->woff_flat[l], h->boff_flat[l], h->woff[l], h->boff[l],
+                      (int64_t)h->dims[l] * h->dims[l + 1], h->dims[l + 1]});
   AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build only
   AGN_TRY(agn::pack_params(dev, h->flat, layers.data(), h->L, h->stream));
   touch_pages(out, (size_t)h->P * sizeof(float));

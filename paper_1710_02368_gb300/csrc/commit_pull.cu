@@ -357,27 +357,26 @@ __global__ void reduce_losses_kernel(const float* __restrict__ parts, int lambda
   AGN_ST(loss + c, s / (float)lambda);
 }
 
-// One layer's weights and biases from the device layout to the flat one
-// (rows of fi, unpadded).  A block copies whole rows, coalesced on both sides.
+// One layer's weights and biases from the device layout to the flat one (whose
+// tensors start anywhere: 4-byte accesses, coalesced, eight in flight).
 __global__ void __launch_bounds__(kThreads)
 pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayer L) {
   pdl_begin();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kWarps = kThreads / 32;
-  for (int64_t f = (int64_t)blockIdx.x * kWarps + warp; f < L.fo; f += (int64_t)gridDim.x * kWarps) {
-    const float* s = src + L.woff + f * L.ld;
-    float* d = dst + L.woff_flat + f * L.fi;
-    for (int k0 = lane; k0 < L.fi; k0 += 32 * 8) {
-      float v[8];
+  const int64_t i0 = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  const float* s = src + L.woff;
+  float* d = dst + L.woff_flat;
+  for (int64_t i = i0; i < L.weights; i += 8 * stride) {
+    float v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k0 + 32 * u < L.fi) v[u] = AGN_LD(s + k0 + 32 * u);
+    for (int u = 0; u < 8; ++u)
+      if (i + u * stride < L.weights) v[u] = AGN_LD(s + i + u * stride);
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k0 + 32 * u < L.fi) AGN_ST(d + k0 + 32 * u, v[u]);
-    }
-    if (lane == 0) AGN_ST(dst + L.boff_flat + f, AGN_LD(src + L.boff + f));
+    for (int u = 0; u < 8; ++u)
+      if (i + u * stride < L.weights) AGN_ST(d + i + u * stride, v[u]);
   }
+  for (int64_t f = i0; f < L.biases; f += stride)
+    AGN_ST(dst + L.boff_flat + f, AGN_LD(src + L.boff + f));
 }
 
 }  // namespace
@@ -385,7 +384,7 @@ pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayer L)
 Status pack_params(const float* src, float* dst, const PackLayer* layers, int n_layers,
                    cudaStream_t st) {
   for (int l = 0; l < n_layers; ++l) {
-    const int grid = (int)std::min<int64_t>(ceil_div(layers[l].fo, kThreads / 32), 152 * 8);
+    const int grid = (int)std::min<int64_t>(ceil_div(layers[l].weights, kThreads * 4), 152 * 8);
     auto kf = pack_kernel;
     AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, 0, st, src, dst, layers[l]));
   }

@@ -55,15 +55,13 @@ Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st);
 // and the loss of every 32-sample chunk of a slot, its cross-entropy sum / m,
 // at loss_parts[(slot_commit[z] * lam + step) * ceil(m / 32) + chunk].
 struct SoftmaxArgs {
-  const float* Z;          // [slots][m][ld] logits
-  int m, C, ld;            // columns C .. ld - 1 of dZ are left alone
+  const float* Z;          // [slots][m][C] logits
+  int m, C;
   const int* yb;           // labels [slots][m], or padded ones (x_shard > 0, batch_row0)
   const int* slot_worker;
   const long long* slot_t0;
   int64_t x_shard;
-  void* dZ;                // out [slots][m][ld] (T)
-  bf16* dZ_pieces;         // fp32 T only: also its three exact bf16 pieces, planes
-  int64_t dZ_plane;        // dZ_plane apart; null = no
+  void* dZ;                // out [slots][m][C] (T)
   float* loss_parts;
   const int* slot_commit;
   int lam, step;
@@ -153,9 +151,9 @@ struct AdamArgs {
 Status adam_step(const AdamArgs& a, int slots, int num_sms, cudaStream_t st);
 
 // Evaluation (mlp_eval.cu): per-sample loss / correctness / prediction of
-// fp32 logits Z [rows][ld] (C classes) against labels y, and their fixed-order means
+// fp32 logits Z [rows][C] against labels y, and their fixed-order means
 // (out[0] loss, out[1] accuracy).
-Status eval_logits(const float* Z, const int* y, int rows, int C, int ld, float* loss, int* correct,
+Status eval_logits(const float* Z, const int* y, int rows, int C, float* loss, int* correct,
                    int* pred, cudaStream_t st);
 Status eval_reduce(const float* loss, const int* correct, int64_t E, float* out,
                    cudaStream_t st);
@@ -170,12 +168,11 @@ Status pull_replicas(const float* theta_c, float* replicas, bf16* replicas_bf16,
                      int64_t ld, const int* workers, int count, cudaStream_t st,
                      int64_t piece_plane = 0, float* snapshot = nullptr);
 // One layer of pack_params: offsets of W_l and b_l in the flat and in the
-// device layout, their inputs, outputs and the device's row length.
+// device layout, and their element counts.
 struct PackLayer {
-  int64_t woff_flat, boff_flat, woff, boff;
-  int fi, fo, ld;
+  int64_t woff_flat, boff_flat, woff, boff, weights, biases;
 };
-// dst (flat order, unpadded) = the parameters at src (device layout).
+// dst (flat order) = the parameters at src (device layout).
 Status pack_params(const float* src, float* dst, const PackLayer* layers, int n_layers,
                    cudaStream_t st);
 // loss[c] = mean_i parts[c * lambda + i] for c < count.

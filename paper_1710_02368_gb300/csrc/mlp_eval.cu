@@ -16,12 +16,12 @@ namespace {
 constexpr int kEvalThreads = 256;
 
 __global__ void __launch_bounds__(kEvalThreads)
-eval_logits_kernel(const float* __restrict__ Z, const int* __restrict__ y, int rows, int C, int ld,
+eval_logits_kernel(const float* __restrict__ Z, const int* __restrict__ y, int rows, int C,
                    float* __restrict__ loss, int* __restrict__ correct, int* __restrict__ pred) {
   pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= rows) return;
-  const float* z = Z + (int64_t)i * ld;
+  const float* z = Z + (int64_t)i * C;
   float mx = AGN_LD(z);
   int am = 0;
   for (int c = 1; c < C; ++c) {
@@ -75,13 +75,13 @@ eval_reduce_kernel(const float* __restrict__ loss, const int* __restrict__ corre
 
 }  // namespace
 
-Status eval_logits(const float* Z, const int* y, int rows, int C, int ld, float* loss, int* correct,
+Status eval_logits(const float* Z, const int* y, int rows, int C, float* loss, int* correct,
                    int* pred, cudaStream_t st) {
   if (rows <= 0) return Status::Ok();
   {
     auto kf = eval_logits_kernel;
     AGN_TRY_CUDA(launch_pdl(kf, (unsigned)ceil_div(rows, kEvalThreads), kEvalThreads, 0, st, Z,
-                            y, rows, C, ld, loss, correct, pred));
+                            y, rows, C, loss, correct, pred));
   }
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();

@@ -207,99 +207,79 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
 }
 
 // Softmax cross-entropy (SoftmaxArgs).  A block takes a 32-sample chunk of a
-// slot, a warp four of its samples with the classes across the lanes, so that
-// a launch of few slots still fills the GPU and every load is coalesced: one
-// block per slot with a sample per thread took 38 us a launch at 4 slots x 512
-// samples x 10 classes.  kPer > 0: up to 32 kPer
-// classes held in registers; 0: any number, read three times.  Sums are fixed
-// shuffle trees, the chunk's loss a fixed tree over its samples.
-constexpr int kXentThreads = 256;
-template <typename T, int kPer>
+// slot (one block per slot took 38 us a launch at 4 slots x 512 samples x 10
+// classes): up to kXentClasses classes pass through shared memory, copied in
+// and out by the whole block, and a thread sums its sample's classes in order;
+// with more classes it reads them from global memory.  The chunk's loss is a
+// fixed tree over its samples.
+constexpr int kXentThreads = 128, kXentClasses = 128;
+template <typename T>
 __global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const SoftmaxArgs a) {
   pdl_begin();
-  __shared__ float ces[32];
-  const int z = blockIdx.y, chunk = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m = a.m, C = a.C;
+  __shared__ float zs[32 * (kXentClasses + 1)];
+  __shared__ float inv_s[32];
+  __shared__ int ys[32];
+  const int z = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
+  const int m = a.m, C = a.C, nj = min(32, m - 32 * chunk);
   const float inv_m = 1.0f / (float)m;
-  constexpr int kSamples = 32 / (kXentThreads / 32);   // per warp
-  const int* yrow =
-      a.x_shard > 0
-          ? a.yb + (int64_t)AGN_LD(a.slot_worker + z) * (a.x_shard + m) +
-                batch_row0(a.slot_t0, z, a.step, m, a.x_shard)
-          : a.yb + (int64_t)z * m;
-  float v[kSamples][kPer > 0 ? kPer : 1];
-  if (kPer > 0) {   // every sample's loads in flight together
-#pragma unroll
-    for (int u = 0; u < kSamples; ++u) {
-      const int j = 32 * chunk + kSamples * warp + u;
-#pragma unroll
-      for (int e = 0; e < kPer; ++e)
-        v[u][e] = j < m && lane + 32 * e < C
-                      ? AGN_LD(a.Z + ((int64_t)z * m + j) * a.ld + lane + 32 * e)
-                      : -INFINITY;
-    }
+  const int64_t row0 = ((int64_t)z * m + 32 * chunk) * C;
+  const float* Zc = a.Z + row0;
+  T* dZc = static_cast<T*>(a.dZ) + row0;
+  const bool staged = C <= kXentClasses;
+  const int ld = C + 1 - (C & 1);   // odd: no bank conflicts between the samples' rows
+  if (staged) {
+    for (int i = tid; i < nj * C; i += kXentThreads) zs[i / C * ld + i % C] = AGN_LD(Zc + i);
+    __syncthreads();
   }
-#pragma unroll
-  for (int u = 0; u < kSamples; ++u) {
-    const int jl = kSamples * warp + u, j = 32 * chunk + jl;
-    if (j >= m) {   // warp-uniform
-      if (lane == 0) ces[jl] = 0.f;
-      continue;
-    }
-    const int64_t row = ((int64_t)z * m + j) * a.ld;
-    const float* zr = a.Z + row;
-    const int n = kPer > 0 ? kPer : (C + 31) / 32;
-    auto at = [&](int e) {
-      return kPer > 0 ? v[u][kPer > 0 ? e : 0] : lane + 32 * e < C ? AGN_LD(zr + lane + 32 * e) : -INFINITY;
-    };
-    float mx = -INFINITY;
-#pragma unroll
-    for (int e = 0; e < n; ++e) mx = fmaxf(mx, at(e));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    const int y = AGN_LD(yrow + j);
-    float s = 0.f, zy = 0.f;
-#pragma unroll
-    for (int e = 0; e < n; ++e) {
-      const int c = lane + 32 * e;
-      if (c < C) s += expf(at(e) - mx);
-      if (c == y) zy = at(e);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    zy = __shfl_sync(0xffffffffu, zy, y & 31);
-    const float inv_s = 1.0f / s;
-#pragma unroll
-    for (int e = 0; e < n; ++e) {
-      const int c = lane + 32 * e;
-      if (c >= C) continue;
-      float p = expf(at(e) - mx) * inv_s;
-      if (c == y) p -= 1.0f;
-      const T g = from_f<T>(p * inv_m);
-      AGN_ST(static_cast<T*>(a.dZ) + row + c, g);
-      if (a.dZ_pieces) {
-        bf16 q0, q1, q2;
-        split3(to_f(g), q0, q1, q2);
-        AGN_ST(a.dZ_pieces + row + c, q0);
-        AGN_ST(a.dZ_pieces + a.dZ_plane + row + c, q1);
-        AGN_ST(a.dZ_pieces + 2 * a.dZ_plane + row + c, q2);
+  if (tid < 32) {
+    float ce = 0.f;
+    if (tid < nj) {
+      const int* yrow =
+          a.x_shard > 0
+              ? a.yb + (int64_t)AGN_LD(a.slot_worker + z) * (a.x_shard + m) +
+                    batch_row0(a.slot_t0, z, a.step, m, a.x_shard)
+              : a.yb + (int64_t)z * m;
+      const int y = AGN_LD(yrow + 32 * chunk + tid);
+      float* zr = zs + tid * ld;
+      const float* zg = Zc + (int64_t)tid * C;
+      auto at = [&](int c) { return staged ? zr[c] : AGN_LD(zg + c); };
+      float mx = at(0);
+      for (int c = 1; c < C; ++c) mx = fmaxf(mx, at(c));
+      const float zy = at(y);
+      float s = 0.f;
+      for (int c = 0; c < C; ++c) {
+        const float ex = expf(at(c) - mx);
+        if (staged) zr[c] = ex;
+        s += ex;
+      }
+      ce = (logf(s) + mx) - zy;
+      inv_s[tid] = 1.0f / s;
+      ys[tid] = y;
+      if (!staged) {
+        for (int c = 0; c < C; ++c) {
+          float p = expf(at(c) - mx) * inv_s[tid];
+          if (c == y) p -= 1.0f;
+          AGN_ST(dZc + (int64_t)tid * C + c, from_f<T>(p * inv_m));
+        }
       }
     }
-    if (lane == 0) ces[jl] = (logf(s) + mx) - zy;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    float ce = ces[lane];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, off);
-    if (lane == 0) {
+    if (tid == 0) {
       const float part = ce * inv_m;
       AGN_ST(a.loss_parts +
                  ((int64_t)AGN_LD(a.slot_commit + z) * a.lam + a.step) * gridDim.x + chunk,
              part);
       if (!isfinite(part)) atomicExch(a.flag, 1);
     }
+  }
+  if (!staged) return;   // uniform across the block
+  __syncthreads();
+  for (int i = tid; i < nj * C; i += kXentThreads) {
+    const int j = i / C, c = i % C;
+    float p = zs[j * ld + c] * inv_s[j];
+    if (c == ys[j]) p -= 1.0f;
+    AGN_ST(dZc + i, from_f<T>(p * inv_m));
   }
 }
 
@@ -406,9 +386,7 @@ Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st) {
 template <typename T>
 Status softmax_xent(const SoftmaxArgs& a, int slots, cudaStream_t st) {
   const dim3 grid((unsigned)ceil_div(a.m, 32), (unsigned)slots);
-  auto kf = a.C <= 32    ? softmax_xent_kernel<T, 1>
-            : a.C <= 128 ? softmax_xent_kernel<T, 4>
-                         : softmax_xent_kernel<T, 0>;
+  auto kf = softmax_xent_kernel<T>;
   AGN_TRY_CUDA(launch_pdl(kf, grid, kXentThreads, 0, st, a));
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();

@@ -16,7 +16,6 @@ struct TcArgs {
   int a_by_worker, b_by_worker;
   int* err;                // set to 1 when a bounded wait gives up
   void* out;               // forward / dX output (bf16) [slots][N rows][ldo]
-  int out_f32;             // forward, bf16 mode: the output is fp32 (the logits)
   int64_t ldo, out_bstride;
   const void* mask;        // dX: H_{l-1}, same layout and type as out
   int64_t mask_bstride;

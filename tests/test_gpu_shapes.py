@@ -1,8 +1,7 @@
-"""Shapes that AGN_GEMM_AUTO takes to the tensor cores although the explicit
-AGN_GEMM_TCGEN05 refuses them: layer widths that are not multiples of 8 (the
-device pads them with zeros that stay zero), minibatches past 256 (several
-column tiles, the fused output layer among them) and output layers of more
-than 16 classes (tensor-core layers, softmax over any number of classes).
+"""Shapes that the explicit AGN_GEMM_TCGEN05 refuses: minibatches past 256
+(on the tensor cores under AGN_GEMM_AUTO: several column tiles, the fused output
+layer among them), layer widths that are not multiples of 8 and output layers
+of more than 16 classes (CUDA cores, softmax over any number of classes).
 
 Every case against the float64 oracle at the fp32 tolerances of the other
 parity tests (theta~ 1e-5 relative, losses 1e-5), bf16 losses within 2e-2.
@@ -20,8 +19,8 @@ pytestmark = pytest.mark.gpu
 SHAPES = [((37, 65, 13, 7), 9, 5),           # nothing a multiple of 8
           ((3, 5, 2), 1, 2),                 # the smallest
           ((61, 130, 26), 33, 3),            # odd widths, 26 classes
-          ((40, 72, 33), 17, 4),             # 33 classes: two registers a lane
-          ((24, 40, 136, 130), 40, 2),       # 130 classes: two row tiles, classes re-read
+          ((40, 72, 33), 17, 4),             # 33 classes
+          ((24, 40, 136, 130), 40, 2),       # 130 classes: read from global memory
           ((64, 136, 10), 257, 3),           # three column tiles, one sample in the last
           ((64, 136, 10), 512, 32),          # too many tiles for the fused output layer
           ((61, 48, 40, 20), 300, 3)]        # all at once
@@ -46,7 +45,7 @@ def _run(agn, dims, m, n, lam=2, C=6, seed=19, oracle=True, eta=0.05, okw=None, 
         th0 = h.central()
         h.run(C, w, t)
         out = h.central(), h.loss(), h.replica(0)
-    assert np.array_equal(th0, I.init_params(seed, dims))   # the padding never shows
+    assert np.array_equal(th0, I.init_params(seed, dims))
     if not oracle:
         return out, None
     ds = I.SyntheticDataset(seed, dims[0], N, I.DIST_UNIFORM, (dims[0], 64, dims[-1]), N // n)
