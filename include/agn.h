@@ -331,6 +331,8 @@ int agn_plan_waves(int32_t n_workers, int32_t lambda, int32_t n_commits, const i
  *     (no fused multiply-add, so results are bit-reproducible);
  *     acc[k] = 0;  replica[p] = theta_c for every p in
  *     pull_workers[pull_offsets[c] .. pull_offsets[c+1]).
+ *   (A replica pulled more than once in a call is written once, at its last
+ *   pull.)
  *   theta_c   : device fp32 [P];  acc, replicas: device fp32 [n][ld],
  *               ld >= P, ld % 4 == 0, all three 16-byte aligned.
  *   replicas_bf16: optional device bf16 [n][ld] that receives bf16(theta_c)

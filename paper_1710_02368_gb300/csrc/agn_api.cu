@@ -1655,6 +1655,9 @@ Status commit_pull(float* theta_c, float* acc, float* reps, void* reps_b, int64_
     for (int p = po[c]; p < po[c + 1]; ++p)
       if (pw[p] < 0 || pw[p] >= n) return Status::Err(AGN_E_INVALID, "pull worker out of range");
   }
+  const agn::LastPulls pulls(n, C, po, pw);
+  po = pulls.offsets.data();
+  pw = pulls.workers.data();
   const float scale = (float)(normalize ? -(eta / (double)lambda) : -eta);
   const int grid = agn::commit_grid(P);
   double* partials = nullptr;
@@ -2020,10 +2023,14 @@ int agn_commit_pull(float* theta_c, float* acc, float* replicas, void* replicas_
                     int64_t ld, int32_t n, int32_t C, const int32_t* commit_worker,
                     const int32_t* pull_offsets, const int32_t* pull_workers, double eta,
                     int32_t lambda, int32_t normalize, float* delta_norm, void* stream) {
-  Status s = commit_pull(theta_c, acc, replicas, replicas_bf16, P, ld, n, C, commit_worker,
-                         pull_offsets, pull_workers, eta, lambda, normalize, delta_norm,
-                         static_cast<cudaStream_t>(stream));
-  return s.ok() ? AGN_OK : fail(nullptr, s);
+  try {
+    Status s = commit_pull(theta_c, acc, replicas, replicas_bf16, P, ld, n, C, commit_worker,
+                           pull_offsets, pull_workers, eta, lambda, normalize, delta_norm,
+                           static_cast<cudaStream_t>(stream));
+    return s.ok() ? AGN_OK : fail(nullptr, s);
+  } catch (const std::bad_alloc&) {
+    return fail(nullptr, AGN_E_OOM, "host allocation failed");
+  }
 }
 
 int agn_debug_waits(agn_handle* h, int64_t wait_ns, int32_t withhold_rank) {

@@ -11,6 +11,7 @@
 // library reserves when it is loaded, instead of from the stream-ordered
 // allocator.
 #include <mutex>
+#include <new>
 #include <string>
 
 #include "mlp.cuh"
@@ -83,6 +84,9 @@ agn::Status commit_pull_noalloc(float* theta_c, float* acc, float* reps, void* r
     for (int p = po[c]; p < po[c + 1]; ++p)
       if (pw[p] < 0 || pw[p] >= n) return Status::Err(AGN_E_INVALID, "pull worker out of range");
   }
+  const agn::LastPulls pulls(n, C, po, pw);
+  po = pulls.offsets.data();
+  pw = pulls.workers.data();
   double* scratch = nullptr;
   AGN_TRY(scratch_on_current_device(&scratch));
   const float scale = (float)(normalize ? -(eta / (double)lambda) : -eta);
@@ -145,9 +149,14 @@ extern "C" int agn_commit_pull_noalloc(float* theta_c, float* acc, float* replic
                                        const int32_t* pull_offsets, const int32_t* pull_workers,
                                        double eta, int32_t lambda, int32_t normalize,
                                        float* delta_norm, void* stream) {
-  agn::Status s = commit_pull_noalloc(theta_c, acc, replicas, replicas_bf16, P, ld, n, C,
-                                      commit_worker, pull_offsets, pull_workers, eta, lambda,
-                                      normalize, delta_norm, static_cast<cudaStream_t>(stream));
+  agn::Status s;
+  try {
+    s = commit_pull_noalloc(theta_c, acc, replicas, replicas_bf16, P, ld, n, C, commit_worker,
+                            pull_offsets, pull_workers, eta, lambda, normalize, delta_norm,
+                            static_cast<cudaStream_t>(stream));
+  } catch (const std::bad_alloc&) {
+    s = agn::Status::Err(AGN_E_OOM, "host allocation failed");
+  }
   if (!s.ok()) agn::set_global_error(s.msg);
   return s.code;
 }
