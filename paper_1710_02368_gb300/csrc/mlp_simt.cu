@@ -6,9 +6,11 @@
 //
 // One launch covers every worker of a wave: grid.z indexes the wave's slots,
 // and slot z reads and updates the replica of worker slot_worker[z].  All
-// three GEMM shapes use one tiled kernel (64x64 tile, 16-deep k slices, 4x4
-// outputs per thread); the element type T is float (fp32 mode) or bf16 (bf16
-// mode: operands bf16, accumulation fp32, master weights fp32).
+// three GEMM shapes use one tiled kernel (square tiles, double-buffered k
+// slices); the element type T is float (fp32 mode) or bf16 (bf16 mode:
+// operands bf16, accumulation fp32, master weights fp32).  Every output is one
+// chain of fused multiply-adds over k in ascending order from zero, whatever
+// the tile, so that the tile never changes a result.
 #include <algorithm>
 
 #include "mlp.cuh"
@@ -17,8 +19,7 @@ namespace agn {
 
 namespace {
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kTM = 4, kTN = 4;
-constexpr int kThreads = (kBM / kTM) * (kBN / kTN);   // 256
+constexpr int kThreads = 256;   // 16 x 16, kTile / 16 rows and columns each
 
 template <typename T>
 __device__ __forceinline__ float to_f(T v);
@@ -49,18 +50,29 @@ __device__ __forceinline__ void write_copy(bf16* tb, int64_t plane, int64_t p, f
 }
 
 // C[M x N] (+)= sum_k A(m, k) B(k, n) for one slot; see GemmArgs for layouts.
-template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi>
+// Bound by a block's chain over k (small launches) or by shared-memory reads:
+// the next k slice's global loads are in flight while the current one is
+// multiplied out of shared memory.  Against one 64 x 64 tile, one buffer and
+// 4-byte shared loads: a forward of 613-301-150-26 at 5 slots of 100 samples
+// 31.1 -> 17.9 us, dX 15.8 -> 9.9, dW 15.3 -> 12.8; the 784-1000-1000 forward of
+// 10000 rows 20 -> 26 TFLOP/s.  A thread's rows are consecutive (its A
+// values come in 16-byte loads), its columns 16 apart (coalesced epilogues).
+template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
 __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
+  constexpr int kBM = kTile, kBN = kTile, kBK = kTile == 32 ? 32 : 16;
+  constexpr int kTM = kTile / 16, kTN = kTile / 16;
+  constexpr int kLoads = kTile * kBK / kThreads;   // per operand, thread and slice
+  constexpr int kLd = kTile + 4;
   pdl_begin();
-  __shared__ float As[kBK][kBM + 1];
-  __shared__ float Bs[kBK][kBN + 1];
+  __shared__ __align__(16) float As[2][kBK][kLd];
+  __shared__ __align__(16) float Bs[2][kBK][kLd];
   const int z = blockIdx.z;
   const int w = AGN_LD(g.slot_worker + z);
   const int64_t m0 = (int64_t)blockIdx.y * kBM, n0 = (int64_t)blockIdx.x * kBN;
   const T* A = reinterpret_cast<const T*>(g.a) + (g.a_by_worker ? (int64_t)w : z) * g.a_bstride;
   const T* B = reinterpret_cast<const T*>(g.b) + (g.b_by_worker ? (int64_t)w : z) * g.b_bstride;
   const int tid = threadIdx.x;
-  const int tx = tid % (kBN / kTN), ty = tid / (kBN / kTN);
+  const int tx = tid % 16, ty = tid / 16;
 
   float acc[kTM][kTN];
 #pragma unroll
@@ -70,37 +82,67 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
   float bsum = 0.f;   // bias gradient (kEpi == kEpiDW, first column tile)
   const bool do_bias = (kEpi == kEpiDW) && blockIdx.x == 0 && tid < kBM;
 
+  // element r of this thread in a k slice: row (or column) o and k
+  auto place = [&](bool k_major, int r, int& o, int& kk) {
+    const int e = tid + r * kThreads;
+    if (k_major) { o = e / kBK; kk = e % kBK; } else { kk = e / kTile; o = e % kTile; }
+  };
+  T ra[kLoads], rb[kLoads];
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int r = 0; r < kLoads; ++r) {
+      int o, kk;
+      place(kAKMajor, r, o, kk);
+      const int64_t gm = m0 + o, gk = k0 + kk;
+      ra[r] = from_f<T>(0.f);
+      if (gm < g.M && gk < g.K) ra[r] = AGN_LD(kAKMajor ? A + gm * g.lda + gk : A + gk * g.lda + gm);
+    }
+#pragma unroll
+    for (int r = 0; r < kLoads; ++r) {
+      int o, kk;
+      place(kBKMajor, r, o, kk);
+      const int64_t gn = n0 + o, gk = k0 + kk;
+      rb[r] = from_f<T>(0.f);
+      if (gn < g.N && gk < g.K) rb[r] = AGN_LD(kBKMajor ? B + gn * g.ldb + gk : B + gk * g.ldb + gn);
+    }
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int r = 0; r < kLoads; ++r) {
+      int o, kk;
+      place(kAKMajor, r, o, kk);
+      As[buf][kk][o] = to_f(ra[r]);
+      place(kBKMajor, r, o, kk);
+      Bs[buf][kk][o] = to_f(rb[r]);
+    }
+  };
+  load(0);
+  stage(0);
+  __syncthreads();
+  int buf = 0;
   for (int64_t k0 = 0; k0 < g.K; k0 += kBK) {
-#pragma unroll
-    for (int r = 0; r < (kBM * kBK) / kThreads; ++r) {
-      const int e = tid + r * kThreads;
-      int mm, kk;
-      if (kAKMajor) { mm = e / kBK; kk = e % kBK; } else { kk = e / kBM; mm = e % kBM; }
-      const int64_t gm = m0 + mm, gk = k0 + kk;
-      float v = 0.f;
-      if (gm < g.M && gk < g.K)
-        v = to_f(AGN_LD(kAKMajor ? A + gm * g.lda + gk : A + gk * g.lda + gm));
-      As[kk][mm] = v;
-    }
-#pragma unroll
-    for (int r = 0; r < (kBN * kBK) / kThreads; ++r) {
-      const int e = tid + r * kThreads;
-      int nn, kk;
-      if (kBKMajor) { nn = e / kBK; kk = e % kBK; } else { kk = e / kBN; nn = e % kBN; }
-      const int64_t gn = n0 + nn, gk = k0 + kk;
-      float v = 0.f;
-      if (gn < g.N && gk < g.K)
-        v = to_f(AGN_LD(kBKMajor ? B + gn * g.ldb + gk : B + gk * g.ldb + gn));
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
+    const bool more = k0 + kBK < g.K;
+    if (more) load(k0 + kBK);
 #pragma unroll
     for (int kk = 0; kk < kBK; ++kk) {
       float a[kTM], b[kTN];
+      const float* ar = &As[buf][kk][ty * kTM];
+      if constexpr (kTM == 2) {
+        const float2 v = *reinterpret_cast<const float2*>(ar);
+        a[0] = v.x;
+        a[1] = v.y;
+      } else {
 #pragma unroll
-      for (int i = 0; i < kTM; ++i) a[i] = As[kk][ty + i * (kBM / kTM)];
+        for (int i = 0; i < kTM; i += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(ar + i);
+          a[i] = v.x;
+          a[i + 1] = v.y;
+          a[i + 2] = v.z;
+          a[i + 3] = v.w;
+        }
+      }
 #pragma unroll
-      for (int j = 0; j < kTN; ++j) b[j] = Bs[kk][tx + j * (kBN / kTN)];
+      for (int j = 0; j < kTN; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
 #pragma unroll
       for (int i = 0; i < kTM; ++i)
 #pragma unroll
@@ -108,9 +150,13 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
     }
     if (do_bias) {
 #pragma unroll
-      for (int kk = 0; kk < kBK; ++kk) bsum += As[kk][tid];
+      for (int kk = 0; kk < kBK; ++kk) bsum += As[buf][kk][tid];
     }
-    __syncthreads();
+    if (more) {   // (the other buffer's readers passed the last barrier)
+      stage(buf ^ 1);
+      __syncthreads();
+      buf ^= 1;
+    }
   }
 
   // Epilogues.
@@ -120,11 +166,11 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
     TO* out = reinterpret_cast<TO*>(g.out) + (int64_t)z * g.out_bstride;
 #pragma unroll
     for (int i = 0; i < kTM; ++i) {
-      const int64_t m = m0 + ty + i * (kBM / kTM);
+      const int64_t m = m0 + ty * kTM + i;
       if (m >= g.M) continue;
 #pragma unroll
       for (int j = 0; j < kTN; ++j) {
-        const int64_t n = n0 + tx + j * (kBN / kTN);
+        const int64_t n = n0 + tx + 16 * j;
         if (n >= g.N) continue;
         float v = acc[i][j] + AGN_LD(bias + n);
         if (g.relu) v = fmaxf(v, 0.f);
@@ -136,11 +182,11 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
     TO* out = reinterpret_cast<TO*>(g.out) + (int64_t)z * g.out_bstride;
 #pragma unroll
     for (int i = 0; i < kTM; ++i) {
-      const int64_t m = m0 + ty + i * (kBM / kTM);
+      const int64_t m = m0 + ty * kTM + i;
       if (m >= g.M) continue;
 #pragma unroll
       for (int j = 0; j < kTN; ++j) {
-        const int64_t n = n0 + tx + j * (kBN / kTN);
+        const int64_t n = n0 + tx + 16 * j;
         if (n >= g.N) continue;
         const float h = to_f(AGN_LD(mask + m * g.ldo + n));
         AGN_ST(out + m * g.ldo + n, from_f<TO>(h > 0.f ? acc[i][j] : 0.f));
@@ -150,11 +196,11 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
     float* go = g.grad_out + (int64_t)w * g.ld_param;
 #pragma unroll
     for (int i = 0; i < kTM; ++i) {
-      const int64_t m = m0 + ty + i * (kBM / kTM);
+      const int64_t m = m0 + ty * kTM + i;
       if (m >= g.M) continue;
 #pragma unroll
       for (int j = 0; j < kTN; ++j) {
-        const int64_t n = n0 + tx + j * (kBN / kTN);
+        const int64_t n = n0 + tx + 16 * j;
         if (n < g.N) AGN_ST(go + g.woff + m * g.N + n, acc[i][j]);
       }
     }
@@ -163,37 +209,41 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
     const bool has_a = g.acc != nullptr;
     float* a = has_a ? g.acc + (int64_t)w * g.ld_param : theta;
     bf16* tb = g.theta_bf16 ? g.theta_bf16 + (int64_t)w * g.ld_param : nullptr;
-    // loads of all 16 outputs first, then the updates (memory-level parallelism)
+    // several rows' loads first, then their updates (memory-level parallelism)
     const float* __restrict__ th_in = theta;
     const float* __restrict__ a_in = a;
-    float th[kTM][kTN], av[kTM][kTN];
+    constexpr int kRows = kTM < 4 ? kTM : 4;   // rows in flight at a time
 #pragma unroll
-    for (int i = 0; i < kTM; ++i) {
-      const int64_t m = m0 + ty + i * (kBM / kTM);
+    for (int i0 = 0; i0 < kTM; i0 += kRows) {
+      float th[kRows][kTN], av[kRows][kTN];
 #pragma unroll
-      for (int j = 0; j < kTN; ++j) {
-        const int64_t n = n0 + tx + j * (kBN / kTN);
-        if (m < g.M && n < g.N) {
-          const int64_t p = g.woff + m * g.N + n;
-          th[i][j] = AGN_LDCS(th_in + p);
-          av[i][j] = has_a ? AGN_LDCS(a_in + p) : 0.f;
+      for (int i = 0; i < kRows; ++i) {
+        const int64_t m = m0 + ty * kTM + i0 + i;
+#pragma unroll
+        for (int j = 0; j < kTN; ++j) {
+          const int64_t n = n0 + tx + 16 * j;
+          if (m < g.M && n < g.N) {
+            const int64_t p = g.woff + m * g.N + n;
+            th[i][j] = AGN_LDCS(th_in + p);
+            av[i][j] = has_a ? AGN_LDCS(a_in + p) : 0.f;
+          }
         }
       }
-    }
 #pragma unroll
-    for (int i = 0; i < kTM; ++i) {
-      const int64_t m = m0 + ty + i * (kBM / kTM);
-      if (m >= g.M) continue;
+      for (int i = 0; i < kRows; ++i) {
+        const int64_t m = m0 + ty * kTM + i0 + i;
+        if (m >= g.M) continue;
 #pragma unroll
-      for (int j = 0; j < kTN; ++j) {
-        const int64_t n = n0 + tx + j * (kBN / kTN);
-        if (n >= g.N) continue;
-        const int64_t p = g.woff + m * g.N + n;
-        const float gr = acc[i][j];
-        const float t = local_step(th[i][j], g.eta, gr);
-        AGN_ST(theta + p, t);
-        if (has_a) AGN_ST(a + p, av[i][j] + gr);
-        if (tb) write_copy(tb, g.piece_plane, p, t);
+        for (int j = 0; j < kTN; ++j) {
+          const int64_t n = n0 + tx + 16 * j;
+          if (n >= g.N) continue;
+          const int64_t p = g.woff + m * g.N + n;
+          const float gr = acc[i0 + i][j];
+          const float t = local_step(th[i][j], g.eta, gr);
+          AGN_ST(theta + p, t);
+          if (has_a) AGN_ST(a + p, av[i][j] + gr);
+          if (tb) write_copy(tb, g.piece_plane, p, t);
+        }
       }
     }
     if (do_bias && m0 + tid < g.M) {
@@ -357,15 +407,28 @@ __global__ void __launch_bounds__(256) gather4_kernel(const T* __restrict__ X,
   if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The largest tile (fewest shared-memory reads per multiply-add) that still
+// gives every SM a block or, of 128, one and a half; small launches take small tiles, since a block's
+// chain over k is then what bounds them.
 template <typename T, typename TO, bool kAK, bool kBK, int kEpi>
 Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
-  dim3 grid((unsigned)ceil_div(g.N, kBN), (unsigned)ceil_div(g.M, kBM), (unsigned)slots);
-  {
-    auto kf = gemm_simt_kernel<T, TO, kAK, kBK, kEpi>;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      (void)cudaGetLastError();
+    return std::max(n, 1);
+  }();
+  auto blocks = [&](int t) { return ceil_div(g.N, t) * ceil_div(g.M, t) * (int64_t)slots; };
+  auto go = [&](auto kf, int t) -> Status {
+    dim3 grid((unsigned)ceil_div(g.N, t), (unsigned)ceil_div(g.M, t), (unsigned)slots);
     AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, 0, st, g));
-  }
-  AGN_TRY_CUDA(cudaGetLastError());
-  return Status::Ok();
+    AGN_TRY_CUDA(cudaGetLastError());
+    return Status::Ok();
+  };
+  if (blocks(128) >= 3 * sms / 2) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 128>, 128);
+  if (blocks(64) >= sms) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 64>, 64);
+  return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 32>, 32);
 }
 
 }  // namespace
