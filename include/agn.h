@@ -208,10 +208,10 @@ int agn_loss(agn_handle* h, float* out, int64_t cap);
  * Loss and accuracy of the current theta~ on the held-out set (the training-
  * accuracy curves of Section 4): softmax cross-entropy mean and the fraction
  * of samples whose argmax (lowest index on ties) is the label.  Forward pass in
- * fp32 on the device (CUDA-core GEMMs), fixed-order reductions; blocks until
- * done.  loss, accuracy: host floats (nullable); pred: host int32 [n_eval]
+ * fp32 on the device (the hidden layers on the tensor cores where training
+ * uses them), fixed-order reductions; blocks until done.  loss, accuracy: host floats (nullable); pred: host int32 [n_eval]
  * predictions (nullable), cap its length.  AGN_E_INVALID without an
- * evaluation set or with a short pred buffer.  No counterpart call in the
+ * evaluation set or with a short pred buffer; AGN_E_TIMEOUT as for agn_run.  No counterpart call in the
  * paper, which reports these metrics.
  */
 int agn_evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int64_t cap);

@@ -182,6 +182,17 @@ struct agn_handle {
   float* Xe = nullptr;        // [n_eval][d0] fp32
   int* ye = nullptr;          // [n_eval]
   float* He[2] = {nullptr, nullptr};   // [eval_chunk][max hidden d]
+  // on the tensor cores (fp32 mode): the rows' three pieces in place of Xe, the
+  // hidden layers' pieces (He[0]: the last one's fp32 values, for a narrow
+  // output layer) and theta~'s maps per layer
+  bool eval_tc = false;
+  bf16* Xe_p = nullptr;                // [3][n_eval][d0]
+  bf16* He_p[2] = {nullptr, nullptr};  // [3][eval_chunk][max hidden d]
+  int64_t eval_plane = 0;
+  struct EvalMaps {
+    CUtensorMap w_k, w_k256, h_k;      // (h_k of layer 1 is made per chunk)
+  };
+  std::vector<EvalMaps> emaps;
   float* Ze = nullptr;        // [eval_chunk][d_L]
   float* e_loss = nullptr;    // [n_eval]
   int* e_correct = nullptr;   // [n_eval]
@@ -560,18 +571,17 @@ Status build_tc_maps(agn_handle* h) {
   return Status::Ok();
 }
 
-// Column tile of a forward or dX GEMM with M rows and N = m columns over s
+// Column tile of a forward or dX GEMM with M rows and m columns over s
 // slots.  fp32 mode, m > 128: 256 only where the tiles nearly fill the SMs.  A
 // tile of 128 takes A's pieces from tensor memory and gives small waves twice
 // the CTAs; one of 256 converts every weight tile half as often.  Measured, us
 // per local step of 784-1000-1000-10 at m = 256: 1 worker 56.5 (128) / 60.9
 // (256), 4 workers 110.7 / 112.0, 16 workers 394 / 357; 784-4096-4096-10, 4
 // workers, 822 / 721; 64-48-10 at m = 200, 41.1 / 60.5.
-int tc_bn(const agn_handle* h, int M, int s) {
-  const int m = h->m;
+int tc_bn(const agn_handle* h, bool split, int M, int m, int s) {
   if (m <= 64) return 64;
   if (m <= 128) return 128;
-  if (!h->split) return 256;
+  if (!split) return 256;
   return 4 * ceil_div(M, 128) * ceil_div(m, 256) * (int64_t)s >= 3 * (int64_t)h->num_sms ? 256 : 128;
 }
 
@@ -579,9 +589,9 @@ int tc_bn(const agn_handle* h, int M, int s) {
 // K inner over s slots: one CTA per output tile, unless the tiles leave SMs idle
 // (small waves); then ks CTAs share each tile, with ks <= SMs / tiles and
 // every CTA's range of 64-deep k steps non-empty.
-int pick_ksplit(const agn_handle* h, int M, int K, int s, int bn) {
+int pick_ksplit(const agn_handle* h, int M, int m, int K, int s, int bn) {
   if (h->tc_mask & 16) return 1;
-  const int64_t tiles = ceil_div(M, 128) * ceil_div(h->m, bn) * (int64_t)s;
+  const int64_t tiles = ceil_div(M, 128) * ceil_div(m, bn) * (int64_t)s;
   if (tiles >= h->num_sms) return 1;
   const int kt = (int)ceil_div(K, 64);
   int ks = (int)std::min<int64_t>(kt, h->num_sms / tiles);
@@ -674,7 +684,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // launch's CTAs fit the SMs at once
     const bool fuse_head_now =
         h->fuse_head && tc_layer(h, L - 1) &&
-        ceil_div(h->dims[L - 1], 128) * ceil_div(m, tc_bn(h, h->dims[L - 1], s)) * (int64_t)s <=
+        ceil_div(h->dims[L - 1], 128) *
+                ceil_div(m, tc_bn(h, h->split, h->dims[L - 1], m, s)) * (int64_t)s <=
             (int64_t)h->num_sms;
     bool head_done = false;
     // forward, l = 1..L
@@ -760,8 +771,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
           t.no_a_prefetch = l == 1 && (h->tc_mask & 512) ? 1 : 0;
-          const int bn = tc_bn(h, fo, s);
-          t.ksplit = pick_ksplit(h, fo, fi, s, bn);
+          const int bn = tc_bn(h, h->split, fo, m, s);
+          t.ksplit = pick_ksplit(h, fo, m, fi, s, bn);
           next_counters(h, &t);
           bool launched = false;
           AGN_TRY(agn::tc_forward_head(h->split && bn == 256 ? mp.w_k256 : mp.w_k, mp.h_k, t, s,
@@ -781,8 +792,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
           t.no_a_prefetch = l == 1 && (h->tc_mask & 512) ? 1 : 0;
-          const int bn = tc_bn(h, fo, s);
-          t.ksplit = pick_ksplit(h, fo, fi, s, bn);
+          const int bn = tc_bn(h, h->split, fo, m, s);
+          t.ksplit = pick_ksplit(h, fo, m, fi, s, bn);
           next_counters(h, &t);
           AGN_TRY(agn::tc_forward(h->split && bn == 256 ? mp.w_k256 : mp.w_k, mp.h_k, t, s,
                                   h->stream, h->split, bn));
@@ -833,8 +844,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         t.mask = Hprev; t.mask_bstride = (int64_t)m * fi;
         t.out_pieces = next_pieces; t.out_plane = dz_plane(l - 1);
         const auto& mp = maps_of(l);
-        const int bn = tc_bn(h, fi, s);
-        t.ksplit = pick_ksplit(h, fi, fo, s, bn);
+        const int bn = tc_bn(h, h->split, fi, m, s);
+        t.ksplit = pick_ksplit(h, fi, m, fo, s, bn);
         next_counters(h, &t);
         AGN_TRY(agn::tc_backward_dx(mp.w_mn, mp.dz_k, t, s, h->stream, h->split, bn));
         have_pieces[l - 1] = next_pieces != nullptr;
@@ -1107,6 +1118,20 @@ Status build_plan(const agn_handle* h, int k, const int32_t* worker, const int32
   return Status::Ok();
 }
 
+// A tensor-core kernel gave up on a bounded wait: its error flag and the
+// arrival counters of CTAs that left tiles unfinished, cleared.
+Status clear_flags(agn_handle* h, bool timed_out) {
+  AGN_TRY_CUDA(cudaMemsetAsync(h->flag, 0, 2 * sizeof(int), h->stream));
+  if (timed_out && h->tc_counter)
+    AGN_TRY_CUDA(cudaMemsetAsync(h->tc_counter, 0, (size_t)(2 * h->num_sms) * sizeof(int),
+                                 h->stream));
+  if (timed_out && h->fuse_head)
+    AGN_TRY_CUDA(cudaMemsetAsync(h->fh_counter, 0,
+                                 (size_t)(2 * h->n * ceil_div(h->m, 32)) * sizeof(int), h->stream));
+  AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+  return Status::Ok();
+}
+
 Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, int ns) {
   const auto t_host0 = std::chrono::steady_clock::now();
   NvtxRange run_range("agn_run");
@@ -1215,16 +1240,7 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
   h->pulled_v = plan.pulled_v;
   h->steps = plan.steps;
   if (flags[0] || flags[1]) {
-    AGN_TRY_CUDA(cudaMemsetAsync(h->flag, 0, 2 * sizeof(int), h->stream));
-    if (flags[1] && h->tc_counter)   // CTAs that gave up may have left tiles unfinished
-      AGN_TRY_CUDA(cudaMemsetAsync(h->tc_counter, 0, (size_t)(2 * h->num_sms) * sizeof(int),
-                                   h->stream));
-    if (flags[1] && h->fuse_head) {
-      AGN_TRY_CUDA(cudaMemsetAsync(h->fh_counter, 0,
-                                   (size_t)(2 * h->n * ceil_div(h->m, 32)) * sizeof(int),
-                                   h->stream));
-    }
-    AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+    AGN_TRY(clear_flags(h, flags[1] != 0));
     if (!bounds.ok()) return bounds;
     if (flags[1])
       return Status::Err(AGN_E_TIMEOUT, "a tensor-core GEMM gave up on a bounded wait");
@@ -1448,13 +1464,17 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   AGN_TRY(dalloc_t(h, &h->head_counter, (size_t)n));
   if (h->n_eval > 0) {
     const int64_t E = h->n_eval;
-    h->eval_chunk = std::min<int64_t>(E, 4096);
     int maxh = 1;
     for (int l = 1; l < h->L; ++l) maxh = std::max(maxh, dims[l]);
+    // the tensor cores evaluate what they train; fewer, larger chunks keep
+    // every SM busy (300 MB of pieces at most, 4096 rows at least)
+    h->eval_tc = h->use_tc;
+    h->eval_chunk = std::min<int64_t>(
+        E, !h->eval_tc ? 4096 : std::max<int64_t>(4096, (48 << 20) / maxh / 256 * 256));
     AGN_TRY(dalloc_t(h, &h->Xe, (size_t)(E * d0)));
     AGN_TRY(dalloc_t(h, &h->ye, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->He[0], (size_t)(h->eval_chunk * maxh)));
-    AGN_TRY(dalloc_t(h, &h->He[1], (size_t)(h->eval_chunk * maxh)));
+    if (!h->eval_tc) AGN_TRY(dalloc_t(h, &h->He[1], (size_t)(h->eval_chunk * maxh)));
     AGN_TRY(dalloc_t(h, &h->Ze, (size_t)(h->eval_chunk * dims[h->L])));
     AGN_TRY(dalloc_t(h, &h->e_loss, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->e_correct, (size_t)E));
@@ -1464,6 +1484,28 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY_CUDA(cudaMemcpy(h->Xe, hXe.data(), hXe.size() * sizeof(float), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemcpy(h->ye, hye.data(), hye.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemset(h->e_sw, 0, sizeof(int)));
+    if (h->eval_tc) {
+      AGN_TRY(dalloc_t(h, &h->Xe_p, (size_t)(3 * E * d0)));
+      h->eval_plane = h->eval_chunk * maxh;
+      for (bf16*& p : h->He_p) AGN_TRY(dalloc_t(h, &p, (size_t)(3 * h->eval_plane)));
+      AGN_TRY(agn::bounds_upload(h->stream));
+      AGN_TRY(agn::split_pieces(h->Xe, h->Xe_p, E * d0, E * d0, h->stream));
+      AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+      dfree(h, h->Xe);
+      h->Xe = nullptr;
+      constexpr uint32_t bk = agn::kTcSplitBK, bn = agn::kTcBoxN;
+      h->emaps.assign(h->L - 1, {});
+      for (int l = 1; l < h->L; ++l) {
+        const uint64_t fi = dims[l - 1], fo = dims[l];
+        auto& mp = h->emaps[l - 1];
+        const float* W = h->theta_c + h->woff[l - 1];
+        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k, W, fi, fo, 1, fi, fi * fo, bk, 128, true));
+        AGN_TRY(agn::make_tmap_f32_3d(&mp.w_k256, W, fi, fo, 1, fi, fi * fo, bk, 128));
+        if (l > 1)
+          AGN_TRY(agn::make_tmap_bf16_4d(&mp.h_k, h->He_p[(l - 1) % 2], fi, h->eval_chunk, 1, fi,
+                                         h->eval_chunk * fi, h->eval_plane, bk, bn));
+      }
+    }
   }
   AGN_TRY_CUDA(cudaMemsetAsync(h->head_counter, 0, (size_t)n * sizeof(int), h->stream));
   if (h->fuse_head) {
@@ -1536,34 +1578,81 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   return Status::Ok();
 }
 
-// Loss and accuracy of theta~ on the held-out set: the forward pass on the
-// CUDA-core fp32 GEMMs (theta~ as every row block's weights), then per-sample
-// log-sum-exp / argmax and fixed-order means.
+// Layer l of the evaluation's forward pass on the CUDA-core fp32 GEMMs (theta~
+// as every row block's weights).
+Status eval_layer_simt(agn_handle* h, int l, const float* in, float* out, int rows) {
+  const int fi = h->dims[l - 1], fo = h->dims[l];
+  agn::GemmArgs g{};
+  g.M = rows; g.N = fo; g.K = fi;
+  g.a = in; g.lda = fi;
+  g.b = h->theta_c + h->woff[l - 1]; g.ldb = fi;   // b_bstride 0: one weight set
+  g.slot_worker = h->e_sw;
+  g.out = out; g.ldo = fo;
+  g.relu = l < h->L;
+  g.theta = h->theta_c; g.ld_param = 0; g.boff = h->boff[l - 1];
+  return agn::simt_forward<float>(g, l == h->L, 1, h->stream);
+}
+
+Status eval_chunk_simt(agn_handle* h, int64_t r0, int rows) {
+  const int L = h->L;
+  const float* in = h->Xe + r0 * h->dims[0];
+  for (int l = 1; l <= L; ++l) {
+    float* out = l == L ? h->Ze : h->He[l % 2];
+    AGN_TRY(eval_layer_simt(h, l, in, out, rows));
+    in = out;
+  }
+  return agn::eval_logits(h->Ze, h->ye + r0, rows, h->dims[L], h->e_loss + r0,
+                          h->e_correct + r0, h->e_pred + r0, h->stream);
+}
+
+// The hidden layers on the tensor cores: theta~ is the replica of the one slot,
+// the chunk's rows its minibatch.  A layer writes only the pieces that the next
+// one reads, the last hidden one its fp32 values; the output layer follows
+// with the samples' results in one kernel (narrow), or on the CUDA cores.
+Status eval_chunk_tc(agn_handle* h, int64_t r0, int rows) {
+  const int L = h->L;
+  const int64_t d0 = h->dims[0];
+  CUtensorMap x_k;
+  AGN_TRY(agn::make_tmap_bf16_4d(&x_k, h->Xe_p + r0 * d0, d0, rows, 1, d0, rows * d0,
+                                 h->n_eval * d0, agn::kTcSplitBK, agn::kTcBoxN));
+  for (int l = 1; l < L; ++l) {
+    const int fi = h->dims[l - 1], fo = h->dims[l];
+    agn::TcArgs t = tc_args(h, h->e_sw, nullptr, 0, 0);
+    t.x_shard = 0;
+    t.M = fo; t.N = rows; t.K = fi;
+    t.a_by_worker = 1;
+    t.theta = h->theta_c; t.ld_param = 0; t.boff = h->boff[l - 1];
+    t.out = l == L - 1 ? h->He[0] : nullptr;
+    t.ldo = fo;
+    t.relu = 1;
+    t.out_pieces = l == L - 1 ? nullptr : h->He_p[l % 2]; t.out_plane = h->eval_plane;
+    const int bn = tc_bn(h, true, fo, rows, 1);
+    t.ksplit = pick_ksplit(h, fo, rows, fi, 1, bn);
+    next_counters(h, &t);
+    const auto& mp = h->emaps[l - 1];
+    AGN_TRY(agn::tc_forward(bn == 256 ? mp.w_k256 : mp.w_k, l == 1 ? x_k : mp.h_k, t, 1, h->stream,
+                            true, bn));
+  }
+  if (h->dims[L] <= agn::kHeadMaxClasses)
+    return agn::eval_head(h->He[0], h->theta_c + h->woff[L - 1], h->theta_c + h->boff[L - 1],
+                          h->ye + r0, rows, h->dims[L - 1], h->dims[L], h->e_loss + r0,
+                          h->e_correct + r0, h->e_pred + r0, h->stream);
+  AGN_TRY(eval_layer_simt(h, L, h->He[0], h->Ze, rows));
+  return agn::eval_logits(h->Ze, h->ye + r0, rows, h->dims[L], h->e_loss + r0,
+                          h->e_correct + r0, h->e_pred + r0, h->stream);
+}
+
+// Loss and accuracy of theta~ on the held-out set: the forward pass in chunks
+// of rows, per-sample log-sum-exp / argmax, fixed-order means.
 Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int64_t cap) {
   if (h->n_eval <= 0)
     return Status::Err(AGN_E_INVALID, "the handle has no evaluation set (agn_options.n_eval)");
   if (pred && cap < h->n_eval) return Status::Err(AGN_E_INVALID, "pred shorter than n_eval");
-  const int L = h->L;
   AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build only
   for (int64_t r0 = 0; r0 < h->n_eval; r0 += h->eval_chunk) {
     const int rows = (int)std::min<int64_t>(h->eval_chunk, h->n_eval - r0);
-    const float* in = h->Xe + r0 * h->dims[0];
-    for (int l = 1; l <= L; ++l) {
-      const int fi = h->dims[l - 1], fo = h->dims[l];
-      agn::GemmArgs g{};
-      g.M = rows; g.N = fo; g.K = fi;
-      g.a = in; g.lda = fi;
-      g.b = h->theta_c + h->woff[l - 1]; g.ldb = fi;   // b_bstride 0: one weight set
-      g.slot_worker = h->e_sw;
-      float* out = l == L ? h->Ze : h->He[l % 2];
-      g.out = out; g.ldo = fo;
-      g.relu = l < L;
-      g.theta = h->theta_c; g.ld_param = 0; g.boff = h->boff[l - 1];
-      AGN_TRY(agn::simt_forward<float>(g, l == L, 1, h->stream));
-      in = out;
-    }
-    AGN_TRY(agn::eval_logits(h->Ze, h->ye + r0, rows, h->dims[L], h->e_loss + r0,
-                             h->e_correct + r0, h->e_pred + r0, h->stream));
+    if (h->eval_tc) AGN_TRY(eval_chunk_tc(h, r0, rows));
+    else AGN_TRY(eval_chunk_simt(h, r0, rows));
   }
   AGN_TRY(agn::eval_reduce(h->e_loss, h->e_correct, h->n_eval, h->e_out, h->stream));
   float o2[2];
@@ -1571,8 +1660,15 @@ Status evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int6
   if (pred)
     AGN_TRY_CUDA(cudaMemcpyAsync(pred, h->e_pred, (size_t)h->n_eval * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, h->stream));
+  int flags[2] = {0, 0};
+  if (h->eval_tc)
+    AGN_TRY_CUDA(cudaMemcpyAsync(flags, h->flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
   AGN_TRY(agn::bounds_collect(h->stream));
+  if (flags[1]) {
+    AGN_TRY(clear_flags(h, true));
+    return Status::Err(AGN_E_TIMEOUT, "a tensor-core GEMM gave up on a bounded wait");
+  }
   if (loss) *loss = o2[0];
   if (accuracy) *accuracy = o2[1];
   return Status::Ok();

@@ -155,6 +155,10 @@ Status adam_step(const AdamArgs& a, int slots, int num_sms, cudaStream_t st);
 // (out[0] loss, out[1] accuracy).
 Status eval_logits(const float* Z, const int* y, int rows, int C, float* loss, int* correct,
                    int* pred, cudaStream_t st);
+// The same from the last hidden layer's fp32 activations H [rows][K] (K % 4 == 0)
+// and a narrow output layer (C <= kHeadMaxClasses) W [C][K], b [C].
+Status eval_head(const float* H, const float* W, const float* b, const int* y, int rows, int K,
+                 int C, float* loss, int* correct, int* pred, cudaStream_t st);
 Status eval_reduce(const float* loss, const int* correct, int64_t E, float* out,
                    cudaStream_t st);
 // Eq. 4 on two sampled curves (host).

@@ -2,9 +2,10 @@
 // time curves of the paper's experiments, Section 4) and the temporal
 // efficiency of two such curves (Eq. 4).
 //
-// The forward pass reuses the CUDA-core fp32 GEMMs with theta~ as the weight
-// operand of every row block (evaluation is not on the training hot path;
-// theta~ has no bf16 copy).  Per sample: log-sum-exp with max subtraction,
+// The forward pass reuses the training GEMMs with theta~ as the one weight set
+// and the rows as one slot's minibatch: the tensor cores' fp32 mode (three
+// exact bf16 pieces of every operand), or the CUDA-core kernels where the
+// handle trains on them.  Per sample: log-sum-exp with max subtraction,
 // loss = lse - z_y, prediction = argmax with the lowest index on ties, as the
 // teacher labels are defined.  Sums are taken in a fixed order (deterministic).
 #include "mlp.cuh"
@@ -37,6 +38,85 @@ eval_logits_kernel(const float* __restrict__ Z, const int* __restrict__ y, int r
   AGN_ST(loss + i, (logf(s) + mx) - AGN_LD(z + yi));
   AGN_ST(correct + i, am == yi ? 1 : 0);
   if (pred) AGN_ST(pred + i, am);
+}
+
+// A narrow output layer and the per-sample results in one pass over the last
+// hidden layer's activations: a warp takes kRows samples, so that each load of
+// W_L (a few tens of KB, resident in L1) serves all of them; every lane sums
+// four inputs at a time, the lanes fold by a fixed shuffle tree.  Bound by the
+// read of H from the L2: 10000 x 1000 (40 MB).
+constexpr int kRows = 4, kHeadWarps = 4;
+template <int kC>
+__global__ void __launch_bounds__(32 * kHeadWarps)
+eval_head_kernel(const float* __restrict__ H, const float* __restrict__ W,
+                 const float* __restrict__ b, const int* __restrict__ y, int rows, int K, int C,
+                 float* __restrict__ loss, int* __restrict__ correct, int* __restrict__ pred) {
+  pdl_begin();
+  const int lane = threadIdx.x & 31;
+  const int r0 = (blockIdx.x * kHeadWarps + (threadIdx.x >> 5)) * kRows;
+  if (r0 >= rows) return;   // uniform across the warp
+  float z[kC][kRows];
+#pragma unroll
+  for (int c = 0; c < kC; ++c)
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) z[c][r] = 0.f;
+  for (int k = 4 * lane; k < K; k += 128) {
+    float4 h[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+      h[r] = r0 + r < rows
+                 ? AGN_LD(reinterpret_cast<const float4*>(H + (int64_t)(r0 + r) * K + k))
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kC; ++c) {
+      if (c >= C) break;
+      const float4 w = AGN_LD(reinterpret_cast<const float4*>(W + (int64_t)c * K + k));
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) {
+        float t = fmaf(h[r].x, w.x, z[c][r]);
+        t = fmaf(h[r].y, w.y, t);
+        t = fmaf(h[r].z, w.z, t);
+        z[c][r] = fmaf(h[r].w, w.w, t);
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < kC; ++c) {
+    if (c >= C) break;
+    const float bc = AGN_LD(b + c);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1)
+        z[c][r] += __shfl_xor_sync(0xffffffffu, z[c][r], off);
+      z[c][r] += bc;
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    if (r0 + r >= rows) break;
+    const int yi = AGN_LD(y + r0 + r);
+    float mx = z[0][r], zy = z[0][r];
+    int am = 0;
+#pragma unroll
+    for (int c = 1; c < kC; ++c) {
+      if (c >= C) break;
+      if (z[c][r] > mx) {   // strict: the lowest index wins ties
+        mx = z[c][r];
+        am = c;
+      }
+      if (c == yi) zy = z[c][r];
+    }
+    float se = 0.f;
+#pragma unroll
+    for (int c = 0; c < kC; ++c)
+      if (c < C) se += expf(z[c][r] - mx);
+    if (lane == 0) {
+      AGN_ST(loss + r0 + r, (logf(se) + mx) - zy);
+      AGN_ST(correct + r0 + r, am == yi ? 1 : 0);
+      AGN_ST(pred + r0 + r, am);
+    }
+  }
 }
 
 // out[0] = mean loss, out[1] = accuracy over E samples: thread t sums samples
@@ -83,6 +163,18 @@ Status eval_logits(const float* Z, const int* y, int rows, int C, float* loss, i
     AGN_TRY_CUDA(launch_pdl(kf, (unsigned)ceil_div(rows, kEvalThreads), kEvalThreads, 0, st, Z,
                             y, rows, C, loss, correct, pred));
   }
+  AGN_TRY_CUDA(cudaGetLastError());
+  return Status::Ok();
+}
+
+Status eval_head(const float* H, const float* W, const float* b, const int* y, int rows, int K,
+                 int C, float* loss, int* correct, int* pred, cudaStream_t st) {
+  if (rows <= 0) return Status::Ok();
+  if (C < 1 || C > kHeadMaxClasses || K % 4)
+    return Status::Err(AGN_E_INVALID, "evaluation head: classes or inputs");
+  auto kf = C <= 4 ? eval_head_kernel<4> : C <= 10 ? eval_head_kernel<10> : eval_head_kernel<16>;
+  AGN_TRY_CUDA(launch_pdl(kf, (unsigned)ceil_div(rows, kRows * kHeadWarps), 32 * kHeadWarps, 0, st,
+                          H, W, b, y, rows, K, C, loss, correct, pred));
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();
 }

@@ -854,7 +854,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                   for (int e = 0; e < 4; ++e) v[e] = hv[e] > 0.f ? v[e] : 0.f;
                 }
                 const int64_t o4 = (int64_t)j * args.ldo + row4;
-                store4(out + o4, v);
+                if (kSplit == 1 || args.out) store4(out + o4, v);
                 if (kSplit == 3 && args.out_pieces) {
                   uint2 q0, q1, q2;
                   split3_x4(v, q0, q1, q2);

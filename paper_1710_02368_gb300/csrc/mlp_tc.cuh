@@ -15,7 +15,8 @@ struct TcArgs {
   const int* slot_worker;
   int a_by_worker, b_by_worker;
   int* err;                // set to 1 when a bounded wait gives up
-  void* out;               // forward / dX output (bf16) [slots][N rows][ldo]
+  void* out;               // forward / dX output (bf16) [slots][N rows][ldo]; split mode: fp32,
+                           // null where only its pieces are read
   int64_t ldo, out_bstride;
   const void* mask;        // dX: H_{l-1}, same layout and type as out
   int64_t mask_bstride;
