@@ -360,11 +360,17 @@ __global__ void reduce_losses_kernel(const float* __restrict__ parts, int lambda
   AGN_ST(loss + c, s / (float)lambda);
 }
 
-// One layer's weights and biases from the device layout to the flat one (whose
-// tensors start anywhere: 4-byte accesses, coalesced, eight in flight).
+// Layer blockIdx.y's weights and biases from the device layout to the flat one
+// (whose tensors start anywhere: 4-byte accesses, coalesced, eight in flight).
+constexpr int kPackLayers = 16;
+struct PackBatch {
+  PackLayer layer[kPackLayers];
+};
 __global__ void __launch_bounds__(kThreads)
-pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayer L) {
+pack_kernel(const float* __restrict__ src, float* __restrict__ dst,
+            const __grid_constant__ PackBatch batch) {
   pdl_begin();
+  const PackLayer& L = batch.layer[blockIdx.y];
   const int64_t i0 = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   const float* s = src + L.woff;
@@ -386,10 +392,17 @@ pack_kernel(const float* __restrict__ src, float* __restrict__ dst, PackLayer L)
 
 Status pack_params(const float* src, float* dst, const PackLayer* layers, int n_layers,
                    cudaStream_t st) {
-  for (int l = 0; l < n_layers; ++l) {
-    const int grid = (int)std::min<int64_t>(ceil_div(layers[l].weights, kThreads * 4), 152 * 8);
+  for (int l0 = 0; l0 < n_layers; l0 += kPackLayers) {
+    PackBatch batch{};
+    const int n = std::min(kPackLayers, n_layers - l0);
+    int64_t most = 1;
+    for (int l = 0; l < n; ++l) {
+      batch.layer[l] = layers[l0 + l];
+      most = std::max(most, batch.layer[l].weights);
+    }
+    const dim3 grid((unsigned)std::min<int64_t>(ceil_div(most, kThreads * 4), 152 * 8), (unsigned)n);
     auto kf = pack_kernel;
-    AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, 0, st, src, dst, layers[l]));
+    AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, 0, st, src, dst, batch));
   }
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();
