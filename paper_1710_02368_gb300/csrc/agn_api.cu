@@ -259,6 +259,12 @@ struct agn_handle {
   // local steps whose activations and dZ the buffers keep ([hist][n][m][d]; 1:
   // only the current one's), see run_wave_steps
   int hist = 1;
+  // local steps over which theta_k stays at a base; the fp32 biases and W_L of
+  // the steps inside a block: [n][ld_work], places of b_l and W_L
+  int block = 1;
+  float* work = nullptr;
+  int64_t ld_work = 0, wwoff = -1;
+  std::vector<int64_t> wboff;
   // the first local step of a commit stores a_k = g, so no commit zeroes a_k
   // (every layer's dW in the persistent tensor-core launch, or Adam)
   bool acc_first = false;
@@ -633,12 +639,23 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     return (h->split && l >= 1 && tc_layer(h, l)) ? h->dZp[l] : nullptr;
   };
   auto dz_plane = [&](int l) -> int64_t { return (int64_t)n * m * h->dims[l]; };
-  // bf16 waves whose accumulators stream from DRAM: each step's activations
-  // and dZ stay in the history, the steps' dW updates theta_k alone, and one
-  // launch sums the gradients of up to `hist` steps into a_k (K = steps m).
+  // bf16 waves whose replicas stream from DRAM: each step's activations and dZ
+  // stay in the history, the steps' dW updates theta_k alone, and one launch
+  // sums the gradients of up to `hist` steps into a_k (K = steps m).  Within a
+  // block of `block` steps theta_k stays at the block's base: each step's dW
+  // sums the block's gradients so far (again K = steps m) and writes the bf16
+  // copy and, for what the forward reads in fp32 (biases, W_L), the working
+  // copy; the last one theta_k instead.
   const bool defer = h->hist > 1 && (int64_t)s * h->P * 4 > agn::kTcRedAccBytes;
   for (int i = 0; i < h->lam; ++i) {
     const int hi = defer ? i % h->hist : 0;   // this step's place in the history
+    const int bi = defer ? hi % h->block : 0;   // and in its block
+    const bool block_end = !defer || bi == h->block - 1 || hi == h->hist - 1 || i == h->lam - 1;
+    // the fp32 biases (and W_L) of this step's theta_k
+    const bool in_work = bi > 0;
+    float* const bias_base = in_work ? h->work : h->rep;
+    const int64_t bias_ld = in_work ? h->ld_work : h->P_pad;
+    auto bias_off = [&](int l) { return in_work ? h->wboff[l - 1] : h->boff[l - 1]; };
     auto Hl = [&](int l) -> void* {
       return static_cast<char*>(h->H[l]) + (int64_t)hi * n * m * h->dims[l] * (int64_t)sizeof(T);
     };
@@ -657,7 +674,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // is counted at its launch)
     const double acc_b = h->elide || defer ? 0.0 : h->acc_first && i == 0 ? 4.0 : 8.0;
     const double upd = h->adam ? 4.0
-                       : theta_share * (h->prec == AGN_PREC_BF16 ? 10.0 : 8.0) + acc_b;
+                       : theta_share * ((block_end ? 8.0 : 4.0) +
+                                        (h->prec == AGN_PREC_BF16 ? 2.0 : 0.0)) + acc_b;
     // this local step's buffer of layer 1's tensor-core operand
     const bool alt = h->early_gather && h->gparity;
     const agn_handle::LayerMaps& l1 = alt ? h->l1_alt : h->tmaps.empty() ? h->l1_alt : h->tmaps[0];
@@ -695,8 +713,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         agn::HeadArgs a{};
         const int fi = h->dims[L - 1], C = h->dims[L];
         a.H = L == 1 ? h->Xb : Hl(L - 1);
-        a.W = W; a.theta = h->rep; a.ld_param = h->P_pad;
-        a.woff = h->woff[L - 1]; a.boff = h->boff[L - 1];
+        a.W = W; a.theta = bias_base; a.ld_param = h->P_pad; a.ld_theta = bias_ld;
+        a.woff = h->woff[L - 1]; a.boff = bias_off(L);
         a.K = fi; a.C = C; a.m = m;
         a.slot_worker = sw; a.yb = h->yb;
         a.slot_t0 = st0; a.x_shard = h->direct_x ? h->S : 0;
@@ -750,9 +768,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           t.M = fo; t.N = m; t.K = fi;
           t.a_by_worker = 1;
           t.out = Hl(l); t.ldo = fo; t.out_bstride = (int64_t)m * fo;
-          t.relu = 1; t.boff = h->boff[l - 1];
+          t.theta = bias_base; t.ld_param = bias_ld;
+          t.relu = 1; t.boff = bias_off(l);
           t.out_pieces = h_pieces; t.out_plane = (int64_t)n * m * fo;
-          t.head_woff = h->woff[L - 1]; t.head_boff = h->boff[L - 1]; t.head_C = C;
+          t.head_woff = in_work ? h->wwoff : h->woff[L - 1]; t.head_boff = bias_off(L); t.head_C = C;
           t.yb = h->yb;
           t.dzl = dZl(L); t.ldz = h->ldz_out;
           t.dzl_pieces = (h->fuse_out_dw && h->split) ? h->dZp[L] : nullptr;
@@ -787,7 +806,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           t.a_by_worker = 1;
           t.out = Hl(l);
           t.ldo = fo; t.out_bstride = (int64_t)m * fo;
-          t.relu = 1; t.boff = h->boff[l - 1];
+          t.theta = bias_base; t.ld_param = bias_ld;
+          t.relu = 1; t.boff = bias_off(l);
           t.out_pieces = h_pieces; t.out_plane = (int64_t)n * m * fo;
           const auto& mp = maps_of(l);
           t.x_b_direct = l == 1;
@@ -887,7 +907,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           const auto& mp = maps_of(l);
           tc_dw.push_back({h->split ? &mp.h_mn32 : &mp.h_mn, h->split ? &mp.dz_mn32 : &mp.dz_mn,
                            &mp.theta, &mp.acc, fi, fo, h->woff[l - 1], h->boff[l - 1],
-                           l == 1 ? 1 : 0});
+                           l == 1 ? 1 : 0, h->work ? h->wboff[l - 1] : 0, -1});
           tc_flops += flops;
           tc_bytes += bytes;
         }
@@ -897,7 +917,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         const auto& mp = h->out_maps;
         tc_dw.insert(tc_dw.begin(), {h->split ? &mp.h_mn32 : &mp.h_mn,
                                      h->split ? &mp.dz_mn32 : &mp.dz_mn, &mp.theta, &mp.acc, fi,
-                                     fo, h->woff[l - 1], h->boff[l - 1]});
+                                     fo, h->woff[l - 1], h->boff[l - 1], 0,
+                                     h->work ? h->wboff[l - 1] : 0, h->wwoff});
         tc_flops += flops;
         tc_bytes += bytes;
         continue;
@@ -928,8 +949,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       }
     }
     if (!tc_dw.empty() && !(defer && acc_only)) {
-      Launch k(h, AGN_K_BACKWARD_DW, tc_flops, tc_bytes, launches);
-      agn::TcArgs t = tc_args(h, sw, st0, i, hi * n);
+      Launch k(h, AGN_K_BACKWARD_DW, tc_flops * (bi + 1), tc_bytes, launches);
+      agn::TcArgs t = tc_args(h, sw, st0, i - bi, (hi - bi) * n);
+      t.hist_steps = bi + 1; t.z_step = n;
+      t.theta_work = block_end ? nullptr : h->work; t.ld_work = h->ld_work;
       t.K = m; t.eta = eta;
       if (defer) t.acc = nullptr;
       if (acc_only) {
@@ -941,7 +964,7 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
                                   h->num_sms));
     }
-    if (defer && (hi == h->hist - 1 || i == h->lam - 1)) {   // a_k of the kept steps
+    if (defer && !h->elide && (hi == h->hist - 1 || i == h->lam - 1)) {   // a_k of the kept steps
       Launch k(h, AGN_K_BACKWARD_DW, tc_flops * (hi + 1), (double)s * h->P * (i > hi ? 8.0 : 4.0),
                launches);
       agn::TcArgs t = tc_args(h, sw, st0, i - hi, 0);
@@ -1447,13 +1470,23 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     else AGN_TRY(dalloc(h, &h->Xb_alt, (size_t)(n * m * d0) * es));
   }
   AGN_TRY(dalloc_t(h, &h->yb, (size_t)(n * (h->direct_x ? h->S + m : m))));
-  if (h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam && !h->elide &&
+  if (h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam &&
       h->lam > 1 && m <= kHistMaxBatch && n * h->P * 4 > agn::kTcRedAccBytes) {
     // no more than twice the accumulators' memory
     int64_t per = h->ldz_out;
     for (int l = 1; l < h->L; ++l) per += 2 * dims[l];
     h->hist = (int)std::min<int64_t>(std::min(h->lam, kHistMaxSteps),
                                      std::max<int64_t>(1, 8 * h->P / (2 * m * per)));
+  }
+  if (h->hist > 1) {
+    h->block = m <= 96 ? 4 : m <= 160 ? 3 : 2;
+    for (int l = 1; l <= h->L; ++l) {
+      h->wboff.push_back(h->ld_work);
+      h->ld_work += round_up(dims[l], 64);
+    }
+    h->wwoff = h->ld_work;
+    h->ld_work += round_up((int64_t)dims[h->L] * dims[h->L - 1], 64);
+    AGN_TRY(dalloc_t(h, &h->work, (size_t)(n * h->ld_work)));
   }
   const int64_t nh = n * h->hist;
   h->H.assign(h->L, nullptr);

@@ -84,6 +84,7 @@ struct HeadArgs {
   const void* W;           // replica operand base [n][ld_param] (T); W_L at woff, [C][K]
   const float* theta;      // fp32 masters (bias b_L at boff)
   int64_t ld_param, woff, boff;
+  int64_t ld_theta;        // row stride of theta (ld_param: W's)
   int K, C, m;
   const int* slot_worker;
   const int* yb;           // labels [slots][m]

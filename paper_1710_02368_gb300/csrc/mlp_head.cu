@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
   float ce = 0.f;
   if (active) {
     const int j = j0 + sj;
-    const float* bias = a.theta + (int64_t)w * a.ld_param + a.boff;
+    const float* bias = a.theta + (int64_t)w * a.ld_theta + a.boff;
     float zc[kMaxC];
 #pragma unroll
     for (int c = 0; c < kMaxC; ++c) {

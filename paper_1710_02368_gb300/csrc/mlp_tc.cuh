@@ -101,6 +101,12 @@ struct TcArgs {
   int acc_ring;
   // dW: 1 stores a_k = g (the first local step of a commit), whatever a_k held
   int acc_set;
+  // dW without accumulator: theta_work != null leaves theta_k at the base of its
+  // block of local steps and writes the updated low-precision copy, and to
+  // theta_work [n][ld_work] what the forward reads in fp32: the biases and the
+  // output layer's weights (DwLayerMaps::wboff / wwoff)
+  float* theta_work;
+  int64_t ld_work;
   // dW: slots with slot_repull[slot] != 0 take no local step, only a_k (their
   // replica is pulled anew before anything reads it); null = none
   const int* slot_repull;
@@ -157,6 +163,7 @@ struct DwLayerMaps {
   int M, N;
   int64_t woff, boff;
   int a_direct = 0;   // h_mn is a padded-shard map (layer 1; args.x_shard > 0)
+  int64_t wboff = 0, wwoff = -1;   // places of b_l and W_l (-1: none) in theta_work
 };
 // Accumulators (bytes) above which a wave streams them from DRAM: a dW launch
 // then takes a_k through the parameter ring, not by L2 adds, or, in bf16 mode,

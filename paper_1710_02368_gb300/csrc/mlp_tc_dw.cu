@@ -77,8 +77,9 @@ constexpr int kThrottleTiles = 8;              // tiles per CTA from which opera
 // through the ring beside theta_k's and stored back (3 slots); kDwUpd = the
 // local step without accumulator (elided: commits from a pull snapshot),
 // theta_k alone (6 slots); kDwGrad = the raw gradient only, stored for a
-// separate optimizer kernel (no chunks).
-enum { kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3 };
+// separate optimizer kernel (no chunks); kDwKeep = kDwUpd that leaves theta_k at
+// the base of its block of local steps (bf16 mode, args.theta_work).
+enum { kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4 };
 template <int BN, int kSplit, int kStages, int kBKs, int kMode>
 struct DwCfg {
   static constexpr bool kAcc = kMode == kDwUpdAcc || kMode == kDwUpdRed;   // a_k += g
@@ -119,6 +120,7 @@ struct DwLayer {
   int tile_begin;    // first tile of this layer in the launch
   int a_direct;      // A = the padded shards' rows of the slot's minibatch (layer 1)
   int64_t woff, boff;
+  int64_t wboff, wwoff;   // in theta_work
 };
 struct DwBatch {
   CUtensorMap a[kMaxDwLayers], b[kMaxDwLayers], th[kMaxDwLayers], ac[kMaxDwLayers];
@@ -187,7 +189,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
   // a slot whose replica nothing reads before its next pull: a_k only (or,
   // where this launch keeps no a_k, nothing)
   auto acc_only = [&](int slot) -> bool {
-    return (kMode == kDwUpdRed || kMode == kDwUpd) && args.slot_repull &&
+    return (kMode == kDwUpdRed || kMode == kDwUpd || kMode == kDwKeep) && args.slot_repull &&
            AGN_LD(args.slot_repull + slot) != 0;
   };
   // k steps of one local step's minibatch, and of the whole launch
@@ -457,6 +459,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
     const int g = warp & 3, hf = (warp - 2) >> 2;
     float* gS = reinterpret_cast<float*>(smem + Cfg::kGOff) + (warp - 2) * (16 * 32);
     const float eta = args.eta;
+    // theta_k left at its base: biases and W_L go to the working copy
+    constexpr bool keep = kMode == kDwKeep;
     uint32_t ch = 0;
     bool ok = true;
     int it = 0;
@@ -480,10 +484,12 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
                              (uint32_t)(16 * hf);
       const int64_t rbase = (int64_t)worker * args.ld_param;
       float* theta = args.theta + rbase;
+      float* work = keep ? args.theta_work + (int64_t)worker * args.ld_work : nullptr;
+      float* ww = keep && L.wwoff >= 0 ? work + L.wwoff : nullptr;
       float* acc = kAcc ? args.acc + rbase : nullptr;
       bf16* tb = args.theta_b ? args.theta_b + rbase : nullptr;   // bf16 mode only
       const bool grad_only = kGrad || acc_only(ti.slot);
-      const int nch = grad_only && kMode == kDwUpd
+      const int nch = grad_only && !kAcc && !kGrad
                           ? 0 : min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
       const bool grad_add = kGrad ? args.grad_add != 0 : !args.acc_set;
       for (int c = 0; c < nch; ++c) {
@@ -546,7 +552,12 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
               tn[2] = local_step(tv.z, eta, gv.z);
               tn[3] = local_step(tv.w, eta, gv.w);
               const int64_t p = L.woff + (int64_t)(fbase + i) * M + k0 + k4;
-              AGN_ST(reinterpret_cast<float4*>(theta + p), make_float4(tn[0], tn[1], tn[2], tn[3]));
+              if (!keep)
+                AGN_ST(reinterpret_cast<float4*>(theta + p),
+                       make_float4(tn[0], tn[1], tn[2], tn[3]));
+              else if (ww)   // the output layer
+                AGN_ST(reinterpret_cast<float4*>(ww + (p - L.woff)),
+                       make_float4(tn[0], tn[1], tn[2], tn[3]));
               if (kAccRing) {
                 const float4 av = *reinterpret_cast<const float4*>(
                     reinterpret_cast<const float*>(slot + kChunkBytes) + so);
@@ -568,7 +579,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           const float gb = gS[lane * 32 + kb];
           const int64_t pb = L.boff + fbase + lane;
           const float tn = local_step(sTb[16 * hf + lane], eta, gb);
-          AGN_ST(theta + pb, tn);
+          AGN_ST(keep ? work + L.wboff + fbase + lane : theta + pb, tn);
           if (kAccRing) AGN_ST(acc + pb, sTb[kCF + 16 * hf + lane] + gb);
           else if (kAcc && args.acc_set) AGN_ST(acc + pb, gb);
           else if (kAcc) AGN_RED(acc + pb, gb);
@@ -645,6 +656,8 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
       L.woff = d.woff;
       L.a_direct = d.a_direct;
       L.boff = d.boff;
+      L.wboff = d.wboff;
+      L.wwoff = d.wwoff;
       L.mt = d.M / 128 + 1;          // rows 0 .. M, row M the bias
       L.nt = (d.N + bn - 1) / bn;
       acc_bytes += ((int64_t)d.M + 1) * d.N * 4 * slots;
@@ -667,6 +680,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     const bool ring = !args.acc_set && !args.slot_repull &&
                       (args.acc_ring || acc_bytes > kTcRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
+                     : args.theta_work ? kDwKeep
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
                                    : kDwUpdRed;
@@ -679,6 +693,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     } else {
       r = mode == kDwGrad     ? launch_dw<kTcDwBN, 1, 4, 64, kDwGrad>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpd>(batch, args, num_sms, st)
+          : mode == kDwKeep   ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpdAcc>(batch, args, num_sms, st)
                               : launch_dw<kTcDwBN, 1, 2, 64, kDwUpdRed>(batch, args, num_sms, st);
     }
