@@ -29,6 +29,8 @@ constexpr int kThreads = 256;
 // commit by commit (groups of one) left DRAM idle: 20.9 M parameters, 64 commits,
 // fp32 and bf16 pulls 3605 us (5.4 TB/s) against 3199 (6.1), without pulls 2610
 // against 1928 (4.4, 5.9 TB/s); 2^24 with a pull per commit 2700 against 2436.
+// (Elided commits load two vectors each: commit by commit 4143 us a pass of 64,
+// four at a time 4872.)
 // Short vectors (a few float4 per thread, the MLP workloads' commits): one
 // float4 per thread and the accumulator loads of eight commits in flight.
 constexpr int kLongUnroll = 2, kLongGroup = 4;
@@ -283,7 +285,7 @@ Status launch_commit_pull(const CommitPlan& plan, float* theta_c, float* acc, fl
   cudaError_t e;
 #define AGN_COMMIT_GO(C, E, RB, PL)                                                            \
   (shrt ? go(commit_pull_kernel<C, E, kShortUnroll, kShortGroup>, RB, PL)                       \
-        : go(commit_pull_kernel<C, E, kLongUnroll, kLongGroup>, RB, PL))
+        : go(commit_pull_kernel<C, E, kLongUnroll, E ? 1 : kLongGroup>, RB, PL))
   if (replicas_bf16 && piece_plane > 0)
     e = elide ? AGN_COMMIT_GO(3, true, replicas_bf16, piece_plane)
               : AGN_COMMIT_GO(3, false, replicas_bf16, piece_plane);
