@@ -21,6 +21,7 @@
 #include <exception>
 #include <string>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -233,6 +234,7 @@ struct agn_handle {
     CUtensorMap w_k, w_mn, h_k, h_mn, dz_k, dz_mn;
     CUtensorMap w_k256;          // split mode: w_k without swizzle, for column tiles of 256
     CUtensorMap theta, acc;      // fp32 W_l of every replica / accumulator, box {128, 32}
+    CUtensorMap mom1, mom2;      // Adam: the same of the moments
     CUtensorMap h_mn32, dz_mn32; // split mode: 32-sample boxes for the dW kernel
   };
   int num_sms = 148;
@@ -309,7 +311,8 @@ struct agn_handle {
   int* plan_worker = nullptr;
   int* plan_commit = nullptr;
   int* plan_repull = nullptr;
-  int64_t cap_plan = 0;       // entries of 20 bytes
+  float2* plan_corr = nullptr;   // Adam: [slots][lambda] bias corrections
+  int64_t cap_plan = 0;       // bytes
   int* pull_list = nullptr;   // [n]
   // host state
   std::vector<float> hX, htheta0;
@@ -481,9 +484,18 @@ Status build_tc_maps(agn_handle* h) {
   const int nh = n * h->hist;   // activation batches: slots of every kept local step
   constexpr uint32_t bn = agn::kTcBoxN;
   h->tmaps.assign(L - 1, {});
+  auto moments = [&](agn_handle::LayerMaps& mp, int l) -> Status {
+    if (!h->adam) return Status::Ok();
+    const uint64_t fi = h->dims[l - 1], fo = h->dims[l];
+    AGN_TRY(agn::make_tmap_f32_3d(&mp.mom1, h->mom1 + h->woff[l - 1], fi, fo, n, fi, h->P_pad,
+                                  128, 32));
+    return agn::make_tmap_f32_3d(&mp.mom2, h->mom2 + h->woff[l - 1], fi, fo, n, fi, h->P_pad, 128,
+                                 32);
+  };
   for (int l = 1; l < L; ++l) {
     const uint64_t fi = h->dims[l - 1], fo = h->dims[l];
     auto& mp = h->tmaps[l - 1];
+    AGN_TRY(moments(mp, l));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.theta, h->rep + h->woff[l - 1], fi, fo, n, fi, h->P_pad,
                                   128, 32));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.acc, h->acc + h->woff[l - 1], fi, fo, n, fi, h->P_pad,
@@ -559,6 +571,7 @@ Status build_tc_maps(agn_handle* h) {
   if (h->fuse_out_dw) {   // the output layer's dW tiles: M = d_{L-1} inputs, N = d_L
     const uint64_t fi = h->dims[L - 1], fo = h->dims[L], lz = (uint64_t)h->ldz_out;
     auto& mp = h->out_maps;
+    AGN_TRY(moments(mp, L));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.theta, h->rep + h->woff[L - 1], fi, fo, n, fi, h->P_pad,
                                   128, 32));
     AGN_TRY(agn::make_tmap_f32_3d(&mp.acc, h->acc + h->woff[L - 1], fi, fo, n, fi, h->P_pad,
@@ -647,6 +660,10 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
   // copy and, for what the forward reads in fp32 (biases, W_L), the working
   // copy; the last one theta_k instead.
   const bool defer = h->hist > 1 && (int64_t)s * h->P * 4 > agn::kTcRedAccBytes;
+  // Adam's step in the dW launch, when that covers every layer: the gradient
+  // takes no trip through memory (8 of 44 bytes per parameter) and a launch
+  // goes.
+  const bool adam_fused = h->adam && h->fuse_out_dw;
   for (int i = 0; i < h->lam; ++i) {
     const int hi = defer ? i % h->hist : 0;   // this step's place in the history
     const int bi = defer ? hi % h->block : 0;   // and in its block
@@ -673,7 +690,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // kernels only store the gradient, 4 bytes (the Adam kernel's own traffic
     // is counted at its launch)
     const double acc_b = h->elide || defer ? 0.0 : h->acc_first && i == 0 ? 4.0 : 8.0;
-    const double upd = h->adam ? 4.0
+    const double upd = adam_fused ? 24.0 + acc_b + (h->rep_b ? 2.0 : 0.0)
+                       : h->adam ? 4.0
                        : theta_share * ((block_end ? 8.0 : 4.0) +
                                         (h->prec == AGN_PREC_BF16 ? 2.0 : 0.0)) + acc_b;
     // this local step's buffer of layer 1's tensor-core operand
@@ -907,7 +925,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
           const auto& mp = maps_of(l);
           tc_dw.push_back({h->split ? &mp.h_mn32 : &mp.h_mn, h->split ? &mp.dz_mn32 : &mp.dz_mn,
                            &mp.theta, &mp.acc, fi, fo, h->woff[l - 1], h->boff[l - 1],
-                           l == 1 ? 1 : 0, h->work ? h->wboff[l - 1] : 0, -1});
+                           l == 1 ? 1 : 0, h->work ? h->wboff[l - 1] : 0, -1,
+                           &mp.mom1, &mp.mom2});
           tc_flops += flops;
           tc_bytes += bytes;
         }
@@ -918,7 +937,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         tc_dw.insert(tc_dw.begin(), {h->split ? &mp.h_mn32 : &mp.h_mn,
                                      h->split ? &mp.dz_mn32 : &mp.dz_mn, &mp.theta, &mp.acc, fi,
                                      fo, h->woff[l - 1], h->boff[l - 1], 0,
-                                     h->work ? h->wboff[l - 1] : 0, h->wwoff});
+                                     h->work ? h->wboff[l - 1] : 0, h->wwoff, &mp.mom1,
+                                     &mp.mom2});
         tc_flops += flops;
         tc_bytes += bytes;
         continue;
@@ -959,6 +979,12 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         t.grad_out = h->acc; t.grad_add = i > 0;
       } else {
         t.acc_set = h->acc_first && i == 0;
+        if (adam_fused) {
+          t.grad_out = nullptr;
+          t.mom1 = h->mom1; t.mom2 = h->mom2;
+          t.corr = h->plan_corr + (int64_t)wv.offset * h->lam; t.lam = h->lam;
+          t.beta1 = h->beta1; t.beta2 = h->beta2; t.eps = h->eps;
+        }
         if (last_acc && wv.repulls > 0) t.slot_repull = h->plan_repull + wv.offset;
       }
       AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
@@ -974,12 +1000,13 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
       AGN_TRY(agn::tc_backward_dw(tc_dw.data(), (int)tc_dw.size(), t, s, h->stream, h->split,
                                   h->num_sms));
     }
-    if (h->adam) {   // the local step: Adam on the gradients the dW kernels stored
+    if (h->adam && !adam_fused) {   // the local step: Adam on the gradients the dW kernels stored
       agn::AdamArgs ad{};
       ad.grad = h->grad; ad.theta = h->rep; ad.acc = h->elide ? nullptr : h->acc;
       ad.m = h->mom1; ad.v = h->mom2; ad.theta_b = h->rep_b; ad.piece_plane = h->piece_plane;
       ad.P = h->P_pad; ad.ld = h->P_pad;
-      ad.slot_worker = sw; ad.slot_t0 = st0; ad.step = i;
+      ad.slot_worker = sw; ad.step = i; ad.lam = h->lam;
+      ad.corr = h->plan_corr + (int64_t)wv.offset * h->lam;
       ad.acc_set = i == 0;
       ad.eta = eta; ad.beta1 = h->beta1; ad.beta2 = h->beta2; ad.eps = h->eps;
       const double copy_b = h->rep_b ? 2.0 : 0.0;
@@ -1145,6 +1172,25 @@ Status build_plan(const agn_handle* h, int k, const int32_t* worker, const int32
   return Status::Ok();
 }
 
+// Adam's bias corrections 1 / (1 - beta^t) of every slot's local steps t = t0 + 1
+// .. t0 + lambda, out [slots][lambda]; workers at the same step share one
+// computation.
+void adam_corrections(const agn_handle* h, const std::vector<long long>& t0, float2* out) {
+  std::unordered_map<long long, size_t> seen;
+  for (size_t s = 0; s < t0.size(); ++s) {
+    const auto first = seen.emplace(t0[s], s);
+    if (!first.second) {
+      std::memcpy(out + s * h->lam, out + first.first->second * h->lam, h->lam * sizeof(float2));
+      continue;
+    }
+    for (int i = 0; i < h->lam; ++i) {
+      const double t = (double)(t0[s] + i + 1);
+      out[s * h->lam + i] = make_float2((float)(1.0 / (1.0 - std::pow((double)h->beta1, t))),
+                                        (float)(1.0 / (1.0 - std::pow((double)h->beta2, t))));
+    }
+  }
+}
+
 // A tensor-core kernel gave up on a bounded wait: its error flag and the
 // arrival counters of CTAs that left tiles unfinished, cleared.
 Status clear_flags(agn_handle* h, bool timed_out) {
@@ -1176,26 +1222,34 @@ Status do_run(agn_handle* h, int k, const int32_t* worker, const int32_t* tau, i
     h->cap_commits = c1;
   }
   AGN_TRY(grow(h, &h->loss_parts, &h->cap_parts, (int64_t)k * h->lam * h->loss_q, 0));
-  if (total_slots > h->cap_plan) {
-    const int64_t cap = std::max(total_slots, 2 * h->cap_plan);
+  const int64_t plan_bytes =
+      total_slots * (kPlanEntry + (h->adam ? h->lam * (int64_t)sizeof(float2) : 0));
+  if (plan_bytes > h->cap_plan) {
+    const int64_t cap = std::max(plan_bytes, 2 * h->cap_plan);
     char* buf = nullptr;
-    AGN_TRY(dalloc_t(h, &buf, (size_t)cap * kPlanEntry));
+    AGN_TRY(dalloc_t(h, &buf, (size_t)cap));
     AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
     dfree(h, h->plan_t0);
     h->plan_t0 = reinterpret_cast<long long*>(buf);
     h->cap_plan = cap;
   }
   AGN_TRY(agn::bounds_upload(h->stream));   // bounds-checked build: buffers as grown
-  std::vector<char> packed((size_t)(total_slots * kPlanEntry));
+  std::vector<char> packed((size_t)plan_bytes);
   if (total_slots > 0) {
-    const size_t ts = (size_t)total_slots;
-    h->plan_worker = reinterpret_cast<int*>(h->plan_t0 + ts);
+    const size_t ts = (size_t)total_slots, corr_bytes = packed.size() - ts * kPlanEntry;
+    h->plan_corr = reinterpret_cast<float2*>(h->plan_t0 + ts);
+    h->plan_worker = reinterpret_cast<int*>(reinterpret_cast<char*>(h->plan_corr) + corr_bytes);
     h->plan_commit = h->plan_worker + ts;
     h->plan_repull = h->plan_commit + ts;
-    std::memcpy(packed.data(), plan.slot_t0.data(), ts * sizeof(long long));
-    std::memcpy(packed.data() + ts * 8, plan.slot_worker.data(), ts * sizeof(int));
-    std::memcpy(packed.data() + ts * 12, plan.slot_commit.data(), ts * sizeof(int));
-    std::memcpy(packed.data() + ts * 16, plan.slot_repull.data(), ts * sizeof(int));
+    char* p = packed.data();
+    std::memcpy(p, plan.slot_t0.data(), ts * sizeof(long long));
+    p += ts * sizeof(long long);
+    if (h->adam) adam_corrections(h, plan.slot_t0, reinterpret_cast<float2*>(p));
+    p += corr_bytes;
+    for (const std::vector<int>* v : {&plan.slot_worker, &plan.slot_commit, &plan.slot_repull}) {
+      std::memcpy(p, v->data(), ts * sizeof(int));
+      p += ts * sizeof(int);
+    }
     AGN_TRY_CUDA(cudaMemcpyAsync(h->plan_t0, packed.data(), packed.size(), cudaMemcpyHostToDevice,
                                  h->stream));
   }

@@ -131,6 +131,17 @@ Status head_backward_dw(const HeadDwArgs& a, int slots, cudaStream_t st);
 template <typename T>
 bool head_fits(int K, int C);
 
+// Adam's step on one parameter: the moments m and v updated in place from the
+// raw gradient gr; returns g = -eta (m c1) / (sqrt(v c2) + eps), c1 and c2 the
+// bias corrections 1 / (1 - beta^t), computed on the host in double (a double pow
+// in the kernels cost them 3-5 us of latency a launch).
+__device__ __forceinline__ float adam_update(float gr, float& m, float& v, float eta, float b1,
+                                             float ob1, float b2, float ob2, float eps, float c1,
+                                             float c2) {
+  m = b1 * m + ob1 * gr;
+  v = b2 * v + ob2 * (gr * gr);
+  return -eta * (m * c1) / (sqrtf(v * c2) + eps);
+}
 // Adam as the local optimizer (optim.cu): from the raw gradients grad of the
 // wave's slots, the moments m, v and theta_k (a_k += the step, unless acc is
 // null; the bf16 copy or pieces of theta_k, unless theta_b is null).
@@ -145,8 +156,8 @@ struct AdamArgs {
   int64_t piece_plane;     // > 0: three pieces, planes this far apart
   int64_t P, ld;           // elements updated per replica (multiple of 4), row stride
   const int* slot_worker;
-  const long long* slot_t0;   // the worker's step counter before this wave
-  int step;                   // local step index within the wave
+  const float2* corr;      // [slots][lam] bias corrections of every local step
+  int lam, step;           // local step index within the wave
   float eta, beta1, beta2, eps;
 };
 Status adam_step(const AdamArgs& a, int slots, int num_sms, cudaStream_t st);

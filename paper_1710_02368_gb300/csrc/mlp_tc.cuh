@@ -50,6 +50,11 @@ struct TcArgs {
   // step.  grad_add: add it to what is there instead.
   float* grad_out;
   int grad_add;
+  // dW: Adam's step fused into the epilogue (DwLayerMaps::mom1 / mom2): the
+  // moments [n][ld_param]; null mom1 = no
+  float *mom1, *mom2;
+  const float2* corr;      // [slots][lam] bias corrections
+  float beta1, beta2, eps;
   // dW: the operands of hist_steps (0 or 1: one) consecutive local steps
   // beginning with `step`, kept z_step batches apart: their gradients summed
   int hist_steps, z_step;
@@ -164,6 +169,7 @@ struct DwLayerMaps {
   int64_t woff, boff;
   int a_direct = 0;   // h_mn is a padded-shard map (layer 1; args.x_shard > 0)
   int64_t wboff = 0, wwoff = -1;   // places of b_l and W_l (-1: none) in theta_work
+  const CUtensorMap *mom1 = nullptr, *mom2 = nullptr;   // Adam: as theta / acc
 };
 // Accumulators (bytes) above which a wave streams them from DRAM: a dW launch
 // then takes a_k through the parameter ring, not by L2 adds, or, in bf16 mode,

@@ -11,7 +11,7 @@
 //              boxes, MN-major, 128-byte swizzle) into a ring of stages, as
 //              fast as the MMA frees them, so the next tile's GEMM runs while
 //              the current tile's epilogue drains.
-//   warp 10    parameter producer: each tile's theta_k rows (and a_k's, for
+//   last warp  parameter producer: each tile's theta_k rows (and a_k's, for
 //              waves whose accumulators exceed 64 MB), 32 output features x
 //              128 inputs per chunk, into a second ring.  Each slot is
 //              refilled as soon as it frees, so DRAM reads of the next chunks
@@ -21,7 +21,7 @@
 //   warp 1     MMA issuer (one thread) and TMEM owner.  Two accumulators
 //              (double buffer): the GEMM of the next tile runs while the
 //              epilogue drains this one.
-//   warps 2-9  epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31, i.e.
+//   warps 2-9  (Adam: 2-17) epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31, i.e.
 //              32 consecutive inputs k of the tile, and 16 of the 32 features
 //              of a chunk; it transposes them through shared memory so that
 //              each lane updates four consecutive inputs of a feature at a
@@ -59,9 +59,7 @@ namespace agn {
 
 namespace {
 
-constexpr int kWarps = 11;
-constexpr int kEpiWarps = 8;
-constexpr int kThreads = 32 * kWarps;
+constexpr int kChunkWarps = 8;                 // epilogue warps on one parameter chunk
 constexpr int kCF = 32;                        // output features per parameter chunk
 constexpr int kChunkBytes = kCF * 128 * 4;     // one fp32 chunk: 32 rows x 128 inputs
 constexpr int kBiasHalf = kCF * 4;            // b_l (or its accumulator) for one chunk
@@ -78,15 +76,26 @@ constexpr int kThrottleTiles = 8;              // tiles per CTA from which opera
 // local step without accumulator (elided: commits from a pull snapshot),
 // theta_k alone (6 slots); kDwGrad = the raw gradient only, stored for a
 // separate optimizer kernel (no chunks); kDwKeep = kDwUpd that leaves theta_k at
-// the base of its block of local steps (bf16 mode, args.theta_work).
-enum { kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4 };
+// the base of its block of local steps (bf16 mode, args.theta_work); kDwAdam = Adam's step, theta_k and the
+// two moments per chunk through the ring (2 slots of 49 KB), the steps added
+// to a_k in the L2.
+enum {
+  kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5
+};
 template <int BN, int kSplit, int kStages, int kBKs, int kMode>
 struct DwCfg {
-  static constexpr bool kAcc = kMode == kDwUpdAcc || kMode == kDwUpdRed;   // a_k += g
+  static constexpr bool kAcc =                                             // a_k += g
+      kMode == kDwUpdAcc || kMode == kDwUpdRed || kMode == kDwAdam;
   static constexpr bool kAccRing = kMode == kDwUpdAcc;                     // a_k via the ring
-  static constexpr int kArrays = kAccRing ? 2 : 1;
+  // Adam's divisions and square roots keep eight warps busy: sixteen take every
+  // other chunk each (no gain without Adam: dW is not bound by its epilogue's chain)
+  static constexpr int kEpiWarps = kMode == kDwAdam ? 2 * kChunkWarps : kChunkWarps;
+  static constexpr int kWarps = kEpiWarps + 3;
+  static constexpr int kThreads = 32 * kWarps;
+  static constexpr int kArrays = kMode == kDwAdam ? 3 : kAccRing ? 2 : 1;
   static constexpr int kSlotBytes = kArrays * (kChunkBytes + kBiasHalf);
-  static constexpr int kRing = kMode == kDwGrad ? 1 : kAccRing ? 3 : 6;   // (kDwGrad: unused)
+  static constexpr int kRing =                                             // (kDwGrad: unused)
+      kMode == kDwGrad ? 1 : kMode == kDwAdam ? 2 : kAccRing ? 3 : 6;
   static constexpr int kBK = kBKs;
   static constexpr int kBox = kBK * 128;
   static constexpr int kABytes = 2 * kBox;
@@ -123,7 +132,9 @@ struct DwLayer {
   int64_t wboff, wwoff;   // in theta_work
 };
 struct DwBatch {
-  CUtensorMap a[kMaxDwLayers], b[kMaxDwLayers], th[kMaxDwLayers], ac[kMaxDwLayers];
+  CUtensorMap a[kMaxDwLayers], b[kMaxDwLayers], th[kMaxDwLayers];
+  CUtensorMap ac[kMaxDwLayers];    // accumulators, or Adam's first moments
+  CUtensorMap ac2[kMaxDwLayers];   // Adam's second moments
   DwLayer layer[kMaxDwLayers];
   int n_layers, total_tiles;
 };
@@ -159,10 +170,12 @@ __device__ __forceinline__ void write_ones_row(uint8_t* sa, int r) {
 }
 
 template <int BN, int kSplit, int kStages, int kBKs, int kMode>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(DwCfg<BN, kSplit, kStages, kBKs, kMode>::kThreads, 1)
 tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
   using Cfg = DwCfg<BN, kSplit, kStages, kBKs, kMode>;
   constexpr bool kAcc = Cfg::kAcc, kAccRing = Cfg::kAccRing, kGrad = kMode == kDwGrad;
+  constexpr bool kAdam = kMode == kDwAdam;
+  constexpr int kWarps = Cfg::kWarps, kEpiWarps = Cfg::kEpiWarps;
   constexpr int kRing = Cfg::kRing, kSlotBytes = Cfg::kSlotBytes;
   constexpr int kBK = Cfg::kBK, kABytes = Cfg::kABytes, kBox = Cfg::kBox;
   extern __shared__ uint8_t smem_raw[];
@@ -171,9 +184,9 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::kBarOff);
   uint64_t* empty = full + kStages;
   uint64_t* cfull = empty + kStages;     // parameter chunk landed
-  uint64_t* cempty = cfull + kRing;      // parameter chunk consumed (8 epilogue warps)
+  uint64_t* cempty = cfull + kRing;      // parameter chunk consumed (its 8 epilogue warps)
   uint64_t* tfull = cempty + kRing;      // accumulator b complete
-  uint64_t* tempty = tfull + 2;          // accumulator b drained (8 epilogue warps)
+  uint64_t* tempty = tfull + 2;          // accumulator b drained (every epilogue warp)
   uint64_t* fin = tempty + 2;            // MMA drain on abort
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(fin + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
@@ -203,7 +216,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
     }
     for (int r = 0; r < kRing; ++r) {
       tc::mbar_init(&cfull[r], 1);
-      tc::mbar_init(&cempty[r], kEpiWarps);
+      tc::mbar_init(&cempty[r], kChunkWarps);
     }
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(&tfull[b], 1);
@@ -218,6 +231,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       tc::tma_prefetch_desc(&B.b[i]);
       tc::tma_prefetch_desc(&B.th[i]);
       tc::tma_prefetch_desc(&B.ac[i]);
+      if (kAdam) tc::tma_prefetch_desc(&B.ac2[i]);
     }
   }
   if (warp == 1) {
@@ -331,25 +345,27 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         constexpr int kA = Cfg::kArrays;
         tc::mbar_arrive_expect_tx(&cfull[r], kA * (kChunkBytes + (bias_tile ? kBiasHalf : 0)));
         tc::tma_load_3d(dst, &B.th[ti.layer], &cfull[r], ti.m_tile * 128, f0, worker);
-        if (kAccRing)
+        if (kAccRing || kAdam)
           tc::tma_load_3d(dst + kChunkBytes, &B.ac[ti.layer], &cfull[r], ti.m_tile * 128, f0,
+                          worker);
+        if (kAdam)
+          tc::tma_load_3d(dst + 2 * kChunkBytes, &B.ac2[ti.layer], &cfull[r], ti.m_tile * 128, f0,
                           worker);
         if (bias_tile) {   // b_l[f0 .. f0 + 31] and its accumulator (within the replica)
           const int64_t pb = (int64_t)worker * args.ld_param + L.boff + f0;
-          if (AGN_BOUNDS_OK(args.theta + pb, kBiasHalf)) {
-            tc::bulk_load(dst + kA * kChunkBytes, args.theta + pb, kBiasHalf, &cfull[r]);
-          } else {   // bounds-checked build: account for the bytes, skip the copy
-            AGN_BOUNDS_FAIL(args.theta + pb);
-            tc::mbar_complete_tx(&cfull[r], kBiasHalf);
-          }
-          if (kAccRing) {
-            if (AGN_BOUNDS_OK(args.acc + pb, kBiasHalf)) {
-              tc::bulk_load(dst + kA * kChunkBytes + kBiasHalf, args.acc + pb, kBiasHalf,
-                            &cfull[r]);
-            } else {
-              AGN_BOUNDS_FAIL(args.acc + pb);
+          auto bias = [&](const float* src, int array) {
+            if (AGN_BOUNDS_OK(src, kBiasHalf)) {
+              tc::bulk_load(dst + kA * kChunkBytes + array * kBiasHalf, src, kBiasHalf, &cfull[r]);
+            } else {   // bounds-checked build: account for the bytes, skip the copy
+              AGN_BOUNDS_FAIL(src);
               tc::mbar_complete_tx(&cfull[r], kBiasHalf);
             }
+          };
+          bias(args.theta + pb, 0);
+          if (kAccRing) bias(args.acc + pb, 1);
+          if (kAdam) {
+            bias(args.mom1 + pb, 1);
+            bias(args.mom2 + pb, 2);
           }
         }
       };
@@ -451,12 +467,18 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       }
     }
   } else {
-    // epilogue warps 2..9: warp w reads TMEM lane quadrant w % 4 (inputs
+    // epilogue warps (from 2): warp w reads TMEM lane quadrant w % 4 (inputs
     // 32 (w % 4) .. + 31 of the tile) and columns 16 hf .. + 15 of each chunk,
-    // hf = (w - 2) / 4.  It stages its 16 x 32 gradients in shared memory
+    // hf = (w - 2) / 4 mod 2.  It stages its 16 x 32 gradients in shared memory
     // (feature-major), then each lane updates four consecutive inputs of four
     // features with 16-byte shared loads and 16-byte global stores.
-    const int g = warp & 3, hf = (warp - 2) >> 2;
+    // Of sixteen warps, the first eight take the even chunks (ch % 2 == 0): a ring
+    // of an even number of slots keeps every slot with one half, which waits for
+    // the slot's phases in order.
+    const int g = warp & 3, hf = ((warp - 2) >> 2) & 1;
+    constexpr bool kHalves = kEpiWarps > kChunkWarps;
+    static_assert(!kHalves || kRing % 2 == 0, "one half of the warps per ring slot");
+    const uint32_t odd = (uint32_t)(warp - 2) / kChunkWarps;
     float* gS = reinterpret_cast<float*>(smem + Cfg::kGOff) + (warp - 2) * (16 * 32);
     const float eta = args.eta;
     // theta_k left at its base: biases and W_L go to the working copy
@@ -470,6 +492,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       const DwLayer& L = B.layer[ti.layer];
       const int M = L.M, N = L.N;
       const int worker = AGN_LD(args.slot_worker + ti.slot);
+      const float2 cc = kAdam ? AGN_LD(args.corr + (int64_t)ti.slot * args.lam + args.step)
+                              : make_float2(0.f, 0.f);
       const int b = it & 1;
       // waits are warp-uniform: a lane that gave up takes its whole warp out
       // before the next .sync.aligned TMEM load
@@ -486,13 +510,22 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       float* theta = args.theta + rbase;
       float* work = keep ? args.theta_work + (int64_t)worker * args.ld_work : nullptr;
       float* ww = keep && L.wwoff >= 0 ? work + L.wwoff : nullptr;
-      float* acc = kAcc ? args.acc + rbase : nullptr;
+      float* acc = kAcc && args.acc ? args.acc + rbase : nullptr;   // (Adam elided: none)
+      float *mom1 = args.mom1 + rbase, *mom2 = args.mom2 + rbase;   // Adam only
+      auto adam = [&](float gr, float& m, float& v) {
+        return adam_update(gr, m, v, eta, args.beta1, 1.0f - args.beta1, args.beta2,
+                           1.0f - args.beta2, args.eps, cc.x, cc.y);
+      };
       bf16* tb = args.theta_b ? args.theta_b + rbase : nullptr;   // bf16 mode only
       const bool grad_only = kGrad || acc_only(ti.slot);
       const int nch = grad_only && !kAcc && !kGrad
                           ? 0 : min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
       const bool grad_add = kGrad ? args.grad_add != 0 : !args.acc_set;
       for (int c = 0; c < nch; ++c) {
+        if (kHalves && (ch & 1) != odd) {   // the other half's chunk
+          ++ch;
+          continue;
+        }
         const int r = ch % kRing;
         uint32_t v[16];
         tc::tmem_ld_32x32b_x16(tbase + (uint32_t)(c * kCF), v);
@@ -542,16 +575,34 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           for (int u = 0; u < 4; ++u) {
             const int i = i0 + 4 * u;                           // feature fbase + i
             if (fbase + i < N) {
-              const float4 gv = *reinterpret_cast<const float4*>(gS + i * 32 + k4);
+              float4 gv = *reinterpret_cast<const float4*>(gS + i * 32 + k4);
               const int so = (16 * hf + i) * 128 + 32 * g + k4;   // in the fp32 chunks
               const float4 tv = *reinterpret_cast<const float4*>(
                   reinterpret_cast<const float*>(slot) + so);
               float tn[4];
-              tn[0] = local_step(tv.x, eta, gv.x);
-              tn[1] = local_step(tv.y, eta, gv.y);
-              tn[2] = local_step(tv.z, eta, gv.z);
-              tn[3] = local_step(tv.w, eta, gv.w);
               const int64_t p = L.woff + (int64_t)(fbase + i) * M + k0 + k4;
+              if constexpr (kAdam) {   // g is then the step: a_k += g, theta_k += g
+                const float4 m4 = *reinterpret_cast<const float4*>(
+                    reinterpret_cast<const float*>(slot + kChunkBytes) + so);
+                const float4 v4 = *reinterpret_cast<const float4*>(
+                    reinterpret_cast<const float*>(slot + 2 * kChunkBytes) + so);
+                float mm[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
+                gv.x = adam(gv.x, mm[0], vv[0]);
+                gv.y = adam(gv.y, mm[1], vv[1]);
+                gv.z = adam(gv.z, mm[2], vv[2]);
+                gv.w = adam(gv.w, mm[3], vv[3]);
+                AGN_ST(reinterpret_cast<float4*>(mom1 + p), make_float4(mm[0], mm[1], mm[2], mm[3]));
+                AGN_ST(reinterpret_cast<float4*>(mom2 + p), make_float4(vv[0], vv[1], vv[2], vv[3]));
+                tn[0] = tv.x + gv.x;
+                tn[1] = tv.y + gv.y;
+                tn[2] = tv.z + gv.z;
+                tn[3] = tv.w + gv.w;
+              } else {
+                tn[0] = local_step(tv.x, eta, gv.x);
+                tn[1] = local_step(tv.y, eta, gv.y);
+                tn[2] = local_step(tv.z, eta, gv.z);
+                tn[3] = local_step(tv.w, eta, gv.w);
+              }
               if (!keep)
                 AGN_ST(reinterpret_cast<float4*>(theta + p),
                        make_float4(tn[0], tn[1], tn[2], tn[3]));
@@ -563,7 +614,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
                     reinterpret_cast<const float*>(slot + kChunkBytes) + so);
                 AGN_ST(reinterpret_cast<float4*>(acc + p),
                        make_float4(av.x + gv.x, av.y + gv.y, av.z + gv.z, av.w + gv.w));
-              } else if (kAcc) {   // a_k += g in the L2 (one add per element and launch)
+              } else if (kAcc && acc) {   // a_k += g in the L2 (one add per element and launch)
                 if (args.acc_set) AGN_ST(reinterpret_cast<float4*>(acc + p), gv);
                 else AGN_RED4(acc + p, gv);
               }
@@ -576,13 +627,22 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         if (kb >= 0 && kb < 32 && lane < 16 && fbase + lane < N) {   // bias row: b_l[f]
           const float* sTb =
               reinterpret_cast<const float*>(slot + Cfg::kArrays * kChunkBytes);
-          const float gb = gS[lane * 32 + kb];
+          float gb = gS[lane * 32 + kb];
           const int64_t pb = L.boff + fbase + lane;
-          const float tn = local_step(sTb[16 * hf + lane], eta, gb);
+          float tn;
+          if constexpr (kAdam) {
+            float mb = sTb[kCF + 16 * hf + lane], vb = sTb[2 * kCF + 16 * hf + lane];
+            gb = adam(gb, mb, vb);
+            AGN_ST(mom1 + pb, mb);
+            AGN_ST(mom2 + pb, vb);
+            tn = sTb[16 * hf + lane] + gb;
+          } else {
+            tn = local_step(sTb[16 * hf + lane], eta, gb);
+          }
           AGN_ST(keep ? work + L.wboff + fbase + lane : theta + pb, tn);
           if (kAccRing) AGN_ST(acc + pb, sTb[kCF + 16 * hf + lane] + gb);
-          else if (kAcc && args.acc_set) AGN_ST(acc + pb, gb);
-          else if (kAcc) AGN_RED(acc + pb, gb);
+          else if (kAcc && acc && args.acc_set) AGN_ST(acc + pb, gb);
+          else if (kAcc && acc) AGN_RED(acc + pb, gb);
           if (kSplit == 1) AGN_ST(tb + pb, __float2bfloat16_rn(tn));
         }
         __syncwarp();
@@ -627,7 +687,7 @@ Status launch_dw(const DwBatch& batch, const TcArgs& args, int num_sms, cudaStre
   const int grid = std::min(batch.total_tiles, num_sms);
   {
     auto kf = kern;
-    AGN_TRY_CUDA(launch_pdl(kf, grid, kThreads, Cfg::kSmem, st, batch, args));
+    AGN_TRY_CUDA(launch_pdl(kf, grid, Cfg::kThreads, Cfg::kSmem, st, batch, args));
   }
   AGN_TRY_CUDA(cudaGetLastError());
   return Status::Ok();
@@ -649,7 +709,8 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
       batch.a[i] = *d.h_mn;
       batch.b[i] = *d.dz_mn;
       batch.th[i] = *d.theta;
-      batch.ac[i] = *d.acc;
+      batch.ac[i] = args.mom1 ? *d.mom1 : *d.acc;
+      if (args.mom1) batch.ac2[i] = *d.mom2;
       DwLayer& L = batch.layer[i];
       L.M = d.M;
       L.N = d.N;
@@ -680,6 +741,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     const bool ring = !args.acc_set && !args.slot_repull &&
                       (args.acc_ring || acc_bytes > kTcRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
+                     : args.mom1  ? kDwAdam
                      : args.theta_work ? kDwKeep
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
@@ -687,11 +749,13 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     Status r = Status::Ok();
     if (split) {
       r = mode == kDwGrad     ? launch_dw<kTcDwBNSplit, 3, 4, 32, kDwGrad>(batch, args, num_sms, st)
+          : mode == kDwAdam   ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwAdam>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpd>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdAcc>(batch, args, num_sms, st)
                               : launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdRed>(batch, args, num_sms, st);
     } else {
       r = mode == kDwGrad     ? launch_dw<kTcDwBN, 1, 4, 64, kDwGrad>(batch, args, num_sms, st)
+          : mode == kDwAdam   ? launch_dw<kTcDwBN, 1, 2, 64, kDwAdam>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpd>(batch, args, num_sms, st)
           : mode == kDwKeep   ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpdAcc>(batch, args, num_sms, st)

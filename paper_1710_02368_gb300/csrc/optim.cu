@@ -7,7 +7,7 @@
 //   a += g (unless the accumulator is elided),  theta_k += g,
 // then the bf16 copy (or the three pieces) of theta_k.  m and v belong to the
 // worker and persist across its commits.  One pass over the replica, 16-byte
-// accesses; the bias corrections are computed once per block in double.
+// accesses; the bias corrections come from the host.
 #include "mlp.cuh"
 
 namespace agn {
@@ -41,14 +41,8 @@ __global__ void __launch_bounds__(kOptThreads) adam_kernel(const AdamArgs a) {
   pdl_wait_only();   // the next forward may read theta_k before its own wait
   const int z = blockIdx.y;
   const int w = AGN_LD(a.slot_worker + z);
-  __shared__ float s_c1, s_c2;
-  if (threadIdx.x == 0) {
-    const double t = (double)(AGN_LD(a.slot_t0 + z) + a.step + 1);
-    s_c1 = (float)(1.0 / (1.0 - pow((double)a.beta1, t)));
-    s_c2 = (float)(1.0 / (1.0 - pow((double)a.beta2, t)));
-  }
-  __syncthreads();
-  const float c1 = s_c1, c2 = s_c2;
+  const float2 cc = AGN_LD(a.corr + (int64_t)z * a.lam + a.step);
+  const float c1 = cc.x, c2 = cc.y;
   const float b1 = a.beta1, b2 = a.beta2, ob1 = 1.0f - a.beta1, ob2 = 1.0f - a.beta2;
   const int64_t base = (int64_t)w * a.ld;
   const int64_t n4 = a.P / 4;
@@ -64,9 +58,7 @@ __global__ void __launch_bounds__(kOptThreads) adam_kernel(const AdamArgs a) {
     float th[4] = {t4.x, t4.y, t4.z, t4.w}, u[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      mm[e] = b1 * mm[e] + ob1 * gr[e];
-      vv[e] = b2 * vv[e] + ob2 * (gr[e] * gr[e]);
-      u[e] = -a.eta * (mm[e] * c1) / (sqrtf(vv[e] * c2) + a.eps);
+      u[e] = adam_update(gr[e], mm[e], vv[e], a.eta, b1, ob1, b2, ob2, a.eps, c1, c2);
       th[e] = th[e] + u[e];
     }
     AGN_ST(reinterpret_cast<float4*>(a.m + p), make_float4(mm[0], mm[1], mm[2], mm[3]));
