@@ -1293,24 +1293,35 @@ Status make_tmap_f32_3d(CUtensorMap* map, const void* base, uint64_t inner, uint
                 swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-// Two 128-row tiles per CTA (kMT = 2) for the bf16 forward and dX when the
-// one-tile launch would need more than one round of CTAs on the SMs (full
-// waves): each B stage then feeds twice the MMAs, and the CTAs of a full
-// wave halve.  Not with split K, nor with column tiles under 128 (there the
-// weights, read once anyway, dominate the stages' bytes).
-bool use_row_pairs(const TcArgs& args, int slots, bool split, int bn) {
-  if (split || bn < 128 || args.ksplit > 1 || args.one_row_tile) return false;
-  static int sms = 0;
-  if (sms == 0) {
+// More than one round of one-tile CTAs on the SMs (full waves).
+bool full_wave(const TcArgs& args, int slots, int bn) {
+  static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       (void)cudaGetLastError();
-      return false;
+      return 1 << 30;
     }
-    sms = n;
-  }
+    return n;
+  }();
   return ceil_div(args.M, 128) * ceil_div(args.N, bn) * (int64_t)slots > sms;
+}
+
+// Two 128-row tiles per CTA (kMT = 2) for the bf16 forward and dX of full
+// waves: each B stage then feeds twice the MMAs, and the CTAs of a full
+// wave halve.  Not with split K, nor with column tiles under 128 (there the
+// weights, read once anyway, dominate the stages' bytes).
+bool use_row_pairs(const TcArgs& args, int slots, bool split, int bn) {
+  return !split && bn >= 128 && args.ksplit <= 1 && !args.one_row_tile &&
+         full_wave(args, slots, bn);
+}
+
+// The bf16 forward and dX of full waves with column tiles of 64: three stages
+// instead of six, so that two CTAs share an SM and one's epilogue and
+// prologue overlap the other's stream of weights (both together keep as many
+// bytes in flight).  64 slots of 4096-4096-10, m = 64: FWDUS.
+bool use_two_ctas(const TcArgs& args, int slots, int bn) {
+  return bn == 64 && args.ksplit <= 1 && full_wave(args, slots, bn);
 }
 
 Status tc_forward(const CUtensorMap& w_k, const CUtensorMap& h_k, const TcArgs& args, int slots,
@@ -1324,6 +1335,8 @@ Status tc_forward(const CUtensorMap& w_k, const CUtensorMap& h_k, const TcArgs& 
     if (bn == 128) return launch_tc<128, false, false, kEpiFwd, 4, 1, 2>(w_k, h_k, args, slots, st);
     return launch_tc<256, false, false, kEpiFwd, 3, 1, 2>(w_k, h_k, args, slots, st);
   }
+  if (use_two_ctas(args, slots, bn))
+    return launch_tc<64, false, false, kEpiFwd, 3, 1>(w_k, h_k, args, slots, st);
   if (bn == 64) return launch_tc<64, false, false, kEpiFwd, 6, 1>(w_k, h_k, args, slots, st);
   if (bn == 128) return launch_tc<128, false, false, kEpiFwd, 5, 1>(w_k, h_k, args, slots, st);
   return launch_tc<256, false, false, kEpiFwd, 4, 1>(w_k, h_k, args, slots, st);
@@ -1362,6 +1375,8 @@ Status tc_backward_dx(const CUtensorMap& w_mn, const CUtensorMap& dz_k, const Tc
     if (bn == 128) return launch_tc<128, true, false, kEpiDX, 4, 1, 2>(w_mn, dz_k, args, slots, st);
     return launch_tc<256, true, false, kEpiDX, 3, 1, 2>(w_mn, dz_k, args, slots, st);
   }
+  if (use_two_ctas(args, slots, bn))
+    return launch_tc<64, true, false, kEpiDX, 3, 1>(w_mn, dz_k, args, slots, st);
   if (bn == 64) return launch_tc<64, true, false, kEpiDX, 6, 1>(w_mn, dz_k, args, slots, st);
   if (bn == 128) return launch_tc<128, true, false, kEpiDX, 5, 1>(w_mn, dz_k, args, slots, st);
   return launch_tc<256, true, false, kEpiDX, 4, 1>(w_mn, dz_k, args, slots, st);
