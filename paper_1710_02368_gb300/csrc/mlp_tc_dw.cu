@@ -95,7 +95,7 @@ struct DwCfg {
   static constexpr int kArrays = kMode == kDwAdam ? 3 : kAccRing ? 2 : 1;
   static constexpr int kSlotBytes = kArrays * (kChunkBytes + kBiasHalf);
   static constexpr int kRing =                                             // (kDwGrad: unused)
-      kMode == kDwGrad ? 1 : kMode == kDwAdam ? 2 : kAccRing ? 3 : 6;
+      kMode == kDwGrad ? 1 : kMode == kDwAdam ? 2 : kAccRing ? 3 : kStages > 2 ? 4 : 6;
   static constexpr int kBK = kBKs;
   static constexpr int kBox = kBK * 128;
   static constexpr int kABytes = 2 * kBox;
@@ -747,7 +747,15 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
                      : ring        ? kDwUpdAcc
                                    : kDwUpdRed;
     Status r = Status::Ok();
-    if (split) {
+    // fp32, long minibatches (a tile's GEMM reads eight stages or more): a third
+    // operand stage for two of the six chunks in flight.  784-1000-1000-10, 4 slots, us a launch at
+    // m = 256, 300, 512: 43.0, 49.1, 70.0 with two stages, 40.5, 45.6, 61.5 with three
+    // (42.9, 46.9, 60.9 with four stages and one chunk)
+    const bool deep = split && ceil_div(args.K, 32) * std::max(1, args.hist_steps) >= 8;
+    if (deep && (mode == kDwUpd || mode == kDwUpdRed)) {
+      r = mode == kDwUpd ? launch_dw<kTcDwBNSplit, 3, 3, 32, kDwUpd>(batch, args, num_sms, st)
+                         : launch_dw<kTcDwBNSplit, 3, 3, 32, kDwUpdRed>(batch, args, num_sms, st);
+    } else if (split) {
       r = mode == kDwGrad     ? launch_dw<kTcDwBNSplit, 3, 4, 32, kDwGrad>(batch, args, num_sms, st)
           : mode == kDwAdam   ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwAdam>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpd>(batch, args, num_sms, st)
