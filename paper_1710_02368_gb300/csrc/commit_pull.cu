@@ -95,11 +95,16 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
        base += stride) {
     int64_t idx[kUnroll];
     bool live[kUnroll];
+    bool skip[kUnroll];   // kLowPull pulls leave the fp32 replica alone here
     float4 th[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       idx[u] = base + (int64_t)u * kThreads;
       live[u] = idx[u] < n4;
+      skip[u] = false;
+      if (kCopy == 1 && !kElide)
+        for (int r = 0; r < plan.n_skip; ++r)
+          skip[u] = skip[u] || (idx[u] >= plan.skip_lo[r] && idx[u] < plan.skip_hi[r]);
       if (live[u]) th[u] = AGN_LD(th4 + idx[u]);
     }
     // commits in groups of kGroup: every accumulator load of a group is in
@@ -152,11 +157,13 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
                       make_float4(0.f, 0.f, 0.f, 0.f));
         }
         for (int p = plan.pull_begin[c]; p < plan.pull_begin[c + 1]; ++p) {
-          const int64_t row = (int64_t)plan.pull_worker[p] * ld;
+          const int32_t pw = plan.pull_worker[p];
+          const int64_t row = (int64_t)(pw & ~kLowPull) * ld;
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u) {
             if (!live[u]) continue;
-            AGN_ST(reinterpret_cast<float4*>(replicas + row) + idx[u], th[u]);
+            if (!(pw & kLowPull) || !skip[u])
+              AGN_ST(reinterpret_cast<float4*>(replicas + row) + idx[u], th[u]);
             if (kElide) AGN_ST(reinterpret_cast<float4*>(acc + row) + idx[u], th[u]);
             if (kCopy == 1)
               AGN_ST(reinterpret_cast<uint2*>(rep_bf16 + row) + idx[u], pack_bf16x4(th[u]));
@@ -192,7 +199,7 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
         if (cc == c) sq[cc] += (double)(d * d);
       if (!kElide && zero_acc) AGN_ST(ap, 0.f);
       for (int p = plan.pull_begin[c]; p < plan.pull_begin[c + 1]; ++p) {
-        const int64_t row = (int64_t)plan.pull_worker[p] * ld;
+        const int64_t row = (int64_t)(plan.pull_worker[p] & ~kLowPull) * ld;
         AGN_ST(replicas + row + i, t);
         if (kElide) AGN_ST(acc + row + i, t);
         if (kCopy == 1) AGN_ST(rep_bf16 + row + i, __float2bfloat16_rn(t));

@@ -153,14 +153,22 @@ constexpr int kMaxCommitsPerLaunch = 16;
 // Pulls one launch may do in total.
 constexpr int kMaxPullsPerLaunch = 256;
 
+// A pull whose worker reads the bf16 copy of the hidden layers' weights alone
+// (flag in CommitPlan::pull_worker).
+constexpr int32_t kLowPull = 1 << 30;
+constexpr int kMaxSkipRanges = 8;
+
 struct CommitPlan {
   int32_t n_commits;                       // <= kMaxCommitsPerLaunch
   int32_t worker[kMaxCommitsPerLaunch];    // accumulator committed by commit c
   int32_t pull_begin[kMaxCommitsPerLaunch + 1];
-  int32_t pull_worker[kMaxPullsPerLaunch];
+  int32_t pull_worker[kMaxPullsPerLaunch];  // + kLowPull: see skip_lo
   int32_t norm_slot[kMaxCommitsPerLaunch]; // index of commit c in the norm output
   int32_t per_commit_scale;                // 1: commit c uses scale[c], else the launch's
   float scale[kMaxCommitsPerLaunch];
+  // fp32 ranges [lo, hi) in float4 units that kLowPull pulls leave alone
+  int32_t n_skip;
+  int32_t skip_lo[kMaxSkipRanges], skip_hi[kMaxSkipRanges];
 };
 
 // The pulls of a standalone call that decide its replicas: each worker's last
