@@ -76,20 +76,25 @@ constexpr int kThrottleTiles = 8;              // tiles per CTA from which opera
 // local step without accumulator (elided: commits from a pull snapshot),
 // theta_k alone (6 slots); kDwGrad = the raw gradient only, stored for a
 // separate optimizer kernel (no chunks); kDwKeep = kDwUpd that leaves theta_k at
-// the base of its block of local steps (bf16 mode, args.theta_work); kDwAdam = Adam's step, theta_k and the
-// two moments per chunk through the ring (2 slots of 49 KB), the steps added
-// to a_k in the L2.
+// the base of its block of local steps (bf16 mode, args.theta_work; kDwKeep8 on
+// eight epilogue warps); kDwAdam = Adam's step, theta_k and the two moments per
+// chunk through the ring (2 slots of 49 KB), the steps added to a_k in the L2.
 enum {
-  kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5
+  kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5, kDwKeep8 = 6
 };
+constexpr bool is_keep(int mode) { return mode == kDwKeep || mode == kDwKeep8; }
 template <int BN, int kSplit, int kStages, int kBKs, int kMode>
 struct DwCfg {
   static constexpr bool kAcc =                                             // a_k += g
       kMode == kDwUpdAcc || kMode == kDwUpdRed || kMode == kDwAdam;
   static constexpr bool kAccRing = kMode == kDwUpdAcc;                     // a_k via the ring
-  // Adam's divisions and square roots keep eight warps busy: sixteen take every
-  // other chunk each (no gain without Adam: dW is not bound by its epilogue's chain)
-  static constexpr int kEpiWarps = kMode == kDwAdam ? 2 * kChunkWarps : kChunkWarps;
+  // Sixteen epilogue warps, every other chunk each, where eight are what bounds
+  // the launch: Adam's divisions and square roots (91 us a launch with eight, 75
+  // with sixteen), and theta_k kept at its base with short minibatches (m = 64:
+  // 1644 and 1595 us; m = 256, kDwKeep8: 950 and 983).  The other modes are bound
+  // by DRAM or latency: no gain.
+  static constexpr int kEpiWarps =
+      kMode == kDwAdam || kMode == kDwKeep ? 2 * kChunkWarps : kChunkWarps;
   static constexpr int kWarps = kEpiWarps + 3;
   static constexpr int kThreads = 32 * kWarps;
   static constexpr int kArrays = kMode == kDwAdam ? 3 : kAccRing ? 2 : 1;
@@ -202,7 +207,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
   // a slot whose replica nothing reads before its next pull: a_k only (or,
   // where this launch keeps no a_k, nothing)
   auto acc_only = [&](int slot) -> bool {
-    return (kMode == kDwUpdRed || kMode == kDwUpd || kMode == kDwKeep) && args.slot_repull &&
+    return (kMode == kDwUpdRed || kMode == kDwUpd || is_keep(kMode)) && args.slot_repull &&
            AGN_LD(args.slot_repull + slot) != 0;
   };
   // k steps of one local step's minibatch, and of the whole launch
@@ -482,7 +487,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
     float* gS = reinterpret_cast<float*>(smem + Cfg::kGOff) + (warp - 2) * (16 * 32);
     const float eta = args.eta;
     // theta_k left at its base: biases and W_L go to the working copy
-    constexpr bool keep = kMode == kDwKeep;
+    constexpr bool keep = is_keep(kMode);
     uint32_t ch = 0;
     bool ok = true;
     int it = 0;
@@ -742,7 +747,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
                       (args.acc_ring || acc_bytes > kTcRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
                      : args.mom1  ? kDwAdam
-                     : args.theta_work ? kDwKeep
+                     : args.theta_work ? (args.K <= 96 ? kDwKeep : kDwKeep8)
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
                                    : kDwUpdRed;
@@ -766,6 +771,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
           : mode == kDwAdam   ? launch_dw<kTcDwBN, 1, 2, 64, kDwAdam>(batch, args, num_sms, st)
           : mode == kDwUpd    ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpd>(batch, args, num_sms, st)
           : mode == kDwKeep   ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep>(batch, args, num_sms, st)
+          : mode == kDwKeep8  ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep8>(batch, args, num_sms, st)
           : mode == kDwUpdAcc ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpdAcc>(batch, args, num_sms, st)
                               : launch_dw<kTcDwBN, 1, 2, 64, kDwUpdRed>(batch, args, num_sms, st);
     }
