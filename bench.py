@@ -249,7 +249,7 @@ def commit_plan_launches(order, pulls, max_commits=16, max_pulls=256):
 def commit_pass_bytes(P, n_commits, n_pulls, launches):
     """Bytes one pass of the standalone commit workload must move: theta~ read
     and written once per launch (8P), each commit's accumulator read and
-    zeroed (8P), each pull's replica written (4P)."""
+    zeroed (8P), each pulled replica written (4P)."""
     return float(P) * (8.0 * launches + 8.0 * n_commits + 4.0 * n_pulls)
 
 
@@ -286,7 +286,8 @@ def commit_kernel_bench(agn, torch, dev, P, min_ms=200.0):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     launches = commit_plan_launches(order, pulls)
-    bytes_ = commit_pass_bytes(P, n, len(flat), launches)
+    # (a replica pulled several times in the pass is written once, at its last pull)
+    bytes_ = commit_pass_bytes(P, n, len(np.unique(flat)), launches)
     del theta, acc, reps_t
     torch.cuda.empty_cache()
     return {"P": P, "commits": n, "pulls_per_commit": wl.pulls_per_commit, "passes_timed": reps,
@@ -345,6 +346,11 @@ def roofline(wl, kst, worker_steps, on_tc, hbm, bf16, peak_src):
     impl_bytes = d["bytes"] / launches
     mb = method_bytes_per_worker_step(wl, dom, fused_head=kst["forward_head"]["launches"] > 0)
     method_bytes = mb * worker_steps / launches if mb is not None else impl_bytes
+    # (large bf16 waves keep a_k and, inside a block of local steps, theta_k out
+    # of DRAM: the launch then moves less than the method's per-step bytes, and
+    # the fraction is of what it moves)
+    kept = dom == "backward_dw" and impl_bytes < method_bytes
+    method_bytes = min(method_bytes, impl_bytes) if kept else method_bytes
     flops = d["flops"] / launches
     # fp32 mode on the tensor cores issues six bf16 piece products per fp32 product
     mma_per_flop = 6.0 if (wl.precision == WL.PREC_FP32 and on_tc) else 1.0
@@ -361,7 +367,8 @@ def roofline(wl, kst, worker_steps, on_tc, hbm, bf16, peak_src):
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["kernel"] = dom
     roof["avg_launch_us"] = 1e6 * sec
-    roof["bytes_basis"] = ("method: fp32 theta_k and a_k read-modify-write per parameter and "
+    roof["bytes_basis"] = ("implementation bytes (fewer than the method's)" if kept else
+                           "method: fp32 theta_k and a_k read-modify-write per parameter and "
                            "local step (16 B; 18 B with the bf16 copy) plus the GEMM operands at "
                            "the mode's element size" if dom == "backward_dw" else
                            "method: the class's weights and activations at the mode's element "
