@@ -906,7 +906,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
     // dW: the output layer, then the hidden layers (on the tensor cores, all
     // in one persistent launch)
     std::vector<agn::DwLayerMaps> tc_dw;
-    double tc_flops = 0.0, tc_bytes = 0.0;
+    std::vector<agn::GemmArgs> simt_dw;   // and the CUDA-core layers, in one launch too
+    double tc_flops = 0.0, tc_bytes = 0.0, simt_flops = 0.0, simt_bytes = 0.0;
     for (int l = L; l >= 1; --l) {
       const int fi = h->dims[l - 1], fo = h->dims[l];
       const void* Hprev = l == 1 ? h->Xb : Hl(l - 1);
@@ -947,8 +948,8 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         tc_bytes += bytes;
         continue;
       }
-      Launch k(h, AGN_K_BACKWARD_DW, flops, bytes, launches);
       if (l == L && h->use_head) {   // narrow output layer
+        Launch k(h, AGN_K_BACKWARD_DW, flops, bytes, launches);
         agn::HeadDwArgs d{};
         d.H = Hprev; d.dZL = dZl(l); d.slot_worker = sw;
         d.theta = h->rep; d.acc = h->elide ? nullptr : h->acc; d.theta_b = h->rep_b;
@@ -969,8 +970,14 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
         g.piece_plane = h->piece_plane;
         g.woff = h->woff[l - 1]; g.boff = h->boff[l - 1]; g.eta = eta;
         g.grad_out = h->adam ? h->grad : nullptr;
-        AGN_TRY(agn::simt_backward_dw<T>(g, s, h->stream));
+        simt_dw.push_back(g);
+        simt_flops += flops;
+        simt_bytes += bytes;
       }
+    }
+    if (!simt_dw.empty()) {
+      Launch k(h, AGN_K_BACKWARD_DW, simt_flops, simt_bytes, launches);
+      AGN_TRY(agn::simt_backward_dw<T>(simt_dw.data(), (int)simt_dw.size(), s, h->stream));
     }
     if (!tc_dw.empty() && !(defer && acc_only)) {
       // (the block's earlier steps multiplied again are no work of the method)

@@ -49,8 +49,9 @@ template <typename T>
 Status simt_forward(const GemmArgs& g, bool last, int slots, cudaStream_t st);
 template <typename T>
 Status simt_backward_dx(const GemmArgs& g, int slots, cudaStream_t st);
+// The dW of n_layers layers in one launch (every dZ complete).
 template <typename T>
-Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st);
+Status simt_backward_dw(const GemmArgs* layers, int n_layers, int slots, cudaStream_t st);
 // Softmax cross-entropy of a wave's logits: dZ = (softmax(Z) - onehot(y)) / m
 // and the loss of every 32-sample chunk of a slot, its cross-entropy sum / m,
 // at loss_parts[(slot_commit[z] * lam + step) * ceil(m / 32) + chunk].

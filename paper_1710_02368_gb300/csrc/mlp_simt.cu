@@ -58,17 +58,16 @@ __device__ __forceinline__ void write_copy(bf16* tb, int64_t plane, int64_t p, f
 // 10000 rows 20 -> 26 TFLOP/s.  A thread's rows are consecutive (its A
 // values come in 16-byte loads), its columns 16 apart (coalesced epilogues).
 template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
-__global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
+__device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, int tile_x, int tile_y) {
   constexpr int kBM = kTile, kBN = kTile, kBK = kTile == 32 ? 32 : 16;
   constexpr int kTM = kTile / 16, kTN = kTile / 16;
   constexpr int kLoads = kTile * kBK / kThreads;   // per operand, thread and slice
   constexpr int kLd = kTile + 4;
-  pdl_begin();
   __shared__ __align__(16) float As[2][kBK][kLd];
   __shared__ __align__(16) float Bs[2][kBK][kLd];
   const int z = blockIdx.z;
   const int w = AGN_LD(g.slot_worker + z);
-  const int64_t m0 = (int64_t)blockIdx.y * kBM, n0 = (int64_t)blockIdx.x * kBN;
+  const int64_t m0 = (int64_t)tile_y * kBM, n0 = (int64_t)tile_x * kBN;
   const T* A = reinterpret_cast<const T*>(g.a) + (g.a_by_worker ? (int64_t)w : z) * g.a_bstride;
   const T* B = reinterpret_cast<const T*>(g.b) + (g.b_by_worker ? (int64_t)w : z) * g.b_bstride;
   const int tid = threadIdx.x;
@@ -80,7 +79,7 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
 #pragma unroll
     for (int j = 0; j < kTN; ++j) acc[i][j] = 0.f;
   float bsum = 0.f;   // bias gradient (kEpi == kEpiDW, first column tile)
-  const bool do_bias = (kEpi == kEpiDW) && blockIdx.x == 0 && tid < kBM;
+  const bool do_bias = (kEpi == kEpiDW) && tile_x == 0 && tid < kBM;
 
   // element r of this thread in a k slice: row (or column) o and k
   auto place = [&](bool k_major, int r, int& o, int& kk) {
@@ -256,6 +255,32 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
   }
 }
 
+template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
+__global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
+  pdl_begin();
+  gemm_simt_tile<T, TO, kAKMajor, kBKMajor, kEpi, kTile>(g, blockIdx.x, blockIdx.y);
+}
+
+// The weight gradients of several layers in one launch (they depend on no other
+// layer's): layer i's tiles are blocks first[i] .. first[i + 1] - 1, columns
+// fastest.
+constexpr int kDwLayers = 8;
+struct DwLayers {
+  GemmArgs g[kDwLayers];
+  int first[kDwLayers + 1];
+  int n;
+};
+template <typename T, int kTile>
+__global__ void __launch_bounds__(kThreads)
+dw_simt_kernel(const __grid_constant__ DwLayers batch) {
+  pdl_begin();
+  int i = 0;
+  while (i + 1 < batch.n && (int)blockIdx.x >= batch.first[i + 1]) ++i;
+  const GemmArgs& g = batch.g[i];
+  const int t = (int)blockIdx.x - batch.first[i], cols = (int)((g.N + kTile - 1) / kTile);
+  gemm_simt_tile<T, T, false, false, kEpiDW, kTile>(g, t % cols, t / cols);
+}
+
 // Softmax cross-entropy (SoftmaxArgs).  A block takes a 32-sample chunk of a
 // slot (one block per slot took 38 us a launch at 4 slots x 512 samples x 10
 // classes): up to kXentClasses classes pass through shared memory, copied in
@@ -407,11 +432,7 @@ __global__ void __launch_bounds__(256) gather4_kernel(const T* __restrict__ X,
   if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// The largest tile (fewest shared-memory reads per multiply-add) that still
-// gives every SM a block or, of 128, one and a half; small launches take small tiles, since a block's
-// chain over k is then what bounds them.
-template <typename T, typename TO, bool kAK, bool kBK, int kEpi>
-Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
+int simt_sms() {
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -419,6 +440,15 @@ Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
       (void)cudaGetLastError();
     return std::max(n, 1);
   }();
+  return sms;
+}
+
+// The largest tile (fewest shared-memory reads per multiply-add) that still
+// gives every SM a block or, of 128, one and a half; small launches take small
+// tiles, since a block's chain over k is then what bounds them.
+template <typename T, typename TO, bool kAK, bool kBK, int kEpi>
+Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
+  const int sms = simt_sms();
   auto blocks = [&](int t) { return ceil_div(g.N, t) * ceil_div(g.M, t) * (int64_t)slots; };
   auto go = [&](auto kf, int t) -> Status {
     dim3 grid((unsigned)ceil_div(g.N, t), (unsigned)ceil_div(g.M, t), (unsigned)slots);
@@ -443,8 +473,33 @@ Status simt_backward_dx(const GemmArgs& g, int slots, cudaStream_t st) {
   return launch_gemm<T, T, true, false, kEpiDX>(g, slots, st);
 }
 template <typename T>
-Status simt_backward_dw(const GemmArgs& g, int slots, cudaStream_t st) {
-  return launch_gemm<T, T, false, false, kEpiDW>(g, slots, st);
+Status simt_backward_dw(const GemmArgs* layers, int n_layers, int slots, cudaStream_t st) {
+  for (int l0 = 0; l0 < n_layers; l0 += kDwLayers) {
+    DwLayers batch{};
+    batch.n = std::min(kDwLayers, n_layers - l0);
+    auto fill = [&](int tile) -> int64_t {   // the layers' tiles; their number
+      int64_t tiles = 0;
+      for (int i = 0; i < batch.n; ++i) {
+        const GemmArgs& g = batch.g[i] = layers[l0 + i];
+        batch.first[i] = (int)tiles;
+        tiles += ceil_div(g.N, tile) * ceil_div(g.M, tile);
+      }
+      batch.first[batch.n] = (int)tiles;
+      return tiles;
+    };
+    // tiles as in launch_gemm
+    int tile = 128;
+    int64_t tiles = fill(tile);
+    if (tiles * slots < 3 * simt_sms() / 2) tiles = fill(tile = 64);
+    if (tile == 64 && tiles * slots < simt_sms()) tiles = fill(tile = 32);
+    if (tiles > INT32_MAX) return Status::Err(AGN_E_UNSUPPORTED, "dW tile count overflows");
+    auto kf = tile == 128 ? dw_simt_kernel<T, 128>
+              : tile == 64 ? dw_simt_kernel<T, 64>
+                           : dw_simt_kernel<T, 32>;
+    AGN_TRY_CUDA(launch_pdl(kf, dim3((unsigned)tiles, 1, (unsigned)slots), kThreads, 0, st, batch));
+    AGN_TRY_CUDA(cudaGetLastError());
+  }
+  return Status::Ok();
 }
 template <typename T>
 Status softmax_xent(const SoftmaxArgs& a, int slots, cudaStream_t st) {
@@ -486,7 +541,7 @@ Status gather_batch(const T* X, const int* y, T* Xb, int* yb, int d0, int m, int
 #define AGN_INST(T)                                                                          \
   template Status simt_forward<T>(const GemmArgs&, bool, int, cudaStream_t);                 \
   template Status simt_backward_dx<T>(const GemmArgs&, int, cudaStream_t);                   \
-  template Status simt_backward_dw<T>(const GemmArgs&, int, cudaStream_t);                   \
+  template Status simt_backward_dw<T>(const GemmArgs*, int, int, cudaStream_t);              \
   template Status softmax_xent<T>(const SoftmaxArgs&, int, cudaStream_t);                    \
   template Status gather_batch<T>(const T*, const int*, T*, int*, int, int, int64_t,          \
                                   const int*, const long long*, int, int, cudaStream_t,       \
