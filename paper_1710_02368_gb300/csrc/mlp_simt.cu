@@ -54,12 +54,18 @@ __device__ __forceinline__ void write_copy(bf16* tb, int64_t plane, int64_t p, f
 // the next k slice's global loads are in flight while the current one is
 // multiplied out of shared memory.  Against one 64 x 64 tile, one buffer and
 // 4-byte shared loads: a forward of 613-301-150-26 at 5 slots of 100 samples
-// 31.1 -> 17.9 us, dX 15.8 -> 9.9, dW 15.3 -> 12.8; the 784-1000-1000 forward of
-// 10000 rows 20 -> 26 TFLOP/s.  A thread's rows are consecutive (its A
+// 31.1 -> 16.4 us, dX 15.8 -> 9.9, dW 46 -> 19 (its three launches in one); the
+// 784-1000-1000 forward of 10000 rows 20 -> 26 TFLOP/s.  A thread's rows are consecutive (its A
 // values come in 16-byte loads), its columns 16 apart (coalesced epilogues).
 template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
 __device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, int tile_x, int tile_y) {
-  constexpr int kBM = kTile, kBN = kTile, kBK = kTile == 32 ? 32 : 16;
+  constexpr int kBM = kTile, kBN = kTile;
+  // k per slice.  Small tiles wait on the next slice's loads: 64 (32: 5 % slower on
+  // 613-301-150-26's forwards).  32 for the fp32 dX at 64 x 64 (784-1001-1001-10, 8
+  // slots of 128: a pass 2.70 -> 2.56 ms); elsewhere 32 cost blocks an SM (bf16
+  // 333-777-29, 16 slots of 200: 1.87 -> 2.05 ms).
+  constexpr int kBK = kTile == 32 ? 64
+                      : kTile == 64 && kEpi == kEpiDX && sizeof(T) == 4 ? 32 : 16;
   constexpr int kTM = kTile / 16, kTN = kTile / 16;
   constexpr int kLoads = kTile * kBK / kThreads;   // per operand, thread and slice
   constexpr int kLd = kTile + 4;

@@ -1,5 +1,5 @@
 """The CUDA-core GEMMs at the edges of their tiles (32, 64 and 128 square, k
-slices of 32 and 16, csrc/mlp_simt.cu): minibatches and widths one below, at and
+slices of 64, 32 and 16, csrc/mlp_simt.cu): minibatches and widths one below, at and
 one above a tile, with enough workers that each tile size is taken.  Against the
 float64 oracle at the fp32 tolerances of the other parity tests, and, since
 every output is one chain over k in order whatever the tile, the same worker's
