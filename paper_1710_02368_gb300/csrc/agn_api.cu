@@ -1554,13 +1554,19 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     else AGN_TRY(dalloc(h, &h->Xb_alt, (size_t)(n * m * d0) * es));
   }
   AGN_TRY(dalloc_t(h, &h->yb, (size_t)(n * (h->direct_x ? h->S + m : m))));
+  size_t dev_free = 0, dev_total = 0;
+  AGN_TRY_CUDA(cudaMemGetInfo(&dev_free, &dev_total));
   if (h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam &&
       h->lam > 1 && m <= kHistMaxBatch && n * h->P * 4 > agn::kTcRedAccBytes) {
-    // no more than twice the accumulators' memory
+    // no more than twice the accumulators' memory or an eighth of the device's;
+    // none where it would take half of what is free (the handle needs no history)
     int64_t per = h->ldz_out;
     for (int l = 1; l < h->L; ++l) per += 2 * dims[l];
+    const int64_t step = 2 * n * m * per;
+    const int64_t most = std::min<int64_t>(8 * n * h->P, (int64_t)(dev_total / 8));
     h->hist = (int)std::min<int64_t>(std::min(h->lam, kHistMaxSteps),
-                                     std::max<int64_t>(1, 8 * h->P / (2 * m * per)));
+                                     std::max<int64_t>(1, most / step));
+    if (h->hist * step > (int64_t)(dev_free / 2)) h->hist = 1;
   }
   if (h->hist > 1) {
     h->block = m <= 96 ? 4 : m <= 160 ? 3 : 2;
@@ -1587,12 +1593,16 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     const int64_t E = h->n_eval;
     int maxh = 1;
     for (int l = 1; l < h->L; ++l) maxh = std::max(maxh, dims[l]);
-    // the tensor cores evaluate what they train; fewer, larger chunks keep
-    // every SM busy (300 MB of pieces at most, 4096 rows at least)
-    h->eval_tc = h->use_tc;
+    // the tensor cores evaluate what they train (unless the rows' pieces, half as
+    // large again as the rows, would take a quarter of what is free); fewer,
+    // larger chunks keep every SM busy (300 MB of pieces at most, 4096 rows at
+    // least)
+    AGN_TRY_CUDA(cudaMemGetInfo(&dev_free, &dev_total));
+    h->eval_tc = h->use_tc && 6 * E * d0 <= (int64_t)(dev_free / 4);
     h->eval_chunk = std::min<int64_t>(
         E, !h->eval_tc ? 4096 : std::max<int64_t>(4096, (48 << 20) / maxh / 256 * 256));
-    AGN_TRY(dalloc_t(h, &h->Xe, (size_t)(E * d0)));
+    const int64_t up = h->eval_tc ? std::min<int64_t>(E, 1 << 16) : E;   // rows uploaded at a time
+    AGN_TRY(dalloc_t(h, &h->Xe, (size_t)(up * d0)));
     AGN_TRY(dalloc_t(h, &h->ye, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->He[0], (size_t)(h->eval_chunk * maxh)));
     if (!h->eval_tc) AGN_TRY(dalloc_t(h, &h->He[1], (size_t)(h->eval_chunk * maxh)));
@@ -1602,7 +1612,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY(dalloc_t(h, &h->e_pred, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->e_out, 2));
     AGN_TRY(dalloc_t(h, &h->e_sw, 1));
-    AGN_TRY_CUDA(cudaMemcpy(h->Xe, hXe.data(), hXe.size() * sizeof(float), cudaMemcpyHostToDevice));
+    if (!h->eval_tc)
+      AGN_TRY_CUDA(cudaMemcpy(h->Xe, hXe.data(), hXe.size() * sizeof(float), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemcpy(h->ye, hye.data(), hye.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
     AGN_TRY_CUDA(cudaMemset(h->e_sw, 0, sizeof(int)));
     if (h->eval_tc) {
@@ -1610,8 +1621,13 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
       h->eval_plane = h->eval_chunk * maxh;
       for (bf16*& p : h->He_p) AGN_TRY(dalloc_t(h, &p, (size_t)(3 * h->eval_plane)));
       AGN_TRY(agn::bounds_upload(h->stream));
-      AGN_TRY(agn::split_pieces(h->Xe, h->Xe_p, E * d0, E * d0, h->stream));
-      AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+      for (int64_t r0 = 0; r0 < E; r0 += up) {
+        const int64_t count = std::min(up, E - r0) * d0;
+        AGN_TRY_CUDA(cudaMemcpyAsync(h->Xe, hXe.data() + r0 * d0, (size_t)count * sizeof(float),
+                                     cudaMemcpyHostToDevice, h->stream));
+        AGN_TRY(agn::split_pieces(h->Xe, h->Xe_p + r0 * d0, count, E * d0, h->stream));
+        AGN_TRY_CUDA(cudaStreamSynchronize(h->stream));
+      }
       dfree(h, h->Xe);
       h->Xe = nullptr;
       constexpr uint32_t bk = agn::kTcSplitBK, bn = agn::kTcBoxN;

@@ -24,7 +24,8 @@ def agn():
 
 CASES = [((8, 8, 2), 1), ((64, 48, 10), 63), ((64, 136, 4), 129), ((72, 264, 40, 16), 257),
          ((200, 1000, 1000, 10), 3001), ((64, 128, 128, 33), 700),
-         ((16, 4096, 10), 12288 + 37)]   # 48 Mi / 4096 rows a chunk, then 37
+         ((16, 4096, 10), 12288 + 37),   # 48 Mi / 4096 rows a chunk, then 37
+         ((8, 16, 3), 65536 + 5)]        # 64 Ki rows uploaded at a time, then 5
 
 
 @pytest.mark.parametrize("dims,rows", CASES)
