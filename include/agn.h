@@ -332,7 +332,7 @@ int agn_plan_waves(int32_t n_workers, int32_t lambda, int32_t n_commits, const i
  *     acc[k] = 0;  replica[p] = theta_c for every p in
  *     pull_workers[pull_offsets[c] .. pull_offsets[c+1]).
  *   (A replica pulled more than once in a call is written once, at its last
- *   pull.)
+ *   pull, while n is at most 4096 or 64 times the pulls; else at each.)
  *   theta_c   : device fp32 [P];  acc, replicas: device fp32 [n][ld],
  *               ld >= P, ld % 4 == 0, all three 16-byte aligned.
  *   replicas_bf16: optional device bf16 [n][ld] that receives bf16(theta_c)
@@ -361,10 +361,12 @@ int agn_commit_pull(float* theta_c, float* acc, float* replicas, void* replicas_
  * Same arguments, same kernels and bit-identical results as agn_commit_pull
  * (theta~, accumulators and replicas always; the norms too whenever the
  * commit kernel's grid fits the fixed array, i.e. on every GPU with at most
- * 256 SMs, GB300 included: they are then reduced in the same fixed order).  It allocates nothing: its scratch (the per-block
- * partial sums of the norms) is a fixed array of 16 x 1024 doubles
+ * 256 SMs, GB300 included: they are then reduced in the same fixed order).  It
+ * allocates nothing, on the device or on the host's heap: its scratch (the
+ * per-block partial sums of the norms) is a fixed array of 16 x 1024 doubles
  * (128 KiB) in device global memory that every GPU loading the library holds
- * until the process exits.
+ * until the process exits.  (A replica pulled more than once in a call is
+ * written once while n is at most 4096, else at each pull.)
  *   - Limit: each commit may have at most 256 pulls (more gives
  *     AGN_E_INVALID with a message saying so); P, C and n are otherwise free.
  *   - The first call on a device looks up the array's device address (with
@@ -374,7 +376,8 @@ int agn_commit_pull(float* theta_c, float* acc, float* replicas, void* replicas_
  *     (nothing in it needs to start at zero).  Calls that overlap on the GPU
  *     (other streams, other host threads) race on it and give wrong norms:
  *     order them on one stream or with events.
- * Errors: AGN_E_INVALID, AGN_E_CUDA, AGN_E_UNSUPPORTED (device ordinal > 63).
+ * Errors: AGN_E_INVALID, AGN_E_CUDA, AGN_E_UNSUPPORTED (device ordinal > 63),
+ * AGN_E_OOM (no host memory for the text of one of these errors).
  */
 int agn_commit_pull_noalloc(float* theta_c, float* acc, float* replicas, void* replicas_bf16,
                             int64_t P, int64_t ld, int32_t n, int32_t C,

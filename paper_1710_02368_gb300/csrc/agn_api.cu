@@ -27,6 +27,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "host_inputs.h"
+#include "last_pulls.h"
 #include "mlp.cuh"
 #include "mlp_tc.cuh"
 
@@ -1900,9 +1901,14 @@ Status commit_pull(float* theta_c, float* acc, float* reps, void* reps_b, int64_
     for (int p = po[c]; p < po[c + 1]; ++p)
       if (pw[p] < 0 || pw[p] >= n) return Status::Err(AGN_E_INVALID, "pull worker out of range");
   }
-  const agn::LastPulls pulls(n, C, po, pw);
-  po = pulls.offsets.data();
-  pw = pulls.workers.data();
+  // A table of every worker: on the stack, or, for more workers, on the heap
+  // where the pulls are not too few for many of them to repeat.
+  int32_t table[agn::kStackPullWorkers];
+  std::vector<int32_t> large;
+  if (n > agn::kStackPullWorkers && n <= 64 * (int64_t)po[C]) large.resize((size_t)n);
+  const agn::LastPulls pulls(pw, po[C], n <= agn::kStackPullWorkers ? table
+                                        : large.empty()            ? nullptr
+                                                                   : large.data());
   const float scale = (float)(normalize ? -(eta / (double)lambda) : -eta);
   const int grid = agn::commit_grid(P);
   double* partials = nullptr;
@@ -1962,7 +1968,7 @@ Status commit_pull(float* theta_c, float* acc, float* reps, void* reps_b, int64_
   for (int c = 0; c < C && result.ok(); ++c) {
     bool dup = false;
     for (int i = 0; i < cp.n_commits; ++i) dup |= cp.worker[i] == cw[c];
-    const int np = po[c + 1] - po[c];
+    const int np = pulls.count(po[c], po[c + 1]);
     if (cp.n_commits == agn::kMaxCommitsPerLaunch || dup ||
         (cp.n_commits > 0 && cp.pull_begin[cp.n_commits] + np > agn::kMaxPullsPerLaunch)) {
       result = flush();
@@ -1973,11 +1979,13 @@ Status commit_pull(float* theta_c, float* acc, float* reps, void* reps_b, int64_
     cp.norm_slot[i] = c;
     int pb = cp.pull_begin[i];
     int p = po[c];
-    for (; p < po[c + 1] && pb < agn::kMaxPullsPerLaunch; ++p) cp.pull_worker[pb++] = pw[p];
+    for (; p < po[c + 1] && pb < agn::kMaxPullsPerLaunch; ++p)
+      if (pulls.writes(p)) cp.pull_worker[pb++] = pw[p];
     cp.pull_begin[i + 1] = pb;
     cp.n_commits = i + 1;
-    if (p < po[c + 1]) {   // more pulls than one launch holds: finish them after it
-      for (; p < po[c + 1]; ++p) extra.push_back(pw[p]);
+    if (pulls.count(p, po[c + 1]) > 0) {   // more than one launch holds: finish them after it
+      for (; p < po[c + 1]; ++p)
+        if (pulls.writes(p)) extra.push_back(pw[p]);
       result = flush();
     }
   }

@@ -14,6 +14,7 @@
 #include <new>
 #include <string>
 
+#include "last_pulls.h"
 #include "mlp.cuh"
 
 namespace agn {
@@ -84,9 +85,9 @@ agn::Status commit_pull_noalloc(float* theta_c, float* acc, float* reps, void* r
     for (int p = po[c]; p < po[c + 1]; ++p)
       if (pw[p] < 0 || pw[p] >= n) return Status::Err(AGN_E_INVALID, "pull worker out of range");
   }
-  const agn::LastPulls pulls(n, C, po, pw);
-  po = pulls.offsets.data();
-  pw = pulls.workers.data();
+  // (more workers than the table holds: every pull is written, in order)
+  int32_t table[agn::kStackPullWorkers];
+  const agn::LastPulls pulls(pw, po[C], n <= agn::kStackPullWorkers ? table : nullptr);
   double* scratch = nullptr;
   AGN_TRY(scratch_on_current_device(&scratch));
   const float scale = (float)(normalize ? -(eta / (double)lambda) : -eta);
@@ -125,7 +126,7 @@ agn::Status commit_pull_noalloc(float* theta_c, float* acc, float* reps, void* r
   for (int c = 0; c < C; ++c) {
     bool dup = false;
     for (int i = 0; i < cp.n_commits; ++i) dup |= cp.worker[i] == cw[c];
-    const int np = po[c + 1] - po[c];
+    const int np = pulls.count(po[c], po[c + 1]);
     if (cp.n_commits == agn::kMaxCommitsPerLaunch || dup ||
         cp.pull_begin[cp.n_commits] + np > agn::kMaxPullsPerLaunch)
       AGN_TRY(flush());
@@ -133,7 +134,8 @@ agn::Status commit_pull_noalloc(float* theta_c, float* acc, float* reps, void* r
     cp.worker[i] = cw[c];
     cp.norm_slot[i] = c;
     int pb = cp.pull_begin[i];
-    for (int p = po[c]; p < po[c + 1]; ++p) cp.pull_worker[pb++] = pw[p];
+    for (int p = po[c]; p < po[c + 1]; ++p)
+      if (pulls.writes(p)) cp.pull_worker[pb++] = pw[p];
     cp.pull_begin[i + 1] = pb;
     cp.n_commits = i + 1;
   }

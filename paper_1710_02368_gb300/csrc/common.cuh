@@ -10,7 +10,6 @@
 #include <cstdio>
 #include <string>
 #include <utility>
-#include <vector>
 
 #include "../../include/agn.h"
 #include "bounds.cuh"
@@ -169,23 +168,6 @@ struct CommitPlan {
   // fp32 ranges [lo, hi) in float4 units that kLowPull pulls leave alone
   int32_t n_skip;
   int32_t skip_lo[kMaxSkipRanges], skip_hi[kMaxSkipRanges];
-};
-
-// The pulls of a standalone call that decide its replicas: each worker's last
-// one.  Nothing reads a replica between two pulls of one call, so the earlier
-// ones would only write bytes that a later one overwrites.  po [C + 1] and pw
-// as in agn_commit_pull (validated, workers < n); kept in the same order.
-struct LastPulls {
-  std::vector<int32_t> offsets, workers;
-  LastPulls(int n, int C, const int32_t* po, const int32_t* pw) : offsets((size_t)C + 1, 0) {
-    std::vector<int32_t> last(po[C] > 0 ? (size_t)n : 0);
-    for (int32_t p = 0; p < po[C]; ++p) last[pw[p]] = p;
-    for (int c = 0; c < C; ++c) {
-      for (int32_t p = po[c]; p < po[c + 1]; ++p)
-        if (last[pw[p]] == p) workers.push_back(pw[p]);
-      offsets[c + 1] = (int32_t)workers.size();
-    }
-  }
 };
 
 // Queue one fused launch for the commits of `plan` plus the partial-norm

@@ -1,7 +1,8 @@
 """A standalone call writes a replica once, at its worker's last pull
-(csrc/common.cuh, LastPulls): random pull lists with repeats within a commit and
+(csrc/last_pulls.h): random pull lists with repeats within a commit and
 across commits, against the float32 oracle that performs every pull in order;
-both entry points, with and without bf16 copies."""
+both entry points, with and without bf16 copies, with up to 4096 workers (the
+table on the stack) and more."""
 
 import numpy as np
 import pytest
@@ -22,7 +23,8 @@ def env():
 
 
 @pytest.mark.parametrize("P,n,C,most", [(1, 1, 1, 3), (1003, 3, 7, 4), (4099, 40, 33, 9),
-                                        (260, 300, 5, 200)])
+                                        (260, 300, 5, 200), (9, 4096, 6, 250),
+                                        (6, 5000, 20, 250), (3, 40000, 2, 20)])
 @pytest.mark.parametrize("noalloc", [False, True])
 @pytest.mark.parametrize("low", [False, True])
 def test_last_pull_wins(env, P, n, C, most, noalloc, low):
