@@ -153,8 +153,9 @@ constexpr int kMaxCommitsPerLaunch = 16;
 constexpr int kMaxPullsPerLaunch = 256;
 
 // A pull whose worker reads the bf16 copy of the hidden layers' weights alone
-// (flag in CommitPlan::pull_worker).
-constexpr int32_t kLowPull = 1 << 30;
+// (flag in CommitPlan::pull_worker: the sign bit, which no worker's index has;
+// the standalone calls take any non-negative one).
+constexpr int32_t kLowPull = INT32_MIN;
 constexpr int kMaxSkipRanges = 8;
 
 struct CommitPlan {

@@ -52,3 +52,28 @@ def test_last_pull_wins(env, P, n, C, most, noalloc, low):
         assert torch.equal(got, want), k
         if low:
             assert torch.equal(repb[k, :P].cpu(), want.to(torch.bfloat16)), k
+
+
+@pytest.mark.parametrize("P", [3, 4])   # the kernel's remainder loop, its vectors
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_worker_past_2_30_is_its_own_row(env, P, noalloc):
+    """Every index below n is a worker: row 2^30 is written, row 0 is not
+    (buffers of 16 GiB; only these rows are touched)."""
+    agn, torch, dev = env
+    n, ld = (1 << 30) + 1, 4
+    acc = torch.empty(n, ld, device=dev)
+    reps = torch.empty(n, ld, device=dev)
+    for t in (acc, reps):
+        t[0] = 5.0
+        t[n - 1] = 7.0
+    theta = torch.arange(4, device=dev, dtype=torch.float32)[:P].contiguous()
+    call = agn.agn_commit_pull_noalloc if noalloc else agn.agn_commit_pull
+    call(theta, acc, reps, None, P, ld, n, [n - 1], [0, 1], [n - 1], 0.5, 1)
+    torch.cuda.synchronize()
+    want = torch.arange(4, dtype=torch.float32)[:P] - 3.5
+    assert torch.equal(theta.cpu(), want)
+    assert torch.equal(reps[n - 1, :P].cpu(), want)
+    assert torch.all(reps[0] == 5.0) and torch.all(acc[0] == 5.0)
+    assert torch.all(acc[n - 1, :P] == 0.0)
+    del acc, reps
+    torch.cuda.empty_cache()
