@@ -154,7 +154,12 @@ void agn_default_options(agn_options* opt);
  * accumulators a_k [n][P] (fp32; plus bf16 working copies [n][P] in bf16
  * mode), the dataset and activation workspaces on the current device;
  * generate (or copy) the dataset, teacher labels and theta~^0 (Glorot-uniform
- * weights, zero biases); every replica pulls version 0.
+ * weights, zero biases); every replica pulls version 0.  Buffers that only
+ * make the handle faster (the activations of kept local steps, evaluation on
+ * the tensor cores, tensor cores past 256 samples) are chosen from the sizes
+ * and the device's total memory, whatever part of it is in use, so that equal
+ * calls give equal bits; a handle that does not fit with them is created
+ * without them, and its results then differ in rounding.
  *   dims     : d_0 .. d_L (n_dims = L + 1 >= 2), all > 0; d_L = classes.
  *   n_workers: n >= 1;  lambda: local steps per commit >= 1 (Algorithm 1);
  *   eta      : learning rate > 0 (constant: Section 4 uses no decay);

@@ -204,6 +204,8 @@ struct agn_handle {
   int tau_lo = 0, tau_hi = 0;
   int64_t N = 0, S = 0;
   std::vector<int> tdims;
+  bool lean = false;          // no kept steps, no evaluation on the tensor cores, CUDA cores past
+                              // 256 samples: agn_create found no room for their buffers
   int64_t P = 0, P_pad = 0;
   std::vector<int64_t> woff, boff, woff_flat, boff_flat;   // per layer (index l-1)
   // CUDA
@@ -215,6 +217,7 @@ struct agn_handle {
   // device state
   float* theta_c = nullptr;   // [P_pad]
   float* flat = nullptr;      // [P]: parameters packed for a read (read_params), past kShortRead
+                              // (null: no room for it)
   float* rep = nullptr;       // [n][P_pad] fp32 master replicas
   float* acc = nullptr;       // [n][P_pad] accumulators (sum of raw gradients)
   bf16* rep_b = nullptr;      // [n][P_pad] bf16 working copies (bf16 mode)
@@ -1435,7 +1438,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     return Status::Err(AGN_E_UNSUPPORTED,
                        "tcgen05 GEMMs need batch <= 256, at least one hidden layer "
                        "and d_0 .. d_{L-1} multiples of 8");
-  h->use_tc = tc_ok && o.gemm != AGN_GEMM_SIMT;
+  h->use_tc = tc_ok && o.gemm != AGN_GEMM_SIMT && !(h->lean && h->m > 256);
   h->split = h->use_tc && h->prec == AGN_PREC_FP32;
   h->tc_mask = (o.tc_mask & 7) == 0 ? (o.tc_mask | 7) : o.tc_mask;
   h->use_head = h->prec == AGN_PREC_BF16 ? agn::head_fits<bf16>(dims[h->L - 1], dims[h->L])
@@ -1503,7 +1506,6 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   const size_t es = elem_size(h);
   const int64_t n = h->n, m = h->m;
   AGN_TRY(dalloc_t(h, &h->theta_c, (size_t)h->P_pad));
-  if (h->P > kShortRead) AGN_TRY(dalloc_t(h, &h->flat, (size_t)h->P));
   AGN_TRY(dalloc_t(h, &h->rep, (size_t)(n * h->P_pad)));
   AGN_TRY(dalloc_t(h, &h->acc, (size_t)(n * h->P_pad)));
   if (h->prec == AGN_PREC_BF16) AGN_TRY(dalloc_t(h, &h->rep_b, (size_t)(n * h->P_pad)));
@@ -1557,17 +1559,15 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   AGN_TRY(dalloc_t(h, &h->yb, (size_t)(n * (h->direct_x ? h->S + m : m))));
   size_t dev_free = 0, dev_total = 0;
   AGN_TRY_CUDA(cudaMemGetInfo(&dev_free, &dev_total));
-  if (h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam &&
+  if (!h->lean && h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam &&
       h->lam > 1 && m <= kHistMaxBatch && n * h->P * 4 > agn::kTcRedAccBytes) {
-    // no more than twice the accumulators' memory or an eighth of the device's;
-    // none where it would take half of what is free (the handle needs no history)
+    // no more than twice the accumulators' memory or an eighth of the device's
     int64_t per = h->ldz_out;
     for (int l = 1; l < h->L; ++l) per += 2 * dims[l];
     const int64_t step = 2 * n * m * per;
     const int64_t most = std::min<int64_t>(8 * n * h->P, (int64_t)(dev_total / 8));
     h->hist = (int)std::min<int64_t>(std::min(h->lam, kHistMaxSteps),
                                      std::max<int64_t>(1, most / step));
-    if (h->hist * step > (int64_t)(dev_free / 2)) h->hist = 1;
   }
   if (h->hist > 1) {
     h->block = m <= 96 ? 4 : m <= 160 ? 3 : 2;
@@ -1594,16 +1594,16 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     const int64_t E = h->n_eval;
     int maxh = 1;
     for (int l = 1; l < h->L; ++l) maxh = std::max(maxh, dims[l]);
-    // the tensor cores evaluate what they train (unless the rows' pieces, half as
-    // large again as the rows, would take a quarter of what is free); fewer,
-    // larger chunks keep every SM busy (300 MB of pieces at most, 4096 rows at
-    // least)
-    AGN_TRY_CUDA(cudaMemGetInfo(&dev_free, &dev_total));
-    h->eval_tc = h->use_tc && 6 * E * d0 <= (int64_t)(dev_free / 4);
-    h->eval_chunk = std::min<int64_t>(
-        E, !h->eval_tc ? 4096 : std::max<int64_t>(4096, (48 << 20) / maxh / 256 * 256));
-    const int64_t up = h->eval_tc ? std::min<int64_t>(E, 1 << 16) : E;   // rows uploaded at a time
-    AGN_TRY(dalloc_t(h, &h->Xe, (size_t)(up * d0)));
+    // The tensor cores evaluate what they train, unless that would take a quarter
+    // of the device: the rows' pieces, the rows of one upload, and for each row
+    // and feature of a chunk two buffers of pieces and one of fp32 values.
+    // Fewer, larger chunks keep every SM busy (4096 rows at least).
+    const int64_t up = std::min<int64_t>(E, 1 << 16);   // rows uploaded at a time
+    const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(4096, (48 << 20) / maxh / 256 * 256));
+    h->eval_tc = h->use_tc && !h->lean &&
+                 (6 * E + 4 * up) * d0 + 16 * rows * maxh <= (int64_t)(dev_total / 4);
+    h->eval_chunk = h->eval_tc ? rows : std::min<int64_t>(E, 4096);
+    AGN_TRY(dalloc_t(h, &h->Xe, (size_t)((h->eval_tc ? up : E) * d0)));
     AGN_TRY(dalloc_t(h, &h->ye, (size_t)E));
     AGN_TRY(dalloc_t(h, &h->He[0], (size_t)(h->eval_chunk * maxh)));
     if (!h->eval_tc) AGN_TRY(dalloc_t(h, &h->He[1], (size_t)(h->eval_chunk * maxh)));
@@ -1688,6 +1688,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     AGN_TRY_CUDA(cudaMemsetAsync(h->tc_counter, 0, (size_t)(2 * h->num_sms) * sizeof(int),
                                  h->stream));
   }
+  // (no room: reads unpack the padded vector on the host, the same values)
+  if (h->P > kShortRead && !dalloc_t(h, &h->flat, (size_t)h->P).ok()) h->flat = nullptr;
   std::vector<int> all(n);
   for (int w = 0; w < n; ++w) all[w] = w;
   AGN_TRY_CUDA(cudaMemcpyAsync(h->pull_list, all.data(), n * sizeof(int), cudaMemcpyHostToDevice,
@@ -1841,7 +1843,7 @@ void touch_pages(void* p, size_t bytes) {
 // padded vector into a host vector, then per-tensor copies: 10.7 ms for 84 MB.)
 Status read_params(agn_handle* h, const float* dev, float* out, int64_t cap) {
   if (!out || cap < h->P) return Status::Err(AGN_E_INVALID, "output buffer shorter than P");
-  if (!h->flat) {   // a short vector: one small copy, unpacked here
+  if (!h->flat) {   // a short vector (or no room for a packed one): one copy, unpacked here
     std::vector<float> tpad((size_t)h->P_pad);
     AGN_TRY_CUDA(cudaMemcpyAsync(tpad.data(), dev, tpad.size() * sizeof(float),
                                  cudaMemcpyDeviceToHost, h->stream));
@@ -2024,21 +2026,31 @@ int agn_create(const int32_t* dims, int32_t n_dims, int32_t n_workers, int32_t l
   *out = nullptr;
   agn_options o;
   if (opt) o = *opt; else agn_default_options(&o);
-  agn_handle* h = new (std::nothrow) agn_handle();
-  if (!h) return fail(nullptr, AGN_E_OOM, "host allocation failed");
-  Status s;
-  try {
-    s = create(h, dims, n_dims, n_workers, lambda, eta, seed, o);
-  } catch (const std::bad_alloc&) {
-    s = Status::Err(AGN_E_OOM, "host allocation failed");
-  }
-  if (!s.ok()) {
+  // Where the device has no room for the buffers that only make a handle faster,
+  // once more without them.
+  for (bool lean : {false, true}) {
+    agn_handle* h = new (std::nothrow) agn_handle();
+    if (!h) return fail(nullptr, AGN_E_OOM, "host allocation failed");
+    h->lean = lean;
+    Status s;
+    bool host = false;
+    try {
+      s = create(h, dims, n_dims, n_workers, lambda, eta, seed, o);
+    } catch (const std::bad_alloc&) {
+      s = Status::Err(AGN_E_OOM, "host allocation failed");
+      host = true;
+    }
+    if (s.ok()) {
+      *out = h;
+      return AGN_OK;
+    }
+    const bool again = !lean && s.code == AGN_E_OOM && !host &&
+                       (h->hist > 1 || h->eval_tc || (h->use_tc && h->m > 256));
     g_error = s.msg;
     agn_destroy(h);
-    return s.code;
+    if (!again) return s.code;
   }
-  *out = h;
-  return AGN_OK;
+  return AGN_E_OOM;   // not reached
 }
 
 int agn_run(agn_handle* h, int32_t n_commits, const int32_t* worker, const int32_t* staleness,
