@@ -1597,9 +1597,10 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     // The tensor cores evaluate what they train, unless that would take a quarter
     // of the device: the rows' pieces, the rows of one upload, and for each row
     // and feature of a chunk two buffers of pieces and one of fp32 values.
-    // Fewer, larger chunks keep every SM busy (4096 rows at least).
+    // Fewer, larger chunks keep every SM busy: up to 48 Mi features, 805 MB
+    // (256 rows at least).
     const int64_t up = std::min<int64_t>(E, 1 << 16);   // rows uploaded at a time
-    const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(4096, (48 << 20) / maxh / 256 * 256));
+    const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(256, (48 << 20) / maxh / 256 * 256));
     h->eval_tc = h->use_tc && !h->lean &&
                  (6 * E + 4 * up) * d0 + 16 * rows * maxh <= (int64_t)(dev_total / 4);
     h->eval_chunk = h->eval_tc ? rows : std::min<int64_t>(E, 4096);

@@ -136,3 +136,21 @@ def test_no_room_for_long_minibatches_on_the_tensor_cores(env):
     with only_free(torch, need - 200 * MB):   # of 287 MB of padded shards
         with make(agn.AGN_GEMM_AUTO) as h:
             assert _same(use(h), ref)
+
+
+def test_wide_hidden_layers_take_short_chunks(env):
+    """Past 12288 features a chunk is under 4096 rows (48 Mi features in all)."""
+    agn, torch = env
+
+    def make(gemm, rows):
+        return agn.AGN((8, 40960, 3), 1, 1, 0.1, 4, batch=2, n_samples=8, n_eval=rows, gemm=gemm)
+
+    def use(h):
+        return h.evaluate(with_pred=True)
+    small, _ = _footprint(torch, lambda: make(agn.AGN_GEMM_AUTO, 1), use)
+    need, got = _footprint(torch, lambda: make(agn.AGN_GEMM_AUTO, 4096), use)
+    assert need - small <= 900 * MB
+    _, ref = _footprint(torch, lambda: make(agn.AGN_GEMM_SIMT, 4096), use)
+    # two fp32 sums of eight products and of 40960 positive ones, in other orders
+    assert got[0] == pytest.approx(ref[0], rel=1e-5)
+    assert np.mean(got[2] != ref[2]) <= 1e-3
