@@ -1509,14 +1509,15 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   AGN_TRY(dalloc_t(h, &h->rep, (size_t)(n * h->P_pad)));
   AGN_TRY(dalloc_t(h, &h->acc, (size_t)(n * h->P_pad)));
   if (h->prec == AGN_PREC_BF16) AGN_TRY(dalloc_t(h, &h->rep_b, (size_t)(n * h->P_pad)));
-  if (h->adam) {   // gradients and the two moments of every worker, zero to start
-    AGN_TRY(dalloc_t(h, &h->grad, (size_t)(n * h->P_pad)));
-    AGN_TRY(dalloc_t(h, &h->mom1, (size_t)(n * h->P_pad)));
-    AGN_TRY(dalloc_t(h, &h->mom2, (size_t)(n * h->P_pad)));
-    for (float* p : {h->grad, h->mom1, h->mom2})
-      AGN_TRY_CUDA(cudaMemset(p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
-  }
   h->fuse_out_dw = h->use_tc && h->use_head && (h->tc_mask & 4) && !(h->tc_mask & 8);
+  if (h->adam) {   // the two moments of every worker, zero to start, and, for a step of
+                   // its own after the dW kernels, the gradients
+    for (float** p : {&h->mom1, &h->mom2, &h->grad}) {
+      if (p == &h->grad && h->fuse_out_dw) continue;
+      AGN_TRY(dalloc_t(h, p, (size_t)(n * h->P_pad)));
+      AGN_TRY_CUDA(cudaMemset(*p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
+    }
+  }
   h->acc_first = h->fuse_out_dw || h->adam;
   h->low_pulls = h->prec == AGN_PREC_BF16 && h->lam == 1 && h->fuse_out_dw && !h->adam &&
                  !h->elide && h->P_pad / 4 < INT32_MAX;

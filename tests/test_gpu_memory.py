@@ -7,6 +7,8 @@ history of kept local steps, the tensor cores' evaluation, the tensor cores past
 256 samples) a handle is created without them and takes the CUDA-core or
 step-by-step route, bit for bit where that route has an option of its own.
 
+Adam keeps gradients only where its step is a kernel of its own.
+
 Each case first measures what the handle takes, then holds all of the device's
 memory but that, plus or minus some."""
 
@@ -154,3 +156,20 @@ def test_wide_hidden_layers_take_short_chunks(env):
     # two fp32 sums of eight products and of 40960 positive ones, in other orders
     assert got[0] == pytest.approx(ref[0], rel=1e-5)
     assert np.mean(got[2] != ref[2]) <= 1e-3
+
+
+@pytest.mark.parametrize("mask,arrays", [(7, 2), (3, 3)])   # fused with dW; dW on the CUDA cores
+def test_adam_keeps_gradients_only_for_its_own_kernel(env, mask, arrays):
+    agn, torch = env
+    n, dims = 4, (1024, 2048, 10)
+    P = sum(a * b + b for a, b in zip(dims, dims[1:]))
+    w = np.arange(n, dtype=np.int32)
+
+    def make(opt):
+        return agn.AGN(dims, n, 1, 1e-3, 4, batch=8, n_samples=64, tc_mask=mask, local_optimizer=opt)
+
+    def use(h):
+        h.run(n, w, w)
+    sgd, _ = _footprint(torch, lambda: make(agn.AGN_OPT_SGD), use)
+    adam, _ = _footprint(torch, lambda: make(agn.AGN_OPT_ADAM), use)
+    assert abs(adam - sgd - arrays * 4 * n * P) <= 6 * MB   # (two MB are the device's unit)
