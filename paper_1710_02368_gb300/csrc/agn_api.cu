@@ -1595,14 +1595,14 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     const int64_t E = h->n_eval;
     int maxh = 1;
     for (int l = 1; l < h->L; ++l) maxh = std::max(maxh, dims[l]);
-    // The tensor cores evaluate what they train, unless that would take a quarter
-    // of the device: the rows' pieces, the rows of one upload, and for each row
-    // and feature of a chunk two buffers of pieces and one of fp32 values.
-    // Fewer, larger chunks keep every SM busy: up to 48 Mi features, 805 MB
-    // (256 rows at least).
+    // The tensor cores evaluate where they train (the forward), unless that would
+    // take a quarter of the device: the rows' pieces, the rows of one upload, and
+    // for each row and feature of a chunk two buffers of pieces and one of fp32
+    // values.  Fewer, larger chunks keep every SM busy: up to 48 Mi features,
+    // 805 MB (256 rows at least).
     const int64_t up = std::min<int64_t>(E, 1 << 16);   // rows uploaded at a time
     const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(256, (48 << 20) / maxh / 256 * 256));
-    h->eval_tc = h->use_tc && !h->lean &&
+    h->eval_tc = h->use_tc && (h->tc_mask & 1) && !h->lean &&
                  (6 * E + 4 * up) * d0 + 16 * rows * maxh <= (int64_t)(dev_total / 4);
     h->eval_chunk = h->eval_tc ? rows : std::min<int64_t>(E, 4096);
     AGN_TRY(dalloc_t(h, &h->Xe, (size_t)((h->eval_tc ? up : E) * d0)));

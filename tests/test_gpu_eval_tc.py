@@ -54,3 +54,13 @@ def test_against_float64(agn, dims, rows, prec):
     clear = top[:, -1] - top[:, -2] > 1e-4
     assert np.array_equal(pred[clear], z.argmax(1)[clear])
     assert acc == pytest.approx(float(np.mean(pred == y)), abs=1e-6)
+
+
+def test_cuda_core_forward_evaluates_on_the_cuda_cores(agn):
+    """tc_mask without bit 0 (the forward): the evaluation's forward is the
+    CUDA cores' too, bit for bit."""
+    dims, out = (65536, 8, 10), []   # long sums, few samples: another order shows in the loss
+    for kw in (dict(gemm=agn.AGN_GEMM_SIMT), dict(tc_mask=6)):
+        with agn.AGN(dims, 1, 1, 0.1, 4, batch=2, n_samples=8, n_eval=512, **kw) as h:
+            out.append(h.evaluate(with_pred=True))
+    assert out[0][:2] == out[1][:2] and np.array_equal(out[0][2], out[1][2])
