@@ -214,10 +214,13 @@ int agn_loss(agn_handle* h, float* out, int64_t cap);
  * accuracy curves of Section 4): softmax cross-entropy mean and the fraction
  * of samples whose argmax (lowest index on ties) is the label.  Forward pass in
  * fp32 on the device (the hidden layers on the tensor cores where training
- * uses them), fixed-order reductions; blocks until done.  loss, accuracy: host floats (nullable); pred: host int32 [n_eval]
- * predictions (nullable), cap its length.  AGN_E_INVALID without an
- * evaluation set or with a short pred buffer; AGN_E_TIMEOUT as for agn_run.  No counterpart call in the
- * paper, which reports these metrics.
+ * uses them), fixed-order reductions; blocks until done.  loss, accuracy: host
+ * floats (nullable); pred: host int32 [n_eval] predictions (nullable), cap its
+ * length.  AGN_E_INVALID without an
+ * evaluation set or with a short pred buffer; AGN_E_TIMEOUT when a
+ * tensor-core kernel gave up on a bounded wait (the results are not valid;
+ * theta~ and the handle stay good).  No counterpart call in the paper, which reports these
+ * metrics.
  */
 int agn_evaluate(agn_handle* h, float* loss, float* accuracy, int32_t* pred, int64_t cap);
 
@@ -395,8 +398,8 @@ int agn_commit_pull_noalloc(float* theta_c, float* acc, float* replicas, void* r
  * counterpart).  The tensor-core GEMMs' split-K exchange and the fused output
  * layer wait, on the device, for the other CTAs of their launch; every such
  * wait gives up after a time limit, the kernel then returns without its
- * results and agn_run reports AGN_E_TIMEOUT.  wait_ns > 0 sets that limit for
- * this handle's later runs (0 = the default, 2 s); withhold_rank >= 0 makes
+ * results and agn_run (or agn_evaluate) reports AGN_E_TIMEOUT.  wait_ns > 0 sets
+ * that limit for this handle's later calls (0 = the default, 2 s); withhold_rank >= 0 makes
  * split-K rank withhold_rank of every split-K launch skip its arrival on the
  * tile counter, so that the ranks waiting for it give up after wait_ns
  * (-1 = none).  After a run that timed out, the handle's results are not

@@ -62,3 +62,31 @@ def test_debug_waits_off_again_gives_a_normal_run(agn):
         agn.agn_debug_waits(h.h, 0, -1)
         h.run(C, w, tau)
         assert np.all(np.isfinite(h.loss()))
+
+
+@pytest.mark.parametrize("rank", [0, 1])
+def test_evaluation_times_out_and_the_handle_goes_on(agn, rank):
+    """agn_evaluate's forward splits K too and shares the training's counters:
+    a withheld arrival gives AGN_E_TIMEOUT; after it, the same handle evaluates
+    and trains as a fresh one, bit for bit (theta~ was only read)."""
+    w, tau = I.make_schedule(N_WORKERS, C + N_WORKERS, 0, 1, SEED)
+
+    def use(h):
+        before = h.evaluate(with_pred=True)
+        h.run(C, w, tau)
+        return [*before, h.central(), h.loss(), *h.evaluate(with_pred=True)]
+
+    def handle():
+        return agn.AGN(DIMS, N_WORKERS, LAM, ETA, SEED, batch=M, n_samples=N_WORKERS * 4 * M,
+                       gemm=agn.AGN_GEMM_TCGEN05, n_eval=70)
+    with handle() as h:
+        want = use(h)
+    with handle() as h:
+        agn.agn_debug_waits(h.h, 2_000_000, rank)
+        for _ in range(2):   # either half of the counters
+            with pytest.raises(agn.AGNError) as e:
+                h.evaluate()
+            assert e.value.code == agn.AGN_E_TIMEOUT
+        agn.agn_debug_waits(h.h, 0, -1)
+        for g, r in zip(use(h), want):
+            assert np.array_equal(g, r)
