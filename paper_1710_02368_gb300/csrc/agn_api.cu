@@ -1571,7 +1571,13 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
                                      std::max<int64_t>(1, most / step));
   }
   if (h->hist > 1) {
-    h->block = m <= 96 ? 4 : m <= 160 ? 3 : 2;
+    // A block's earlier steps are multiplied again in each of its launches, which
+    // pays while a step is one 64-deep k step of the dW.  GPU ms of ten steps of
+    // 48 slots of 784-4096-4096-10 with blocks of 1, 2, 3, 4: m = 64: 24.9, 21.4,
+    // 20.4, 20.6; m = 65: 26.2, 22.7, 23.7, 24.0; 16 slots at m = 128: 9.24, 8.23,
+    // 8.58, 8.66; m = 192: 10.00, 9.84, 10.34, 10.38; m = 256: 11.09, 10.85, 11.46,
+    // 11.76; the 3072-2048x3-10 net alike.
+    h->block = m <= 64 ? 4 : 2;
     for (int l = 1; l <= h->L; ++l) {
       h->wboff.push_back(h->ld_work);
       h->ld_work += round_up(dims[l], 64);

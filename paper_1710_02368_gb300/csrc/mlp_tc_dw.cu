@@ -90,9 +90,10 @@ struct DwCfg {
   static constexpr bool kAccRing = kMode == kDwUpdAcc;                     // a_k via the ring
   // Sixteen epilogue warps, every other chunk each, where eight are what bounds
   // the launch: Adam's divisions and square roots (91 us a launch with eight, 75
-  // with sixteen), and theta_k kept at its base with short minibatches (m = 64:
-  // 1644 and 1595 us; m = 256, kDwKeep8: 950 and 983).  The other modes are bound
-  // by DRAM or latency: no gain.
+  // with sixteen), and theta_k kept at its base with minibatches to 128 (ten steps
+  // of 16 slots of 784-4096-4096-10, GPU ms with eight and sixteen: m = 64 7.18 and
+  // 7.00, m = 128 8.40 and 8.23, m = 192 9.84 and 9.90, m = 256 10.87 and 11.01).
+  // The other modes are bound by DRAM or latency: no gain.
   static constexpr int kEpiWarps =
       kMode == kDwAdam || kMode == kDwKeep ? 2 * kChunkWarps : kChunkWarps;
   static constexpr int kWarps = kEpiWarps + 3;
@@ -747,7 +748,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
                       (args.acc_ring || acc_bytes > kTcRedAccBytes);
     const int mode = args.grad_out ? kDwGrad
                      : args.mom1  ? kDwAdam
-                     : args.theta_work ? (args.K <= 96 ? kDwKeep : kDwKeep8)
+                     : args.theta_work ? (args.K <= 128 ? kDwKeep : kDwKeep8)
                      : !args.acc   ? kDwUpd
                      : ring        ? kDwUpdAcc
                                    : kDwUpdRed;
