@@ -346,11 +346,12 @@ def roofline(wl, kst, worker_steps, on_tc, hbm, bf16, peak_src):
     impl_bytes = d["bytes"] / launches
     mb = method_bytes_per_worker_step(wl, dom, fused_head=kst["forward_head"]["launches"] > 0)
     method_bytes = mb * worker_steps / launches if mb is not None else impl_bytes
-    # (large bf16 waves keep a_k and, inside a block of local steps, theta_k out
-    # of DRAM: the launch then moves less than the method's per-step bytes, and
-    # the fraction is of what it moves)
-    kept = dom == "backward_dw" and impl_bytes < method_bytes
-    method_bytes = min(method_bytes, impl_bytes) if kept else method_bytes
+    # (where the launches move less than the method's per-step bytes, the fraction
+    # is of what they move: a commit's first step only stores a_k, its last one
+    # leaves theta_k of a worker about to pull, and large bf16 waves keep a_k and,
+    # inside a block of local steps, theta_k out of DRAM)
+    fewer = dom == "backward_dw" and impl_bytes < method_bytes
+    method_bytes = min(method_bytes, impl_bytes) if fewer else method_bytes
     flops = d["flops"] / launches
     # fp32 mode on the tensor cores issues six bf16 piece products per fp32 product
     mma_per_flop = 6.0 if (wl.precision == WL.PREC_FP32 and on_tc) else 1.0
@@ -367,7 +368,7 @@ def roofline(wl, kst, worker_steps, on_tc, hbm, bf16, peak_src):
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["kernel"] = dom
     roof["avg_launch_us"] = 1e6 * sec
-    roof["bytes_basis"] = ("implementation bytes (fewer than the method's)" if kept else
+    roof["bytes_basis"] = ("implementation bytes (fewer than the method's)" if fewer else
                            "method: fp32 theta_k and a_k read-modify-write per parameter and "
                            "local step (16 B; 18 B with the bf16 copy) plus the GEMM operands at "
                            "the mode's element size" if dom == "backward_dw" else

@@ -64,7 +64,8 @@ extern "C" {
                                   bf16 pieces, fp32 accumulation); needs at
                                   least one hidden layer, batch <= 256 and
                                   d_0 .. d_{L-1} multiples of 8 (else
-                                  AGN_E_UNSUPPORTED).  The output layer's
+                                  AGN_E_UNSUPPORTED: callers rely on the limit,
+                                  which AUTO does not have).  The output layer's
                                   forward, softmax-CE and dX run on CUDA cores
                                   or in the last hidden layer's forward; a
                                   narrow one's dW (d_L <= 16) joins the
@@ -115,7 +116,8 @@ typedef struct agn_options {
      per CTA instead of two that share each B stage.  Bit 8 makes the
      persistent dW kernel read each accumulator chunk into shared memory and
      store a_k + g even for waves whose accumulators fit well within the L2,
-     where it otherwise adds g to a_k in the L2 (red.add).  Bit 9 makes the
+     where it otherwise adds g to a_k in the L2 (red.add); a commit's first
+     local step and its last before a pull in the same run keep their own way.  Bit 9 makes the
      forward of layer 1 request no weight stage before its dependency wait.
      Any other bit: AGN_E_INVALID. */
   int32_t tc_mask;

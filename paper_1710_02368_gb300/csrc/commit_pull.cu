@@ -7,10 +7,11 @@
 // the normalisation step of Algorithm 1; or a per-commit s = fp32(-eta /
 // (tau_c + 1)) for the DynSGD rule), adds it to theta~ with a plain
 // round-to-nearest add (no FMA, so the sequence is bit-reproducible), zeroes
-// the accumulator (Algorithm 1 restarts a at 0) and writes theta~ into every
-// replica that pulls at the new version (Pull).  theta~ is written back once.
+// the accumulator (Algorithm 1 restarts a at 0; not where the next commit's
+// first local step stores a) and writes theta~ into every replica that pulls at
+// the new version (Pull).  theta~ is written back once.
 // Bytes per launch: 8P (theta~) + C (4P read a + 4P zero a) + pulls * 4P
-// (+ 2P per pull for the bf16 working copy).
+// (+ 2P per pull for the bf16 working copy; that alone where kLowPull says so).
 //
 // Per-commit ||Delta||_2: per-thread double partial sums, a warp-shuffle
 // tree, a fixed-order sum over the warps of the block, one partial per block,

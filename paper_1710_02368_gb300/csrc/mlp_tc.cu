@@ -1319,7 +1319,10 @@ bool use_row_pairs(const TcArgs& args, int slots, bool split, int bn) {
 // The bf16 forward and dX of full waves with column tiles of 64: three stages
 // instead of six, so that two CTAs share an SM and one's epilogue and
 // prologue overlap the other's stream of weights (both together keep as many
-// bytes in flight).  64 slots of 4096-4096-10, m = 64: FWDUS.
+// bytes in flight).  us a launch, forward and dX, six stages and three: 64 slots of
+// 784-4096-4096-10 at m = 64 254 and 222, 392 and 342, at m = 16 246 and 215, 362 and
+// 321; 32 of 784-2048-2048-10 57 and 48, 70 and 58; 64 of 784-1024-1024-10 46 and 37,
+// 50 and 37; 64 of 784-512-512-10 23 and 18.5, 19 and 14.
 bool use_two_ctas(const TcArgs& args, int slots, int bn) {
   return bn == 64 && args.ksplit <= 1 && full_wave(args, slots, bn);
 }

@@ -12,8 +12,8 @@
 //              fast as the MMA frees them, so the next tile's GEMM runs while
 //              the current tile's epilogue drains.
 //   last warp  parameter producer: each tile's theta_k rows (and a_k's, for
-//              waves whose accumulators exceed 64 MB), 32 output features x
-//              128 inputs per chunk, into a second ring.  Each slot is
+//              fp32 waves whose accumulators exceed 64 MB, or Adam's moments),
+//              32 output features x 128 inputs per chunk, into a second ring.  Each slot is
 //              refilled as soon as it frees, so DRAM reads of the next chunks
 //              (and of the next tile) are in flight while the current one is
 //              updated.  Smaller waves add g to a_k in the L2 (red.add) and
@@ -21,7 +21,8 @@
 //   warp 1     MMA issuer (one thread) and TMEM owner.  Two accumulators
 //              (double buffer): the GEMM of the next tile runs while the
 //              epilogue drains this one.
-//   warps 2-9  (Adam: 2-17) epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31, i.e.
+//   warps 2-9  (2-17 for Adam and for kept steps of short minibatches)
+//              epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31, i.e.
 //              32 consecutive inputs k of the tile, and 16 of the 32 features
 //              of a chunk; it transposes them through shared memory so that
 //              each lane updates four consecutive inputs of a feature at a
@@ -74,10 +75,11 @@ constexpr int kThrottleTiles = 8;              // tiles per CTA from which opera
 // nothing read back into the SM); kDwUpdAcc = the same with a_k's chunk read
 // through the ring beside theta_k's and stored back (3 slots); kDwUpd = the
 // local step without accumulator (elided: commits from a pull snapshot),
-// theta_k alone (6 slots); kDwGrad = the raw gradient only, stored for a
-// separate optimizer kernel (no chunks); kDwKeep = kDwUpd that leaves theta_k at
-// the base of its block of local steps (bf16 mode, args.theta_work; kDwKeep8 on
-// eight epilogue warps); kDwAdam = Adam's step, theta_k and the two moments per
+// theta_k alone (6 slots); kDwGrad = the raw gradient only, stored or added
+// (no chunks): for a separate optimizer kernel, as a_k of workers about to pull,
+// or as a_k of the kept local steps' operands; kDwKeep = kDwUpd that leaves
+// theta_k at the base of its block of local steps (bf16 mode, args.theta_work;
+// kDwKeep8 on eight epilogue warps); kDwAdam = Adam's step, theta_k and the two moments per
 // chunk through the ring (2 slots of 49 KB), the steps added to a_k in the L2.
 enum {
   kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5, kDwKeep8 = 6
