@@ -11,9 +11,10 @@
 //              boxes, MN-major, 128-byte swizzle) into a ring of stages, as
 //              fast as the MMA frees them, so the next tile's GEMM runs while
 //              the current tile's epilogue drains.
-//   last warp  parameter producer: each tile's theta_k rows (and a_k's, for
-//              fp32 waves whose accumulators exceed 64 MB, or Adam's moments),
-//              32 output features x 128 inputs per chunk, into a second ring.  Each slot is
+//   last warp  parameter producer: each tile's theta_k rows (with Adam's moments;
+//              with a_k's for waves whose accumulators exceed 64 MB, unless one
+//              launch sums several steps' into a_k), 32 output features x
+//              128 inputs per chunk, into a second ring.  Each slot is
 //              refilled as soon as it frees, so DRAM reads of the next chunks
 //              (and of the next tile) are in flight while the current one is
 //              updated.  Smaller waves add g to a_k in the L2 (red.add) and
