@@ -1178,10 +1178,16 @@ Status launch_tc(const CUtensorMap& a, const CUtensorMap& b, const TcArgs& args,
     // them (16 KB per chunk and rank) in its stage ring
     const int ring = (int)(kEpi == kEpiFwdHead ? Epi::kHeadOff : Epi::kRingFree);
     auto need = [](int k) { return ((BN / 32 + k - 1) / k) * (k - 1) * (128 * 32 * 4); };
-    while (ks > 1 && need(ks) > ring) --ks;
+    // the most ranks that, dealt equal ranges of k steps (which may leave fewer
+    // ranks, and then more chunks to each), fit the ring
     const int kt = (args.K + kBK - 1) / kBK;
-    ks = std::min(ks, kt);
-    if (ks > 1) ks = (kt + (kt + ks - 1) / ks - 1) / ((kt + ks - 1) / ks);
+    for (ks = std::min(ks, kt); ks > 1; --ks) {
+      const int per = (kt + ks - 1) / ks, even = (kt + per - 1) / per;
+      if (need(ks) <= ring && need(even) <= ring) {
+        ks = even;
+        break;
+      }
+    }
   }
   if (ks > 1 || kEpi == kEpiFwdHead) {
     // the split-K exchange and the fused output layer's wait need every CTA
