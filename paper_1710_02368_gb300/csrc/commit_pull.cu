@@ -70,9 +70,10 @@ __device__ __forceinline__ void pack_pieces_x4(float4 v, uint2& p0, uint2& p1, u
   }
 }
 
-// kCopy: 0 = fp32 replicas only, 1 = plus a bf16 copy, 3 = plus the three
-// exact bf16 pieces (planes `plane` elements apart) of the fp32 mode's
-// tensor-core operands.
+// kCopy: 0 = fp32 replicas only, 1 = plus a bf16 copy, 2 = the same with kLowPull
+// pulls (a kernel of its own: their tests in every bf16 commit + pull cost the
+// short vectors 20 %: 64 workers of 784-128-10, 242 us a run against 192), 3 = plus the three exact bf16 pieces (planes `plane` elements
+// apart) of the fp32 mode's tensor-core operands.
 // kElide: no accumulators.  `acc` then holds each worker's snapshot theta_pull
 // of its last pull, the committed quantity is fp32(theta_k - theta_pull) (the
 // sum of the local updates) with s = fp32(1/lambda) (or fp32(1/(tau_c + 1)),
@@ -83,6 +84,9 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
                    float* __restrict__ acc, float* __restrict__ replicas,
                    bf16* __restrict__ rep_bf16, int64_t P, int64_t ld, float s, int zero_acc,
                    double* __restrict__ partials, int64_t plane) {
+  constexpr bool kLow = kCopy == 2, kBf16 = kCopy == 1 || kLow;
+  // (masked in every form: a value known to be non-negative made the fp32 one 4 % faster)
+  auto pulling = [&](int p) { return plan.pull_worker[p] & ~kLowPull; };
   pdl_begin();
   const int nc = plan.n_commits;
   double sq[kMaxCommitsPerLaunch];
@@ -103,7 +107,7 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
       idx[u] = base + (int64_t)u * kThreads;
       live[u] = idx[u] < n4;
       skip[u] = false;
-      if (kCopy == 1 && !kElide)
+      if (kLow)
         for (int r = 0; r < plan.n_skip; ++r)
           skip[u] = skip[u] || (idx[u] >= plan.skip_lo[r] && idx[u] < plan.skip_hi[r]);
       if (live[u]) th[u] = AGN_LD(th4 + idx[u]);
@@ -158,15 +162,15 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
                       make_float4(0.f, 0.f, 0.f, 0.f));
         }
         for (int p = plan.pull_begin[c]; p < plan.pull_begin[c + 1]; ++p) {
-          const int32_t pw = plan.pull_worker[p];
-          const int64_t row = (int64_t)(pw & ~kLowPull) * ld;
+          const int64_t row = (int64_t)pulling(p) * ld;
+          const bool low = kLow && (plan.pull_worker[p] & kLowPull);
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u) {
             if (!live[u]) continue;
-            if (!(pw & kLowPull) || !skip[u])
+            if (!low || !skip[u])
               AGN_ST(reinterpret_cast<float4*>(replicas + row) + idx[u], th[u]);
             if (kElide) AGN_ST(reinterpret_cast<float4*>(acc + row) + idx[u], th[u]);
-            if (kCopy == 1)
+            if (kBf16)
               AGN_ST(reinterpret_cast<uint2*>(rep_bf16 + row) + idx[u], pack_bf16x4(th[u]));
             if (kCopy == 3) {
               uint2 q0, q1, q2;
@@ -200,10 +204,10 @@ commit_pull_kernel(const __grid_constant__ CommitPlan plan, float* __restrict__ 
         if (cc == c) sq[cc] += (double)(d * d);
       if (!kElide && zero_acc) AGN_ST(ap, 0.f);
       for (int p = plan.pull_begin[c]; p < plan.pull_begin[c + 1]; ++p) {
-        const int64_t row = (int64_t)(plan.pull_worker[p] & ~kLowPull) * ld;
+        const int64_t row = (int64_t)pulling(p) * ld;
         AGN_ST(replicas + row + i, t);
         if (kElide) AGN_ST(acc + row + i, t);
-        if (kCopy == 1) AGN_ST(rep_bf16 + row + i, __float2bfloat16_rn(t));
+        if (kBf16) AGN_ST(rep_bf16 + row + i, __float2bfloat16_rn(t));
         if (kCopy == 3) {
           const bf16 q0 = __float2bfloat16_rn(t);
           const float r1 = __fsub_rn(t, __bfloat162float(q0));
@@ -298,7 +302,9 @@ Status launch_commit_pull(const CommitPlan& plan, float* theta_c, float* acc, fl
     e = elide ? AGN_COMMIT_GO(3, true, replicas_bf16, piece_plane)
               : AGN_COMMIT_GO(3, false, replicas_bf16, piece_plane);
   else if (replicas_bf16)
-    e = elide ? AGN_COMMIT_GO(1, true, replicas_bf16, 0) : AGN_COMMIT_GO(1, false, replicas_bf16, 0);
+    e = elide             ? AGN_COMMIT_GO(1, true, replicas_bf16, 0)
+        : plan.n_skip > 0 ? AGN_COMMIT_GO(2, false, replicas_bf16, 0)
+                          : AGN_COMMIT_GO(1, false, replicas_bf16, 0);
   else
     e = elide ? AGN_COMMIT_GO(0, true, nullptr, 0) : AGN_COMMIT_GO(0, false, nullptr, 0);
 #undef AGN_COMMIT_GO
