@@ -214,41 +214,37 @@ __device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, int tile_x, in
     const bool has_a = g.acc != nullptr;
     float* a = has_a ? g.acc + (int64_t)w * g.ld_param : theta;
     bf16* tb = g.theta_bf16 ? g.theta_bf16 + (int64_t)w * g.ld_param : nullptr;
-    // several rows' loads first, then their updates (memory-level parallelism)
+    // loads of all outputs first, then the updates (memory-level parallelism)
     const float* __restrict__ th_in = theta;
     const float* __restrict__ a_in = a;
-    constexpr int kRows = kTM < 4 ? kTM : 4;   // rows in flight at a time
+    float th[kTM][kTN], av[kTM][kTN];
 #pragma unroll
-    for (int i0 = 0; i0 < kTM; i0 += kRows) {
-      float th[kRows][kTN], av[kRows][kTN];
+    for (int i = 0; i < kTM; ++i) {
+      const int64_t m = m0 + ty * kTM + i;
 #pragma unroll
-      for (int i = 0; i < kRows; ++i) {
-        const int64_t m = m0 + ty * kTM + i0 + i;
-#pragma unroll
-        for (int j = 0; j < kTN; ++j) {
-          const int64_t n = n0 + tx + 16 * j;
-          if (m < g.M && n < g.N) {
-            const int64_t p = g.woff + m * g.N + n;
-            th[i][j] = AGN_LDCS(th_in + p);
-            av[i][j] = has_a ? AGN_LDCS(a_in + p) : 0.f;
-          }
+      for (int j = 0; j < kTN; ++j) {
+        const int64_t n = n0 + tx + 16 * j;
+        if (m < g.M && n < g.N) {
+          const int64_t p = g.woff + m * g.N + n;
+          th[i][j] = AGN_LDCS(th_in + p);
+          av[i][j] = has_a ? AGN_LDCS(a_in + p) : 0.f;
         }
       }
+    }
 #pragma unroll
-      for (int i = 0; i < kRows; ++i) {
-        const int64_t m = m0 + ty * kTM + i0 + i;
-        if (m >= g.M) continue;
+    for (int i = 0; i < kTM; ++i) {
+      const int64_t m = m0 + ty * kTM + i;
+      if (m >= g.M) continue;
 #pragma unroll
-        for (int j = 0; j < kTN; ++j) {
-          const int64_t n = n0 + tx + 16 * j;
-          if (n >= g.N) continue;
-          const int64_t p = g.woff + m * g.N + n;
-          const float gr = acc[i0 + i][j];
-          const float t = local_step(th[i][j], g.eta, gr);
-          AGN_ST(theta + p, t);
-          if (has_a) AGN_ST(a + p, av[i][j] + gr);
-          if (tb) write_copy(tb, g.piece_plane, p, t);
-        }
+      for (int j = 0; j < kTN; ++j) {
+        const int64_t n = n0 + tx + 16 * j;
+        if (n >= g.N) continue;
+        const int64_t p = g.woff + m * g.N + n;
+        const float gr = acc[i][j];
+        const float t = local_step(th[i][j], g.eta, gr);
+        AGN_ST(theta + p, t);
+        if (has_a) AGN_ST(a + p, av[i][j] + gr);
+        if (tb) write_copy(tb, g.piece_plane, p, t);
       }
     }
     if (do_bias && m0 + tid < g.M) {
@@ -450,8 +446,10 @@ int simt_sms() {
 }
 
 // The largest tile (fewest shared-memory reads per multiply-add) that still
-// gives every SM a block or, of 128, one and a half; small launches take small
-// tiles, since a block's chain over k is then what bounds them.
+// gives every SM a block or, of 128, one and a half, and of 128 is not mostly
+// padding; small launches take small tiles, since a block's chain over k is then
+// what bounds them.  (785-2001-2001-10, 16 slots of one sample, us a run of six
+// steps with tiles of 128 and 64: forward 4100 and 2660, dX 3155 and 1990.)
 template <typename T, typename TO, bool kAK, bool kBK, int kEpi>
 Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
   const int sms = simt_sms();
@@ -462,7 +460,8 @@ Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
     AGN_TRY_CUDA(cudaGetLastError());
     return Status::Ok();
   };
-  if (blocks(128) >= 3 * sms / 2) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 128>, 128);
+  if (g.M > 64 && g.N > 64 && blocks(128) >= 3 * sms / 2)
+    return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 128>, 128);
   if (blocks(64) >= sms) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 64>, 64);
   return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 32>, 32);
 }
@@ -493,15 +492,16 @@ Status simt_backward_dw(const GemmArgs* layers, int n_layers, int slots, cudaStr
       batch.first[batch.n] = (int)tiles;
       return tiles;
     };
-    // tiles as in launch_gemm
-    int tile = 128;
+    // tiles as in launch_gemm, but none of 128: bound by the update of theta_k
+    // and a_k, whose 186 registers a thread would leave one block an SM (three
+    // of 64).  us a run of six steps of 784-1000-1000-10 with 128 and 64: fp32, 16
+    // slots of 128 samples 3430 and 1890, 4 slots 955 and 580; 785-1001-1001-10, 16
+    // slots of 8 samples 2040 and 938 (bf16 2260 and 853)
+    int tile = 64;
     int64_t tiles = fill(tile);
-    if (tiles * slots < 3 * simt_sms() / 2) tiles = fill(tile = 64);
-    if (tile == 64 && tiles * slots < simt_sms()) tiles = fill(tile = 32);
+    if (tiles * slots < simt_sms()) tiles = fill(tile = 32);
     if (tiles > INT32_MAX) return Status::Err(AGN_E_UNSUPPORTED, "dW tile count overflows");
-    auto kf = tile == 128 ? dw_simt_kernel<T, 128>
-              : tile == 64 ? dw_simt_kernel<T, 64>
-                           : dw_simt_kernel<T, 32>;
+    auto kf = tile == 64 ? dw_simt_kernel<T, 64> : dw_simt_kernel<T, 32>;
     AGN_TRY_CUDA(launch_pdl(kf, dim3((unsigned)tiles, 1, (unsigned)slots), kThreads, 0, st, batch));
     AGN_TRY_CUDA(cudaGetLastError());
   }
