@@ -72,8 +72,9 @@ __device__ __forceinline__ void pack_pieces_x4(float4 v, uint2& p0, uint2& p1, u
 
 // kCopy: 0 = fp32 replicas only, 1 = plus a bf16 copy, 2 = the same with kLowPull
 // pulls (a kernel of its own: their tests in every bf16 commit + pull cost the
-// short vectors 20 %: 64 workers of 784-128-10, 242 us a run against 192), 3 = plus the three exact bf16 pieces (planes `plane` elements
-// apart) of the fp32 mode's tensor-core operands.
+// short vectors 20 %: 64 workers of 784-128-10, 242 us a run against 192), 3 =
+// plus the three exact bf16 pieces (planes `plane` elements apart) of the fp32
+// mode's tensor-core operands.
 // kElide: no accumulators.  `acc` then holds each worker's snapshot theta_pull
 // of its last pull, the committed quantity is fp32(theta_k - theta_pull) (the
 // sum of the local updates) with s = fp32(1/lambda) (or fp32(1/(tau_c + 1)),

@@ -287,14 +287,17 @@ dw_simt_kernel(const __grid_constant__ DwLayers batch) {
 // slot (one block per slot took 38 us a launch at 4 slots x 512 samples x 10
 // classes): up to kXentClasses classes pass through shared memory, copied in
 // and out by the whole block, and a thread sums its sample's classes in order;
-// with more classes it reads them from global memory.  The chunk's loss is a
-// fixed tree over its samples.
+// more classes pass through in tiles of as many, twice (maximum, then sum).  The
+// chunk's loss is a fixed tree over its samples.  A thread reading its sample's
+// classes from global memory instead took 215 us a launch at 16 slots x 128 samples x
+// 1000 classes by itself, and a millisecond beside the dW launch waiting behind
+// it, whose shared memory leaves the lines no room in L1; the tiles take 68.
 constexpr int kXentThreads = 128, kXentClasses = 128;
 template <typename T>
 __global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const SoftmaxArgs a) {
   pdl_begin();
   __shared__ float zs[32 * (kXentClasses + 1)];
-  __shared__ float inv_s[32];
+  __shared__ float inv_s[32], mx_s[32];
   __shared__ int ys[32];
   const int z = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
   const int m = a.m, C = a.C, nj = min(32, m - 32 * chunk);
@@ -303,10 +306,42 @@ __global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const Softma
   const float* Zc = a.Z + row0;
   T* dZc = static_cast<T*>(a.dZ) + row0;
   const bool staged = C <= kXentClasses;
-  const int ld = C + 1 - (C & 1);   // odd: no bank conflicts between the samples' rows
+  // odd row strides: no bank conflicts between the samples' rows
+  const int ld = staged ? C + 1 - (C & 1) : kXentClasses + 1;
+  float mx = -INFINITY, s = 0.f;   // of sample tid
+  float* zr = zs + tid * ld;       // its row (tid < 32)
   if (staged) {
     for (int i = tid; i < nj * C; i += kXentThreads) zs[i / C * ld + i % C] = AGN_LD(Zc + i);
     __syncthreads();
+  } else {
+    const int warp = tid >> 5, lane = tid & 31;
+    constexpr int kRowsPerWarp = 32 / (kXentThreads / 32), kLoads = kXentClasses / 32;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int c0 = 0; c0 < C; c0 += kXentClasses) {
+        float v[kRowsPerWarp][kLoads];
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+          for (int q = 0; q < kLoads; ++q) {
+            const int j = warp * kRowsPerWarp + r, c = c0 + 32 * q + lane;
+            v[r][q] = j < nj && c < C ? AGN_LD(Zc + (int64_t)j * C + c) : 0.f;
+          }
+        __syncthreads();   // the tile before is read
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r)
+#pragma unroll
+          for (int q = 0; q < kLoads; ++q)
+            zs[(warp * kRowsPerWarp + r) * ld + 32 * q + lane] = v[r][q];
+        __syncthreads();
+        if (tid < nj) {
+          const int w = min(kXentClasses, C - c0);
+          if (pass == 0)
+            for (int c = 0; c < w; ++c) mx = fmaxf(mx, zr[c]);
+          else
+            for (int c = 0; c < w; ++c) s += expf(zr[c] - mx);
+        }
+      }
+    }
   }
   if (tid < 32) {
     float ce = 0.f;
@@ -317,28 +352,19 @@ __global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const Softma
                     batch_row0(a.slot_t0, z, a.step, m, a.x_shard)
               : a.yb + (int64_t)z * m;
       const int y = AGN_LD(yrow + 32 * chunk + tid);
-      float* zr = zs + tid * ld;
-      const float* zg = Zc + (int64_t)tid * C;
-      auto at = [&](int c) { return staged ? zr[c] : AGN_LD(zg + c); };
-      float mx = at(0);
-      for (int c = 1; c < C; ++c) mx = fmaxf(mx, at(c));
-      const float zy = at(y);
-      float s = 0.f;
-      for (int c = 0; c < C; ++c) {
-        const float ex = expf(at(c) - mx);
-        if (staged) zr[c] = ex;
-        s += ex;
+      const float zy = staged ? zr[y] : AGN_LD(Zc + (int64_t)tid * C + y);
+      if (staged) {
+        for (int c = 0; c < C; ++c) mx = fmaxf(mx, zr[c]);
+        for (int c = 0; c < C; ++c) {
+          const float ex = expf(zr[c] - mx);
+          zr[c] = ex;
+          s += ex;
+        }
       }
       ce = (logf(s) + mx) - zy;
       inv_s[tid] = 1.0f / s;
+      mx_s[tid] = mx;
       ys[tid] = y;
-      if (!staged) {
-        for (int c = 0; c < C; ++c) {
-          float p = expf(at(c) - mx) * inv_s[tid];
-          if (c == y) p -= 1.0f;
-          AGN_ST(dZc + (int64_t)tid * C + c, from_f<T>(p * inv_m));
-        }
-      }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, off);
@@ -350,11 +376,10 @@ __global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const Softma
       if (!isfinite(part)) atomicExch(a.flag, 1);
     }
   }
-  if (!staged) return;   // uniform across the block
   __syncthreads();
   for (int i = tid; i < nj * C; i += kXentThreads) {
     const int j = i / C, c = i % C;
-    float p = zs[j * ld + c] * inv_s[j];
+    float p = (staged ? zs[j * ld + c] : expf(AGN_LD(Zc + i) - mx_s[j])) * inv_s[j];
     if (c == ys[j]) p -= 1.0f;
     AGN_ST(dZc + i, from_f<T>(p * inv_m));
   }

@@ -20,7 +20,7 @@ SHAPES = [((37, 65, 13, 7), 9, 5),           # nothing a multiple of 8
           ((3, 5, 2), 1, 2),                 # the smallest
           ((61, 130, 26), 33, 3),            # odd widths, 26 classes
           ((40, 72, 33), 17, 4),             # 33 classes
-          ((24, 40, 136, 130), 40, 2),       # 130 classes: read from global memory
+          ((24, 40, 136, 130), 40, 2),       # 130 classes: the softmax in two tiles
           ((64, 136, 10), 257, 3),           # three column tiles, one sample in the last
           ((64, 136, 10), 512, 32),          # too many tiles for the fused output layer
           ((61, 48, 40, 20), 300, 3)]        # all at once
