@@ -278,6 +278,16 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
         // minibatch row (samples past m multiply dZ rows that are zero fill)
         const bool a_direct = B.layer[ti.layer].a_direct && args.x_shard > 0;
         int a_row0 = 0, b_z = 0, a_z = 0;
+        auto operands = [&](int st) {   // of local step st: batches and the first row
+          b_z = args.z0 + st * args.z_step + ti.slot;
+          a_z = a_direct ? AGN_LD(args.slot_worker + ti.slot) : b_z;
+          if (a_direct)
+            a_row0 = (int)batch_row0(args.slot_t0, ti.slot, args.step + st, args.K, args.x_shard);
+        };
+        // the first step's before the wait for chunks, not after it: the row's
+        // 64-bit division stands before the tile's first copy (8 slots of 3072-
+        // 2048x3-10 at m = 160: 204 and 199 us a launch)
+        operands(0);
         if (throttle && itp > 0 && *chunk_tiles < itp) {
           const uint64_t t0 = tc::globaltimer_ns();
           while (*chunk_tiles < itp) {
@@ -290,12 +300,6 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           if (!ok) break;
         }
         for (int kt = 0, kr = 0, st = 0; kt < KT; ++kt) {
-          if (kr == 0) {   // the next local step's operands
-            b_z = args.z0 + st * args.z_step + ti.slot;
-            a_z = a_direct ? AGN_LD(args.slot_worker + ti.slot) : b_z;
-            if (a_direct)
-              a_row0 = (int)batch_row0(args.slot_t0, ti.slot, args.step + st, args.K, args.x_shard);
-          }
           const int s = ml % kStages;
           if (ml >= kStages &&
               !tc::wait_or_abort(&empty[s], ((ml / kStages) - 1) & 1, abort_flag, kWaitNs)) {
@@ -330,7 +334,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           ++ml;
           if (++kr == KTs) {
             kr = 0;
-            ++st;
+            if (kt + 1 < KT) operands(++st);
           }
         }
       }
