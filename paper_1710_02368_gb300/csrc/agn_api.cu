@@ -486,11 +486,25 @@ void next_counters(agn_handle* h, agn::TcArgs* t) {
   h->ctr_parity ^= 1;
 }
 
+// Column tile of a forward or dX GEMM with M rows and m columns over s
+// slots.  fp32 mode, m > 128: 256 only where the tiles nearly fill the SMs.  A
+// tile of 128 takes A's pieces from tensor memory and gives small waves twice
+// the CTAs; one of 256 converts every weight tile half as often.  Measured, us
+// per local step of 784-1000-1000-10 at m = 256: 1 worker 56.5 (128) / 60.9
+// (256), 4 workers 110.7 / 112.0, 16 workers 394 / 357; 784-4096-4096-10, 4
+// workers, 822 / 721; 64-48-10 at m = 200, 41.1 / 60.5.
+int tc_bn(const agn_handle* h, bool split, int M, int m, int s) {
+  if (m <= 64) return 64;
+  if (m <= 128) return 128;
+  if (!split) return 256;
+  return 4 * ceil_div(M, 128) * ceil_div(m, 256) * (int64_t)s >= 3 * (int64_t)h->num_sms ? 256 : 128;
+}
+
 // Tensor maps of the tcgen05 path (addresses are fixed for the handle's life).
 Status build_tc_maps(agn_handle* h) {
   const int n = h->n, m = h->m, L = h->L;
   const int nh = n * h->hist;   // activation batches: slots of every kept local step
-  constexpr uint32_t bn = agn::kTcBoxN;
+  const uint32_t bn = h->split ? agn::kTcBoxN : tc_bn(h, false, 0, m, 0);   // rows of a box
   h->tmaps.assign(L - 1, {});
   auto moments = [&](agn_handle::LayerMaps& mp, int l) -> Status {
     if (!h->adam) return Status::Ok();
@@ -596,20 +610,6 @@ Status build_tc_maps(agn_handle* h) {
     }
   }
   return Status::Ok();
-}
-
-// Column tile of a forward or dX GEMM with M rows and m columns over s
-// slots.  fp32 mode, m > 128: 256 only where the tiles nearly fill the SMs.  A
-// tile of 128 takes A's pieces from tensor memory and gives small waves twice
-// the CTAs; one of 256 converts every weight tile half as often.  Measured, us
-// per local step of 784-1000-1000-10 at m = 256: 1 worker 56.5 (128) / 60.9
-// (256), 4 workers 110.7 / 112.0, 16 workers 394 / 357; 784-4096-4096-10, 4
-// workers, 822 / 721; 64-48-10 at m = 200, 41.1 / 60.5.
-int tc_bn(const agn_handle* h, bool split, int M, int m, int s) {
-  if (m <= 64) return 64;
-  if (m <= 128) return 128;
-  if (!split) return 256;
-  return 4 * ceil_div(M, 128) * ceil_div(m, 256) * (int64_t)s >= 3 * (int64_t)h->num_sms ? 256 : 128;
 }
 
 // Split K of a forward or dX GEMM with M rows, N = m columns in tiles of bn and

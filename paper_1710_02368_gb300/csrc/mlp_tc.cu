@@ -174,6 +174,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   constexpr int kABytes = Cfg::kABytes;
   constexpr uint32_t kA32Bytes = Cfg::kA32Bytes;
   constexpr int kBox = kBK * 128;   // one 64-wide MN box of kBK rows (MN-major operands)
+  constexpr int kBoxN = kSplit == 1 ? BN : kTcBoxN;   // rows of a K-major B box
   using TAct = typename std::conditional<kSplit == 1, bf16, float>::type;
   // fp32 mode, forward and dX: A = W arrives as fp32 (TMA, 128 x kBK floats
   // into the first 16 KB of the stage's 24 KB of A pieces) and warps 2-7
@@ -309,9 +310,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           uint8_t* sb = sb0 + p * Cfg::kBBytes;
           if (!kBMN) {
 #pragma unroll
-            for (int c = 0; c < BN / kTcBoxN; ++c)
-              load(sb + c * (kTcBoxN * Cfg::kRowBytes), &tmB, kc,
-                   n_tile * BN + c * kTcBoxN + b_row0, b_z, p, &full[s]);
+            for (int c = 0; c < BN / kBoxN; ++c)
+              load(sb + c * (kBoxN * Cfg::kRowBytes), &tmB, kc, n_tile * BN + c * kBoxN + b_row0,
+                   b_z, p, &full[s]);
           } else {
 #pragma unroll
             for (int c = 0; c < BN / 64; ++c)

@@ -120,7 +120,10 @@ struct TcArgs {
 };
 
 // Column tiles of the forward and dX are 64, 128 or 256 samples wide
-// (tc_bn); their activation operand lands in boxes of kTcBoxN rows.
+// (tc_bn).  Their activation operand lands in one box of as many rows in bf16
+// mode (four of 64 took the dX of 8 slots of 3072-2048x3-10 at m = 160 from 266
+// to 279 us a run of five steps), in boxes of kTcBoxN rows in fp32 mode, where the
+// tile's width depends on the wave.
 constexpr int kTcBoxN = 64;
 constexpr int kTcSplitBK = 32;      // forward / dX k per stage, split (fp32) mode
 constexpr int kTcDwBN = 256;        // dW column tile, bf16 mode
@@ -144,11 +147,11 @@ Status make_tmap_bf16_4d(CUtensorMap* map, const void* base, uint64_t inner, uin
 // split = false: bf16 operands (3D maps), bf16 activations.
 // split = true : fp32 operands as three exact bf16 pieces (4D maps), fp32
 //                activations; dW writes the three pieces of the new weights.
-// forward: w_k box {64, 128} over W (K-major); h_k box {64, kTcBoxN} over
-// H_{l-1}; bn the column tile (64, 128 or 256).  Small waves split K (args.ksplit).
+// forward: w_k box {64, 128} over W (K-major); h_k box {64, bn} (fp32 mode: kTcBoxN)
+// over H_{l-1}; bn the column tile (64, 128 or 256).  Small waves split K (args.ksplit).
 Status tc_forward(const CUtensorMap& w_k, const CUtensorMap& h_k, const TcArgs& args, int slots,
                   cudaStream_t st, bool split, int bn);
-// dX: w_mn box {64, 64} over W (MN-major view); dz_k box {64, kTcBoxN} over dZ_l.
+// dX: w_mn box {64, 64} over W (MN-major view); dz_k box as the forward's over dZ_l.
 // The forward GEMM of the last hidden layer with the output layer fused
 // (args.head_* set, args.relu = 1).  Needs every CTA of the launch resident at
 // once; when the launch would exceed the SMs nothing is queued and *launched
