@@ -641,8 +641,11 @@ Status split_act(agn_handle* h, const void* src, bf16* dst, int d, int slots, in
 // One wave: lambda local steps of every slot (Algorithm 1's inner loop)
 // ---------------------------------------------------------------------------
 
-// The history of a wave's local steps: see agn_handle::hist.
-constexpr int kHistMaxSteps = 16, kHistMaxBatch = 256;
+// The history of a wave's local steps: see agn_handle::hist.  Without accumulators
+// (elided) it only leaves theta_k at its base, which pays up to 128 samples: GPU ms
+// of 16 steps, with and without, 4 slots of 784-4096-4096-10 at m = 128 3.73 and
+// 4.07, at 160 4.38 and 4.34; 16 slots of 1024-2056-10 at 256 2.86 and 2.78.
+constexpr int kHistMaxSteps = 16, kHistMaxBatch = 256, kHistMaxBatchElided = 128;
 
 template <typename T>
 Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
@@ -1561,7 +1564,8 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   size_t dev_free = 0, dev_total = 0;
   AGN_TRY_CUDA(cudaMemGetInfo(&dev_free, &dev_total));
   if (!h->lean && h->prec == AGN_PREC_BF16 && h->direct_x && h->acc_first && !h->adam &&
-      h->lam > 1 && m <= kHistMaxBatch && n * h->P * 4 > agn::kTcRedAccBytes) {
+      h->lam > 1 && m <= (h->elide ? kHistMaxBatchElided : kHistMaxBatch) &&
+      n * h->P * 4 > agn::kTcRedAccBytes) {
     // no more than twice the accumulators' memory or an eighth of the device's
     int64_t per = h->ldz_out;
     for (int l = 1; l < h->L; ++l) per += 2 * dims[l];
