@@ -73,23 +73,30 @@ constexpr int kThrottleTiles = 8;              // tiles per CTA from which opera
 // B = BN / 64 boxes.
 // kMode: kDwUpdRed = the local step and accumulation, theta_k per chunk
 // through the ring (6 slots in flight) and a_k += g as L2 adds (red.add,
-// nothing read back into the SM); kDwUpdAcc = the same with a_k's chunk read
-// through the ring beside theta_k's and stored back (3 slots); kDwUpd = the
-// local step without accumulator (elided: commits from a pull snapshot),
-// theta_k alone (6 slots); kDwGrad = the raw gradient only, stored or added
-// (no chunks): for a separate optimizer kernel, as a_k of workers about to pull,
-// or as a_k of the kept local steps' operands; kDwKeep = kDwUpd that leaves
-// theta_k at the base of its block of local steps (bf16 mode, args.theta_work;
-// kDwKeep8 on eight epilogue warps); kDwAdam = Adam's step, theta_k and the two moments per
-// chunk through the ring (2 slots of 49 KB), the steps added to a_k in the L2.
+// nothing read back into the SM); kDwSet = the same of a commit's first step,
+// a_k = g; kDwRepull = either, with slots that only take a_k (args.slot_repull);
+// kDwUpdAcc = kDwUpdRed with a_k's chunk read through the ring beside theta_k's
+// and stored back (3 slots); kDwUpd = the local step without accumulator
+// (elided: commits from a pull snapshot), theta_k alone (6 slots); kDwBlock =
+// the same from several kept local steps' operands, or with slots that take
+// nothing; kDwGrad = the raw gradient only, stored or added (no chunks): for a
+// separate optimizer kernel, as a_k of workers about to pull, or as a_k of the
+// kept local steps' operands; kDwKeep = kDwBlock that leaves theta_k at the base
+// of its block of local steps (bf16 mode, args.theta_work; kDwKeep8 on eight
+// epilogue warps); kDwAdam = Adam's step, theta_k and the two moments per chunk
+// through the ring (2 slots of 49 KB), the steps added to a_k in the L2.
+// (Modes, not arguments: an epilogue runs few times a launch on small waves, and
+// the tests and code of the others cost 0.4-1.4 us a launch there.)
 enum {
-  kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5, kDwKeep8 = 6
+  kDwUpdAcc = 0, kDwUpd = 1, kDwGrad = 2, kDwUpdRed = 3, kDwKeep = 4, kDwAdam = 5, kDwKeep8 = 6,
+  kDwSet = 7, kDwRepull = 8, kDwBlock = 9
 };
 constexpr bool is_keep(int mode) { return mode == kDwKeep || mode == kDwKeep8; }
 template <int BN, int kSplit, int kStages, int kBKs, int kMode>
 struct DwCfg {
   static constexpr bool kAcc =                                             // a_k += g
-      kMode == kDwUpdAcc || kMode == kDwUpdRed || kMode == kDwAdam;
+      kMode == kDwUpdAcc || kMode == kDwUpdRed || kMode == kDwSet || kMode == kDwRepull ||
+      kMode == kDwAdam;
   static constexpr bool kAccRing = kMode == kDwUpdAcc;                     // a_k via the ring
   // Sixteen epilogue warps, every other chunk each, where eight are what bounds
   // the launch: Adam's divisions and square roots (91 us a launch with eight, 75
@@ -210,13 +217,16 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
   const int T = B.total_tiles;
   // a slot whose replica nothing reads before its next pull: a_k only (or,
   // where this launch keeps no a_k, nothing)
+  constexpr bool kBlock = kMode == kDwBlock || is_keep(kMode);
   auto acc_only = [&](int slot) -> bool {
-    return (kMode == kDwUpdRed || kMode == kDwUpd || is_keep(kMode)) && args.slot_repull &&
+    return (kMode == kDwRepull || kBlock) && args.slot_repull &&
            AGN_LD(args.slot_repull + slot) != 0;
   };
+  // a_k = g, whatever it held
+  const bool acc_set = kMode == kDwSet || ((kMode == kDwRepull || kAdam) && args.acc_set);
   // k steps of one local step's minibatch, and of the whole launch
   const int KTs = (args.K + kBK - 1) / kBK;
-  const int KT = KTs * max(1, args.hist_steps);
+  const int KT = KTs * (kGrad || kBlock ? max(1, args.hist_steps) : 1);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -523,7 +533,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       float* theta = args.theta + rbase;
       float* work = keep ? args.theta_work + (int64_t)worker * args.ld_work : nullptr;
       float* ww = keep && L.wwoff >= 0 ? work + L.wwoff : nullptr;
-      float* acc = kAcc && args.acc ? args.acc + rbase : nullptr;   // (Adam elided: none)
+      float* acc = kAcc ? args.acc + rbase : nullptr;
+      const bool has_acc = kAcc && (!kAdam || args.acc);   // (Adam elided: none)
       float *mom1 = args.mom1 + rbase, *mom2 = args.mom2 + rbase;   // Adam only
       auto adam = [&](float gr, float& m, float& v) {
         return adam_update(gr, m, v, eta, args.beta1, 1.0f - args.beta1, args.beta2,
@@ -533,7 +544,7 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
       const bool grad_only = kGrad || acc_only(ti.slot);
       const int nch = grad_only && !kAcc && !kGrad
                           ? 0 : min(Cfg::kChunks, (N - ti.n_tile * BN + kCF - 1) / kCF);
-      const bool grad_add = kGrad ? args.grad_add != 0 : !args.acc_set;
+      const bool grad_add = kGrad ? args.grad_add != 0 : !acc_set;
       for (int c = 0; c < nch; ++c) {
         if (kHalves && (ch & 1) != odd) {   // the other half's chunk
           ++ch;
@@ -627,8 +638,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
                     reinterpret_cast<const float*>(slot + kChunkBytes) + so);
                 AGN_ST(reinterpret_cast<float4*>(acc + p),
                        make_float4(av.x + gv.x, av.y + gv.y, av.z + gv.z, av.w + gv.w));
-              } else if (kAcc && acc) {   // a_k += g in the L2 (one add per element and launch)
-                if (args.acc_set) AGN_ST(reinterpret_cast<float4*>(acc + p), gv);
+              } else if (has_acc) {   // a_k += g in the L2 (one add per element and launch)
+                if (acc_set) AGN_ST(reinterpret_cast<float4*>(acc + p), gv);
                 else AGN_RED4(acc + p, gv);
               }
               // the bf16 copy (bf16 mode); the fp32 mode's GEMMs split the
@@ -654,8 +665,8 @@ tc_dw_kernel(const __grid_constant__ DwBatch B, const TcArgs args) {
           }
           AGN_ST(keep ? work + L.wboff + fbase + lane : theta + pb, tn);
           if (kAccRing) AGN_ST(acc + pb, sTb[kCF + 16 * hf + lane] + gb);
-          else if (kAcc && acc && args.acc_set) AGN_ST(acc + pb, gb);
-          else if (kAcc && acc) AGN_RED(acc + pb, gb);
+          else if (has_acc && acc_set) AGN_ST(acc + pb, gb);
+          else if (has_acc) AGN_RED(acc + pb, gb);
           if (kSplit == 1) AGN_ST(tb + pb, __float2bfloat16_rn(tn));
         }
         __syncwarp();
@@ -756,33 +767,55 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     const int mode = args.grad_out ? kDwGrad
                      : args.mom1  ? kDwAdam
                      : args.theta_work ? (args.K <= 128 ? kDwKeep : kDwKeep8)
-                     : !args.acc   ? kDwUpd
-                     : ring        ? kDwUpdAcc
-                                   : kDwUpdRed;
+                     : !args.acc  ? (args.hist_steps > 1 || args.slot_repull ? kDwBlock : kDwUpd)
+                     : ring       ? kDwUpdAcc
+                     : args.slot_repull ? kDwRepull
+                     : args.acc_set     ? kDwSet
+                                        : kDwUpdRed;
+    if (split && (args.theta_work || mode == kDwBlock))
+      return Status::Err(AGN_E_INVALID, "kept local steps: bf16 mode only");
     Status r = Status::Ok();
     // fp32, long minibatches (a tile's GEMM reads eight stages or more): a third
     // operand stage for two of the six chunks in flight.  784-1000-1000-10, 4 slots, us a launch at
     // m = 256, 300, 512: 43.0, 49.1, 70.0 with two stages, 40.5, 45.6, 61.5 with three
     // (42.9, 46.9, 60.9 with four stages and one chunk)
-    const bool deep = split && ceil_div(args.K, 32) * std::max(1, args.hist_steps) >= 8;
-    if (deep && (mode == kDwUpd || mode == kDwUpdRed)) {
-      r = mode == kDwUpd ? launch_dw<kTcDwBNSplit, 3, 3, 32, kDwUpd>(batch, args, num_sms, st)
-                         : launch_dw<kTcDwBNSplit, 3, 3, 32, kDwUpdRed>(batch, args, num_sms, st);
+    const bool deep = ceil_div(args.K, 32) * std::max(1, args.hist_steps) >= 8;
+#define AGN_DW_CASE(BN, SPLIT, STAGES, BK, MODE)                                 \
+  case MODE:                                                                     \
+    r = launch_dw<BN, SPLIT, STAGES, BK, MODE>(batch, args, num_sms, st);        \
+    break
+    if (split && deep && mode != kDwGrad && mode != kDwAdam && mode != kDwUpdAcc) {
+      switch (mode) {
+        AGN_DW_CASE(kTcDwBNSplit, 3, 3, 32, kDwUpd);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 3, 32, kDwSet);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 3, 32, kDwRepull);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 3, 32, kDwUpdRed);
+      }
     } else if (split) {
-      r = mode == kDwGrad     ? launch_dw<kTcDwBNSplit, 3, 4, 32, kDwGrad>(batch, args, num_sms, st)
-          : mode == kDwAdam   ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwAdam>(batch, args, num_sms, st)
-          : mode == kDwUpd    ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpd>(batch, args, num_sms, st)
-          : mode == kDwUpdAcc ? launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdAcc>(batch, args, num_sms, st)
-                              : launch_dw<kTcDwBNSplit, 3, 2, 32, kDwUpdRed>(batch, args, num_sms, st);
+      switch (mode) {
+        AGN_DW_CASE(kTcDwBNSplit, 3, 4, 32, kDwGrad);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwAdam);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwUpd);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwUpdAcc);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwSet);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwRepull);
+        AGN_DW_CASE(kTcDwBNSplit, 3, 2, 32, kDwUpdRed);
+      }
     } else {
-      r = mode == kDwGrad     ? launch_dw<kTcDwBN, 1, 4, 64, kDwGrad>(batch, args, num_sms, st)
-          : mode == kDwAdam   ? launch_dw<kTcDwBN, 1, 2, 64, kDwAdam>(batch, args, num_sms, st)
-          : mode == kDwUpd    ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpd>(batch, args, num_sms, st)
-          : mode == kDwKeep   ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep>(batch, args, num_sms, st)
-          : mode == kDwKeep8  ? launch_dw<kTcDwBN, 1, 2, 64, kDwKeep8>(batch, args, num_sms, st)
-          : mode == kDwUpdAcc ? launch_dw<kTcDwBN, 1, 2, 64, kDwUpdAcc>(batch, args, num_sms, st)
-                              : launch_dw<kTcDwBN, 1, 2, 64, kDwUpdRed>(batch, args, num_sms, st);
+      switch (mode) {
+        AGN_DW_CASE(kTcDwBN, 1, 4, 64, kDwGrad);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwAdam);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwUpd);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwBlock);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwKeep);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwKeep8);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwUpdAcc);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwSet);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwRepull);
+        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwUpdRed);
+      }
     }
+#undef AGN_DW_CASE
     if (!r.ok()) return r;
   }
   return Status::Ok();
