@@ -20,6 +20,7 @@ namespace agn {
 namespace {
 
 constexpr int kThreads = 256;   // 16 x 16, kTile / 16 rows and columns each
+constexpr int64_t kShortK = 48;   // k up to which 32-square tiles take slices of 16
 
 template <typename T>
 __device__ __forceinline__ float to_f(T v);
@@ -57,14 +58,18 @@ __device__ __forceinline__ void write_copy(bf16* tb, int64_t plane, int64_t p, f
 // 31.1 -> 16.4 us, dX 15.8 -> 9.9, dW 46 -> 19 (its three launches in one); the
 // 784-1000-1000 forward of 10000 rows 20 -> 26 TFLOP/s.  A thread's rows are consecutive (its A
 // values come in 16-byte loads), its columns 16 apart (coalesced epilogues).
-template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
+// (kShort: a 32-square tile with at most kShortK k.)
+template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile, bool kShort>
 __device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, int tile_x, int tile_y) {
   constexpr int kBM = kTile, kBN = kTile;
   // k per slice.  Small tiles wait on the next slice's loads: 64 (32: 5 % slower on
   // 613-301-150-26's forwards).  32 for the fp32 dX at 64 x 64 (784-1001-1001-10, 8
   // slots of 128: a pass 2.70 -> 2.56 ms); elsewhere 32 cost blocks an SM (bf16
   // 333-777-29, 16 slots of 200: 1.87 -> 2.05 ms).
-  constexpr int kBK = kTile == 32 ? 64
+  // Few k take slices of 16: the rest of a longer one would be multiplied zeros
+  // (16-344-4, 17 slots, us a run of ten steps with slices of 64 and 16: one sample
+  // 312 and 250, 33 samples 338 and 318; 333-165-40-7, 8 slots of 48: 554 and 558).
+  constexpr int kBK = kTile == 32 ? (kShort ? 16 : 64)
                       : kTile == 64 && kEpi == kEpiDX && sizeof(T) == 4 ? 32 : 16;
   constexpr int kTM = kTile / 16, kTN = kTile / 16;
   constexpr int kLoads = kTile * kBK / kThreads;   // per operand, thread and slice
@@ -257,10 +262,11 @@ __device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, int tile_x, in
   }
 }
 
-template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile>
+template <typename T, typename TO, bool kAKMajor, bool kBKMajor, int kEpi, int kTile,
+          bool kShort = false>
 __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmArgs g) {
   pdl_begin();
-  gemm_simt_tile<T, TO, kAKMajor, kBKMajor, kEpi, kTile>(g, blockIdx.x, blockIdx.y);
+  gemm_simt_tile<T, TO, kAKMajor, kBKMajor, kEpi, kTile, kShort>(g, blockIdx.x, blockIdx.y);
 }
 
 // The weight gradients of several layers in one launch (they depend on no other
@@ -272,7 +278,7 @@ struct DwLayers {
   int first[kDwLayers + 1];
   int n;
 };
-template <typename T, int kTile>
+template <typename T, int kTile, bool kShort = false>
 __global__ void __launch_bounds__(kThreads)
 dw_simt_kernel(const __grid_constant__ DwLayers batch) {
   pdl_begin();
@@ -280,7 +286,7 @@ dw_simt_kernel(const __grid_constant__ DwLayers batch) {
   while (i + 1 < batch.n && (int)blockIdx.x >= batch.first[i + 1]) ++i;
   const GemmArgs& g = batch.g[i];
   const int t = (int)blockIdx.x - batch.first[i], cols = (int)((g.N + kTile - 1) / kTile);
-  gemm_simt_tile<T, T, false, false, kEpiDW, kTile>(g, t % cols, t / cols);
+  gemm_simt_tile<T, T, false, false, kEpiDW, kTile, kShort>(g, t % cols, t / cols);
 }
 
 // Softmax cross-entropy (SoftmaxArgs).  A block takes a 32-sample chunk of a
@@ -488,6 +494,7 @@ Status launch_gemm(const GemmArgs& g, int slots, cudaStream_t st) {
   if (g.M > 64 && g.N > 64 && blocks(128) >= 3 * sms / 2)
     return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 128>, 128);
   if (blocks(64) >= sms) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 64>, 64);
+  if (g.K <= kShortK) return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 32, true>, 32);
   return go(gemm_simt_kernel<T, TO, kAK, kBK, kEpi, 32>, 32);
 }
 
@@ -526,7 +533,9 @@ Status simt_backward_dw(const GemmArgs* layers, int n_layers, int slots, cudaStr
     int64_t tiles = fill(tile);
     if (tiles * slots < simt_sms()) tiles = fill(tile = 32);
     if (tiles > INT32_MAX) return Status::Err(AGN_E_UNSUPPORTED, "dW tile count overflows");
-    auto kf = tile == 64 ? dw_simt_kernel<T, 64> : dw_simt_kernel<T, 32>;
+    auto kf = tile == 64               ? dw_simt_kernel<T, 64>
+              : batch.g[0].K <= kShortK ? dw_simt_kernel<T, 32, true>
+                                        : dw_simt_kernel<T, 32>;
     AGN_TRY_CUDA(launch_pdl(kf, dim3((unsigned)tiles, 1, (unsigned)slots), kThreads, 0, st, batch));
     AGN_TRY_CUDA(cudaGetLastError());
   }

@@ -1,6 +1,6 @@
 """The CUDA-core GEMMs at the edges of their tiles (32, 64 and 128 square, k
 slices of 64, 32 and 16, csrc/mlp_simt.cu): minibatches and widths one below, at and
-one above a tile, with enough workers that each tile size is taken.  Against the
+one above a tile and the k up to which 32-square tiles take short slices, with enough workers that each tile size is taken.  Against the
 float64 oracle at the fp32 tolerances of the other parity tests, and, since
 every output is one chain over k in order whatever the tile, the same worker's
 commit bit for bit whether it trains alone or in a wave of many."""
@@ -23,7 +23,8 @@ def agn():
 
 
 @pytest.mark.parametrize("dims,m", [((31, 33, 5), 1), ((65, 63, 20), 31), ((129, 64, 17), 33),
-                                    ((127, 128, 129, 40), 65), ((257, 129, 18), 129)])
+                                    ((127, 128, 129, 40), 65), ((257, 129, 18), 129),
+                                    ((48, 49, 5), 48), ((49, 48, 18), 49)])
 def test_fp32_matches_oracle(agn, dims, m):
     n, lam, C, seed = 3, 2, 5, 23
     N = n * 2 * m + 1
