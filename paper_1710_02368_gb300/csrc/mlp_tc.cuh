@@ -126,7 +126,7 @@ struct TcArgs {
 // tile's width depends on the wave.
 constexpr int kTcBoxN = 64;
 constexpr int kTcSplitBK = 32;      // forward / dX k per stage, split (fp32) mode
-constexpr int kTcDwBN = 256;        // dW column tile, bf16 mode
+constexpr int kTcDwBN = 256;        // dW column tile, bf16 mode (but Adam's)
 constexpr int kTcDwBNSplit = 128;   // dW column tile, split (fp32) mode
 
 Status tc_init();

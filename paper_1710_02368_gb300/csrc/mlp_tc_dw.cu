@@ -692,8 +692,8 @@ template <int BN, int kSplit, int kStages, int kBKs, int kMode>
 Status launch_dw(const DwBatch& batch, const TcArgs& args, int num_sms, cudaStream_t st) {
   using Cfg = DwCfg<BN, kSplit, kStages, kBKs, kMode>;
   static_assert(Cfg::kSmem <= 232448, "shared memory");
-  static_assert(Cfg::kSmem > 232448 / 2, "one CTA per SM (all 512 TMEM columns)");
-  static_assert(Cfg::kTmemCols == 512, "TMEM columns");
+  static_assert(Cfg::kSmem > 232448 / 2, "one CTA per SM (up to all 512 TMEM columns)");
+  static_assert(Cfg::kTmemCols == 256 || Cfg::kTmemCols == 512, "TMEM columns");
   auto kern = tc_dw_kernel<BN, kSplit, kStages, kBKs, kMode>;
   static std::mutex mu;
   static std::set<int> done;
@@ -721,7 +721,11 @@ Status launch_dw(const DwBatch& batch, const TcArgs& args, int num_sms, cudaStre
 
 Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& args, int slots,
                       cudaStream_t st, bool split, int num_sms) {
-  const int bn = split ? kTcDwBNSplit : kTcDwBN;
+  // Adam's chunks take longest: in bf16 mode too its tiles are 128 features wide,
+  // which deals them out more evenly.  us a run of 64-512-10, 8 workers, 517 against
+  // 670 with tiles of 256; 784-1000-1000-10, 4, m = 128 1344 and 1441; 2616-16-24-1400-5,
+  // one, 412 and 494; 4 of 784-4096-4096-10 3961 and 3965
+  const int bn = split || (args.mom1 && !args.grad_out) ? kTcDwBNSplit : kTcDwBN;
   for (int l0 = 0; l0 < n_layers; l0 += kMaxDwLayers) {
     DwBatch batch;
     std::memset(&batch, 0, sizeof(batch));
@@ -804,7 +808,7 @@ Status tc_backward_dw(const DwLayerMaps* layers, int n_layers, const TcArgs& arg
     } else {
       switch (mode) {
         AGN_DW_CASE(kTcDwBN, 1, 4, 64, kDwGrad);
-        AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwAdam);
+        AGN_DW_CASE(kTcDwBNSplit, 1, 2, 64, kDwAdam);
         AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwUpd);
         AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwBlock);
         AGN_DW_CASE(kTcDwBN, 1, 2, 64, kDwKeep);
