@@ -673,8 +673,9 @@ Status run_wave_steps(agn_handle* h, const Wave& wv, int64_t* launches) {
   const bool defer = h->hist > 1 && (int64_t)s * h->P * 4 > agn::kTcRedAccBytes;
   // Adam's step in the dW launch, when that covers every layer: the gradient
   // takes no trip through memory (8 of 44 bytes per parameter) and a launch
-  // goes.
-  const bool adam_fused = h->adam && h->fuse_out_dw;
+  // goes.  Not on large waves without accumulators where h->grad is kept for them.
+  const bool adam_fused =
+      h->adam && h->fuse_out_dw && !(h->grad && (int64_t)s * h->P * 4 > agn::kTcRedAccBytes);
   for (int i = 0; i < h->lam; ++i) {
     const int hi = defer ? i % h->hist : 0;   // this step's place in the history
     const int bi = defer ? hi % h->block : 0;   // and in its block
@@ -1515,8 +1516,17 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   h->fuse_out_dw = h->use_tc && h->use_head && (h->tc_mask & 4) && !(h->tc_mask & 8);
   if (h->adam) {   // the two moments of every worker, zero to start, and, for a step of
                    // its own after the dW kernels, the gradients
+    // Large waves without accumulators: with 26 bytes a parameter left to move in
+    // the dW launch, its two ring slots lose more against a streaming kernel than
+    // the gradient's 8 bytes cost, unless the fp32 products take longer.  ms a run of
+    // six steps, one launch and two: 16 slots of 784-4096-4096-10 bf16 m = 64 14.9 and
+    // 13.9, m = 256 15.6 and 15.0, fp32 m = 64 17.6 and 16.7, m = 256 22.3 and 23.6;
+    // 4 of them fp32 m = 65 4.68 and 4.58, m = 128 4.75 and 4.82
+    const bool own_step =
+        !h->fuse_out_dw || (h->elide && n * h->P * 4 > agn::kTcRedAccBytes &&
+                            (h->prec == AGN_PREC_BF16 || m <= 96));
     for (float** p : {&h->mom1, &h->mom2, &h->grad}) {
-      if (p == &h->grad && h->fuse_out_dw) continue;
+      if (p == &h->grad && !own_step) continue;
       AGN_TRY(dalloc_t(h, p, (size_t)(n * h->P_pad)));
       AGN_TRY_CUDA(cudaMemset(*p, 0, (size_t)(n * h->P_pad) * sizeof(float)));
     }
