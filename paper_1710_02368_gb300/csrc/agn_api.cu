@@ -275,8 +275,10 @@ struct agn_handle {
   // (every layer's dW in the persistent tensor-core launch, or Adam)
   bool acc_first = false;
   // bf16, lambda = 1: a worker that pulls anew after its one local step reads
-  // of its fp32 replica the biases and W_L only, so its pull writes no more (the
-  // commits of 784-4096-4096-10, 32 workers: 2.60 -> 2.34 ms a pass of 64)
+  // of its fp32 replica the biases and W_L only, so its pull writes no more.  Long
+  // vectors alone, us a run of two rounds with 32 workers, full pulls and these:
+  // 784-4096-4096-10 4313 and 3971, 784-4096-1024-10 (7.4 M) 1719 and 1576; 784-2048-
+  // 1024-10 (3.7 M) 951 and 996, 784-128-10 137 and 156.
   bool low_pulls = false;
   float* ce_partial = nullptr;    // [n][ceil(m / kHeadSamples)]
   int* head_counter = nullptr;    // [n]
@@ -1533,7 +1535,7 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
   }
   h->acc_first = h->fuse_out_dw || h->adam;
   h->low_pulls = h->prec == AGN_PREC_BF16 && h->lam == 1 && h->fuse_out_dw && !h->adam &&
-                 !h->elide && h->P_pad / 4 < INT32_MAX;
+                 !h->elide && agn::commit_low_pulls(h->P_pad);
   h->ldz_out = h->fuse_out_dw ? (int)round_up(dims[h->L], 8) : dims[h->L];
   h->fuse_head = h->use_tc && h->use_head && (h->tc_mask & 1) &&
                  !(h->tc_mask & 32) && dims[h->L] <= agn::kHeadMaxClasses;

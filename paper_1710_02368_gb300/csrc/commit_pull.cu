@@ -71,8 +71,8 @@ __device__ __forceinline__ void pack_pieces_x4(float4 v, uint2& p0, uint2& p1, u
 }
 
 // kCopy: 0 = fp32 replicas only, 1 = plus a bf16 copy, 2 = the same with kLowPull
-// pulls (a kernel of its own: their tests in every bf16 commit + pull cost the
-// short vectors 20 %: 64 workers of 784-128-10, 242 us a run against 192), 3 =
+// pulls (a kernel of its own, long vectors alone: their tests cost every bf16 commit +
+// pull of the short ones 20 %, 64 workers of 784-128-10, 242 us a run against 192), 3 =
 // plus the three exact bf16 pieces (planes `plane` elements apart) of the fp32
 // mode's tensor-core operands.
 // kElide: no accumulators.  `acc` then holds each worker's snapshot theta_pull
@@ -269,7 +269,12 @@ reduce_norms_kernel(const double* __restrict__ partials, int grid, const __grid_
 
 int g_num_sms = 0;
 
+// Short vectors: at most 8 float4 per thread over the grid.
+bool is_short(int64_t P, int grid) { return P / 4 <= (int64_t)grid * kThreads * 8; }
+
 }  // namespace
+
+bool commit_low_pulls(int64_t P) { return !is_short(P, commit_grid(P)) && P / 4 < INT32_MAX; }
 
 int commit_grid(int64_t P) {
   if (g_num_sms == 0) {
@@ -293,8 +298,7 @@ Status launch_commit_pull(const CommitPlan& plan, float* theta_c, float* acc, fl
     return launch_pdl(kern, grid, kThreads, 0, stream, plan, theta_c, acc, replicas, rb, P, ld,
                       scale, z, partials, plane);
   };
-  // short vectors: at most 8 float4 per thread over the grid
-  const bool shrt = P / 4 <= (int64_t)grid * kThreads * 8;
+  const bool shrt = is_short(P, grid);
   cudaError_t e;
 #define AGN_COMMIT_GO(C, E, RB, PL)                                                            \
   (shrt ? go(commit_pull_kernel<C, E, kShortUnroll, kShortGroup>, RB, PL)                       \
@@ -304,7 +308,8 @@ Status launch_commit_pull(const CommitPlan& plan, float* theta_c, float* acc, fl
               : AGN_COMMIT_GO(3, false, replicas_bf16, piece_plane);
   else if (replicas_bf16)
     e = elide             ? AGN_COMMIT_GO(1, true, replicas_bf16, 0)
-        : plan.n_skip > 0 ? AGN_COMMIT_GO(2, false, replicas_bf16, 0)
+        : plan.n_skip > 0   // (long vectors alone)
+            ? go(commit_pull_kernel<2, false, kLongUnroll, kLongGroup>, replicas_bf16, 0)
                           : AGN_COMMIT_GO(1, false, replicas_bf16, 0);
   else
     e = elide ? AGN_COMMIT_GO(0, true, nullptr, 0) : AGN_COMMIT_GO(0, false, nullptr, 0);

@@ -189,5 +189,7 @@ Status launch_commit_norms(const CommitPlan& plan, const double* partials, int g
 // Grid size used by the commit kernel for P parameters (a multiple of the SM
 // count, capped by the work).
 int commit_grid(int64_t P);
+// Whether commits of P parameters may have kLowPull pulls (long vectors).
+bool commit_low_pulls(int64_t P);
 
 }  // namespace agn

@@ -44,11 +44,14 @@ CASES = [((64, 48, 10), 33, 3, 1, (5, 3), True, 0),          # lambda 1: a_k onl
          ((784, 200, 136, 10), 100, 5, 3, (7, 4), True, 0),  # some pull within the run, some later
          ((256, 130, 26), 17, 4, 2, (8,), False, 3),         # no look-ahead: replicas keep theta_k
          ((1024, 2056, 10), 64, 8, 1, (8, 8), True, 7),      # accumulators over 64 MB
-         # lambda 1: bf16 pulls without the fp32 weights, then ones with them for
-         # the next call; several hidden layers, the output layer's own kernel
+         # lambda 1, several hidden layers, the output layer's own kernel
          ((136, 72, 264, 40, 10), 24, 6, 1, (13, 5, 9), True, 0),
          ((64, 4096, 5), 9, 9, 1, (20, 11), True, 8),
-         ((1024, 2056, 10), 40, 8, 3, (8, 9), True, 0)]
+         ((1024, 2056, 10), 40, 8, 3, (8, 9), True, 0),
+         # lambda 1, over 5 M parameters: bf16 pulls without the fp32 weights, then
+         # ones with them for the next call
+         ((1024, 5000, 10), 16, 4, 1, (9, 6), True, 0),
+         ((784, 2400, 1400, 10), 24, 3, 1, (7, 5, 6), True, 2)]
 
 
 @pytest.mark.parametrize("dims,m,n,lam,calls,look,tau_lo", CASES)
