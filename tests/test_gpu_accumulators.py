@@ -51,7 +51,7 @@ CASES = [((64, 48, 10), 33, 3, 1, (5, 3), True, 0),          # lambda 1: a_k onl
          # lambda 1, over 5 M parameters: bf16 pulls without the fp32 weights, then
          # ones with them for the next call
          ((1024, 5000, 10), 16, 4, 1, (9, 6), True, 0),
-         ((784, 2400, 1400, 10), 24, 3, 1, (7, 5, 6), True, 2)]
+         ((784, 2400, 1400, 10), 24, 3, 1, (3, 2, 3), True, 2)]
 
 
 @pytest.mark.parametrize("dims,m,n,lam,calls,look,tau_lo", CASES)
