@@ -1622,9 +1622,17 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     // for each row and feature of a chunk two buffers of pieces and one of fp32
     // values.  Fewer, larger chunks keep every SM busy: up to 48 Mi features,
     // 805 MB (256 rows at least).
+    // (Few rows of narrow inputs are faster on the CUDA cores, whose chain over k is
+    // short then.  us a call there and on the tensor cores: 48-8-8-8-10, 4 to 4096 rows,
+    // 47-50 and 62-72; 64-64-10, 512 rows 44 and 53, 4097 60 and 64, 10000 79 and 77;
+    // 128-128-10, 4096 rows 58 and 63; 136-136-136-10, 1024 rows 60 and 69, 2048 75 and 69;
+    // 256-256-256-10, 512 rows 58 and 67; 784-512-512-10, one row 84 and 68.)
+    int max_in = 1;
+    for (int l = 0; l + 1 < h->L; ++l) max_in = std::max(max_in, dims[l]);
+    const bool narrow = max_in <= 256 && E <= 8192 && E * max_in <= (max_in <= 128 ? 1 << 19 : 1 << 18);
     const int64_t up = std::min<int64_t>(E, 1 << 16);   // rows uploaded at a time
     const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(256, (48 << 20) / maxh / 256 * 256));
-    h->eval_tc = h->use_tc && (h->tc_mask & 1) && !h->lean &&
+    h->eval_tc = h->use_tc && (h->tc_mask & 1) && !h->lean && !narrow &&
                  (6 * E + 4 * up) * d0 + 16 * rows * maxh <= (int64_t)(dev_total / 4);
     h->eval_chunk = h->eval_tc ? rows : std::min<int64_t>(E, 4096);
     AGN_TRY(dalloc_t(h, &h->Xe, (size_t)((h->eval_tc ? up : E) * d0)));

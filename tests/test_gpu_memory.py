@@ -149,10 +149,10 @@ def test_wide_hidden_layers_take_short_chunks(env):
 
     def use(h):
         return h.evaluate(with_pred=True)
-    small, _ = _footprint(torch, lambda: make(agn.AGN_GEMM_AUTO, 1), use)
-    need, got = _footprint(torch, lambda: make(agn.AGN_GEMM_AUTO, 4096), use)
+    small, _ = _footprint(torch, lambda: make(agn.AGN_GEMM_SIMT, 1), use)
+    need, got = _footprint(torch, lambda: make(agn.AGN_GEMM_AUTO, 8193), use)
     assert need - small <= 900 * MB
-    _, ref = _footprint(torch, lambda: make(agn.AGN_GEMM_SIMT, 4096), use)
+    _, ref = _footprint(torch, lambda: make(agn.AGN_GEMM_SIMT, 8193), use)
     # two fp32 sums of eight products and of 40960 positive ones, in other orders
     assert got[0] == pytest.approx(ref[0], rel=1e-5)
     assert np.mean(got[2] != ref[2]) <= 1e-3
