@@ -1625,11 +1625,16 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     // (Few rows of narrow inputs are faster on the CUDA cores, whose chain over k is
     // short then.  us a call there and on the tensor cores: 48-8-8-8-10, 4 to 4096 rows,
     // 47-50 and 62-72; 64-64-10, 512 rows 44 and 53, 4097 60 and 64, 10000 79 and 77;
-    // 128-128-10, 4096 rows 58 and 63; 136-136-136-10, 1024 rows 60 and 69, 2048 75 and 69;
-    // 256-256-256-10, 512 rows 58 and 67; 784-512-512-10, one row 84 and 68.)
-    int max_in = 1;
-    for (int l = 0; l + 1 < h->L; ++l) max_in = std::max(max_in, dims[l]);
-    const bool narrow = max_in <= 256 && E <= 8192 && E * max_in <= (max_in <= 128 ? 1 << 19 : 1 << 18);
+    // 128-128-10, 4096 rows 58 and 63; 256-64-10, 2048 rows 47 and 64; 136-136-136-10, 1024
+    // rows 60 and 69, 2048 75 and 71; 256-256-256-10, 512 rows 58 and 67, 1024 71 and 67;
+    // 784-512-512-10, one row 84 and 68.)
+    bool narrow = E <= 8192;
+    int64_t row_macs = 0;   // the hidden layers' products of a row
+    for (int l = 0; l + 1 < h->L; ++l) {
+      narrow = narrow && dims[l] <= 256;
+      row_macs += (int64_t)dims[l] * dims[l + 1];
+    }
+    narrow = narrow && E * row_macs <= 1 << 26;
     const int64_t up = std::min<int64_t>(E, 1 << 16);   // rows uploaded at a time
     const int64_t rows = std::min<int64_t>(E, std::max<int64_t>(256, (48 << 20) / maxh / 256 * 256));
     h->eval_tc = h->use_tc && (h->tc_mask & 1) && !h->lean && !narrow &&

@@ -28,7 +28,7 @@ CASES = [((8, 8, 2), 1), ((64, 48, 10), 63), ((64, 136, 4), 129), ((72, 264, 40,
          ((8, 16, 3), 65536 + 5),        # 64 Ki rows uploaded at a time, then 5
          # (few rows of up to 256 inputs a layer: the CUDA cores, in any case above)
          ((264, 24, 2), 1), ((264, 136, 4), 129), ((8, 16, 3), 8192), ((8, 16, 3), 8193),
-         ((256, 24, 2), 1024), ((256, 24, 2), 1025)]
+         ((256, 256, 2), 1024), ((256, 256, 2), 1025)]
 
 
 @pytest.mark.parametrize("dims,rows", CASES)
