@@ -1627,11 +1627,11 @@ Status create(agn_handle* h, const int32_t* dims, int32_t n_dims, int32_t n_work
     // 47-50 and 62-72; 64-64-10, 512 rows 44 and 53, 4097 60 and 64, 10000 79 and 77;
     // 128-128-10, 4096 rows 58 and 63; 256-64-10, 2048 rows 47 and 64; 136-136-136-10, 1024
     // rows 60 and 69, 2048 75 and 71; 256-256-256-10, 512 rows 58 and 67, 1024 71 and 67;
-    // 784-512-512-10, one row 84 and 68.)
+    // 272-16-12, 324 rows 46 and 63; 384-384-384-10, 324 rows 71 and 68.)
     bool narrow = E <= 8192;
     int64_t row_macs = 0;   // the hidden layers' products of a row
     for (int l = 0; l + 1 < h->L; ++l) {
-      narrow = narrow && dims[l] <= 256;
+      narrow = narrow && dims[l] <= 320;
       row_macs += (int64_t)dims[l] * dims[l + 1];
     }
     narrow = narrow && E * row_macs <= 1 << 26;

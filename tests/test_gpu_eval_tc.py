@@ -26,8 +26,8 @@ CASES = [((8, 8, 2), 1), ((64, 48, 10), 63), ((64, 136, 4), 129), ((72, 264, 40,
          ((200, 1000, 1000, 10), 3001), ((64, 128, 128, 33), 700),
          ((16, 4096, 10), 12288 + 37),   # 48 Mi / 4096 rows a chunk, then 37
          ((8, 16, 3), 65536 + 5),        # 64 Ki rows uploaded at a time, then 5
-         # (few rows of up to 256 inputs a layer: the CUDA cores, in any case above)
-         ((264, 24, 2), 1), ((264, 136, 4), 129), ((8, 16, 3), 8192), ((8, 16, 3), 8193),
+         # (few rows of up to 320 inputs a layer: the CUDA cores, in any case above)
+         ((328, 24, 2), 1), ((320, 136, 4), 129), ((328, 136, 4), 129), ((8, 16, 3), 8192), ((8, 16, 3), 8193),
          ((256, 256, 2), 1024), ((256, 256, 2), 1025)]
 
 
