@@ -215,8 +215,8 @@ int agn_loss(agn_handle* h, float* out, int64_t cap);
  * Loss and accuracy of the current theta~ on the held-out set (the training-
  * accuracy curves of Section 4): softmax cross-entropy mean and the fraction
  * of samples whose argmax (lowest index on ties) is the label.  Forward pass in
- * fp32 on the device (the hidden layers on the tensor cores where training
- * uses them), fixed-order reductions; blocks until done.  loss, accuracy: host
+ * fp32 on the device (the hidden layers on the tensor cores where the training
+ * forward runs there, except few rows of narrow nets), fixed-order reductions; blocks until done.  loss, accuracy: host
  * floats (nullable); pred: host int32 [n_eval] predictions (nullable), cap its
  * length.  AGN_E_INVALID without an
  * evaluation set or with a short pred buffer; AGN_E_TIMEOUT when a
