@@ -1,9 +1,10 @@
 """The CUDA-core GEMMs at the edges of their tiles (32, 64 and 128 square, k
 slices of 64, 32 and 16, csrc/mlp_simt.cu): minibatches and widths one below, at and
-one above a tile and the k up to which 32-square tiles take short slices, with enough workers that each tile size is taken.  Against the
-float64 oracle at the fp32 tolerances of the other parity tests, and, since
-every output is one chain over k in order whatever the tile, the same worker's
-commit bit for bit whether it trains alone or in a wave of many."""
+one above a tile and the k up to which 32-square tiles take short slices, with
+enough workers that each tile size is taken.  Against the float64 oracle at the
+fp32 tolerances of the other parity tests, and, since every output is one chain
+over k in order whatever the tile, the same worker's commit bit for bit whether it
+trains alone or in a wave of many."""
 
 import numpy as np
 import pytest
